@@ -17,26 +17,29 @@
 
 namespace lbnci {
 
-__global__ void __launch_bounds__(256) reduce_partials_kernel(const double* __restrict__ partials,
-                                                              long long nblocks, double* __restrict__ out) {
-  // One block: thread t sums blocks t, t+256, ... in order, then a fixed tree.
-  __shared__ double s[256];
-  for (int q = 0; q < kRedSlots; ++q) {
-    double v = 0.0;
-    for (long long b = threadIdx.x; b < nblocks; b += blockDim.x) v += partials[b * kRedSlots + q];
-    s[threadIdx.x] = v;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-      if ((int)threadIdx.x < w) s[threadIdx.x] += s[threadIdx.x + w];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) out[q] = s[0];
-    __syncthreads();
+// One block over the flat array of block sums: thread t takes the elements t, t + 320, ...,
+// which all belong to slot t mod kRedSlots (320 is a multiple of it), so the loads are
+// coalesced and eight of them in flight; the 32 sums of a slot are then added in order.
+constexpr int kReduceThreads = 32 * kRedSlots;
+__global__ void __launch_bounds__(kReduceThreads) reduce_partials_kernel(const double* __restrict__ partials,
+                                                                         long long nblocks, double* __restrict__ out) {
+  __shared__ double s[kReduceThreads];
+  const long long n = nblocks * kRedSlots;
+  double v = 0.0;
+#pragma unroll 8
+  for (long long b = threadIdx.x; b < n; b += kReduceThreads) v += partials[b];
+  s[threadIdx.x] = v;
+  __syncthreads();
+  if (threadIdx.x < kRedSlots) {
+    double r = 0.0;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) r += s[threadIdx.x + k * kRedSlots];
+    out[threadIdx.x] = r;
   }
 }
 
 cudaError_t reduce_partials(const double* partials, long long nblocks, double* out, cudaStream_t s) {
-  reduce_partials_kernel<<<1, 256, 0, s>>>(partials, nblocks, out);
+  reduce_partials_kernel<<<1, kReduceThreads, 0, s>>>(partials, nblocks, out);
   return cudaGetLastError();
 }
 
@@ -133,7 +136,9 @@ size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 constexpr int kErrSlot = 12;
 
 struct Layout {
-  size_t fa, fb, psi, partials, result, carry, ring, ghost, ng, hit, rho1, total;
+  size_t fa, fb, psi, partials, result, carry, ring, ghost, ng, hit, rho1, sites;
+  size_t total;  // with the scratch of the step's per-site passes
+  size_t least;  // without it, where the step has kernels that need none
 };
 
 const Launchers* launchers_for(const lb_config* c) {
@@ -201,11 +206,19 @@ lb_status validate(const lb_config* c, HostParams* p, Layout* lay, long long* nb
   // D3Q27 FP32 / FP16-dev step on lattices of whole 32 x 8 columns: the streaming step
   // (moments, normals, collision with the ray), the fastest measured; LBNCI_D3_KERNEL=carry
   // selects the single-read step (density carry), march or tiled the two-pass step, which
-  // the other lattices and FP64 run
+  // the other lattices run
   const bool col_ok = c->lattice == LB_D3Q27 && (c->precision == LB_FP32 || c->precision == LB_FP16DEV) &&
                       c->nx % 32 == 0 && c->ny % 8 == 0 && (c->wall_z || c->nz >= 2);
   p->carry3d = 0;
   p->stream3d = col_ok ? 1 : 0;
+  // FP64 steps with Guo forcing run the per-site passes of lb_sites.cuh at every size: the
+  // FP64 pipe bounds both ways, and the passes recompute nothing over halos (128 x 128: 29 us
+  // per step against 117 us with the fused kernel, whose 32 tiles also leave most
+  // multiprocessors idle; 128 x 48 x 48 duct: 0.64 ms against 1.40 ms with the march).
+  // An environment variable that names another kernel selects that one.
+  bool sites = c->precision == LB_FP64 && c->forcing == 0;
+  if (c->lattice == LB_D3Q27) sites = sites && !std::getenv("LBNCI_D3_KERNEL");
+  else sites = sites && !std::getenv("LBNCI_FUSED_SPT") && !std::getenv("LBNCI_FUSED");
   if (const char* e = std::getenv("LBNCI_D3_KERNEL")) {
     if (std::strcmp(e, "march") == 0 || std::strcmp(e, "tiled") == 0) p->stream3d = 0;
     if (std::strcmp(e, "carry") == 0 && col_ok) { p->carry3d = 1; p->stream3d = 0; }
@@ -232,7 +245,7 @@ lb_status validate(const lb_config* c, HostParams* p, Layout* lay, long long* nb
   lay->psi = off; off = align256(off + (size_t)N * L->compute_elem);
   lay->partials = off; off = align256(off + (size_t)(*nblocks) * kRedSlots * sizeof(double));
   lay->result = off; off = align256(off + 16 * sizeof(double));
-  lay->carry = lay->ring = lay->ghost = lay->ng = lay->hit = lay->rho1 = off;
+  lay->carry = lay->ring = lay->ghost = lay->ng = lay->hit = lay->rho1 = lay->sites = off;
   if (p->carry3d) {
     lay->carry = off; off = align256(off + (size_t)N * 8);
     lay->ring = off; off = align256(off + carry3d_ring_bytes(*p));
@@ -243,6 +256,11 @@ lb_status validate(const lb_config* c, HostParams* p, Layout* lay, long long* nb
   if (p->stream3d) {
     lay->ng = off; off = align256(off + (size_t)N * 16);
     lay->rho1 = off; off = align256(off + (size_t)N * 2 * sizeof(float));
+  }
+  lay->least = off;
+  p->sites = nullptr;
+  if (sites) {
+    lay->sites = off; off = align256(off + L->step_scratch((size_t)N));
   }
   lay->total = off;
   return LB_OK;
@@ -258,17 +276,24 @@ long long staging_chunk(const lb_sim* s) {
   return fit >= s->p.N ? s->p.N : fit;
 }
 
-// Run the fields kernel on the current state with the given device outputs and
-// fill s->host_result with the reduced observables (synchronises the stream).
-lb_status run_fields(lb_sim* s, const FieldOut& outs) {
+// Run the fields kernels on the current state with the given device outputs and
+// fill s->host_result with the reduced observables (synchronises the stream). Their scratch
+// is the end of the back buffer, beyond the first `staged` bytes of it that the outputs use
+// (FP16-dev D2Q9 fields staged for the host leave too little: the kernels without scratch).
+lb_status run_fields(lb_sim* s, const FieldOut& outs, size_t staged = 0) {
   FieldOut fo = outs;
   fo.partials = s->partials;
   int nk = 0;
-  cudaError_t e = s->totals_state ? stream3d_form_fields(s->fa, s->psi, s->p, fo, s->stream, &nk)
-                                  : s->L->fields(s->fa, s->psi, s->p, fo, s->stream, &nk);
+  const size_t state = s->L->state_bytes((size_t)s->p.N) & ~(size_t)255;
+  const size_t need = s->L->fields_scratch((size_t)s->p.N);
+  void* scratch = need + staged <= state ? (void*)((unsigned char*)s->fb + (state - need)) : nullptr;
+  long long rows = s->nblocks;
+  cudaError_t e = s->totals_state
+                      ? stream3d_form_fields(s->fa, s->psi, s->p, fo, s->stream, &nk, scratch, s->nblocks, &rows)
+                      : s->L->fields(s->fa, s->psi, s->p, fo, s->stream, &nk, scratch, s->nblocks, &rows);
   s->launches += nk + 1;
   if (e != cudaSuccess) return cuda_fail(s, e, "fields launch");
-  e = reduce_partials(s->partials, s->nblocks, s->result, s->stream);
+  e = reduce_partials(s->partials, rows, s->result, s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e, "reduce launch");
   e = cudaMemcpyAsync(s->host_result, s->result, 16 * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e, "result copy");
@@ -354,19 +379,26 @@ lb_status lb_create(const lb_config* cfg, lb_sim** out) {
   s->stream = (cudaStream_t)cfg->stream;
   s->nblocks = nblocks;
   unsigned char* base = nullptr;
+  bool passes = true;  // room for the scratch of the step's per-site passes
   if (cfg->workspace) {
     if (((uintptr_t)cfg->workspace & 255u) != 0) {
       delete s;
       return fail(nullptr, LB_EINVAL, "workspace must be 256-byte aligned");
     }
-    if (cfg->workspace_bytes < lay.total) {
+    if (cfg->workspace_bytes < lay.least) {
       delete s;
-      return fail(nullptr, LB_ENOMEM, "workspace has %zu bytes, %zu needed", cfg->workspace_bytes, lay.total);
+      return fail(nullptr, LB_ENOMEM, "workspace has %zu bytes, %zu needed", cfg->workspace_bytes, lay.least);
     }
+    if (cfg->workspace_bytes < lay.total) passes = false;
     base = (unsigned char*)cfg->workspace;
     s->owns = false;
   } else {
     e = cudaMalloc((void**)&base, lay.total);
+    if (e == cudaErrorMemoryAllocation && lay.least < lay.total) {
+      cudaGetLastError();
+      passes = false;
+      e = cudaMalloc((void**)&base, lay.least);
+    }
     if (e != cudaSuccess) {
       delete s;
       cudaGetLastError();
@@ -406,9 +438,9 @@ lb_status lb_create(const lb_config* cfg, lb_sim** out) {
   if (s->p.stream3d) {
     s->ng = base + lay.ng;
     s->rho1 = base + lay.rho1;
-    if (!stream3d_supported(s->p)) s->p.stream3d = 0;
   }
   if (!s->p.stream3d) s->p.totals = 0;
+  if (passes && lay.total > lay.sites && lay.sites >= lay.least) s->p.sites = base + lay.sites;
   s->totals_state = false;
   s->carry_ok = false;
   e = cudaMallocHost((void**)&s->host_result, 16 * sizeof(double));
@@ -524,7 +556,7 @@ lb_status lb_fields(lb_sim* s, double* rho1, double* rho2, double* psi, double* 
       case 5: fo.hit = (int*)st; break;
       case 6: fo.u = st; break;
     }
-    lb_status stt = run_fields(s, fo);
+    lb_status stt = run_fields(s, fo, r.bytes);
     if (stt != LB_OK) return stt;
     cudaError_t e = cudaMemcpy(r.host, st, r.bytes, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(s, e, "field download");
@@ -725,7 +757,8 @@ extern "C" lb_status lb_observables_noalloc(const lb_config* cfg, const void* f,
   FieldOut fo{};
   fo.partials = (double*)(base + part_off);
   int nk = 0;
-  cudaError_t e = L->fields(f, base + psi_off, p, fo, stream, &nk);
+  long long rows = nblocks;
+  cudaError_t e = L->fields(f, base + psi_off, p, fo, stream, &nk, nullptr, nblocks, &rows);
   if (e != cudaSuccess) return fail(nullptr, LB_ECUDA, "fields launch: %s", cudaGetErrorString(e));
   double* result = (double*)(base + res_off);
   e = reduce_partials(fo.partials, nblocks, result, stream);
@@ -879,8 +912,12 @@ lb_status lb_ensemble_create(const lb_config* cfgs, int n, lb_ensemble** out) {
   for (int m = 0; m < n; ++m) {
     lb_config c = cfgs[m];
     c.workspace = nullptr;
-    lb_status st = lb_workspace_size(&c, &ws[m]);
+    HostParams p{};
+    Layout lay;
+    long long nb;
+    lb_status st = validate(&c, &p, &lay, &nb);
     if (st != LB_OK) return efail(nullptr, st, "member %d: %s", m, g_err);
+    ws[m] = lay.least;  // the batched kernels step the members: no scratch for passes of their own
     total += align256(ws[m]);
   }
   lb_ensemble* e = new (std::nothrow) lb_ensemble();

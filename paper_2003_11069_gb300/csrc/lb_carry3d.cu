@@ -224,15 +224,13 @@ cudaError_t launch_collide3d(const void* fa, void* fb, const float4* ng, const S
                              cudaStream_t s) {
   if (p.edm)
     collide3d_kernel<ST, true><<<grid, dim3(32, 8), 0, s>>>(ST::reader(fa, (unsigned)p.N),
-                                                            ST::writer(fb, (unsigned)p.N), ng, p);
+                                                                    ST::writer(fb, (unsigned)p.N), ng, p);
   else
     collide3d_kernel<ST, false><<<grid, dim3(32, 8), 0, s>>>(ST::reader(fa, (unsigned)p.N),
-                                                             ST::writer(fb, (unsigned)p.N), ng, p);
+                                                                     ST::writer(fb, (unsigned)p.N), ng, p);
   return cudaGetLastError();
 }
 }  // namespace
-
-bool stream3d_supported(const HostParams& h) { return h.nx % 32 == 0 && h.ny % 8 == 0; }
 
 bool stream3d_stores_totals(const HostParams& h) { return h.totals && h.forcing != 1; }
 
@@ -285,9 +283,7 @@ cudaError_t stream3d_step(const void* fa, void* fb, void* psi, void* ng, void* r
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   ++*nk;
-  const dim3 gridn((unsigned)(h.nx / 32), (unsigned)(h.ny / 8), (unsigned)((h.nz + kN3Z - 1) / kN3Z));
-  normals3d_kernel<<<gridn, dim3(32, 8), 0, s>>>((const float*)psi, (float4*)ng, p);
-  e = cudaGetLastError();
+  e = launch_normals3d<float>((const float*)psi, (Quad<float>*)ng, p, s);
   if (e != cudaSuccess) return e;
   ++*nk;
   if (totals_out && h.half) {
@@ -308,34 +304,18 @@ cudaError_t stream3d_step(const void* fa, void* fb, void* psi, void* ng, void* r
   return e;
 }
 
-namespace {
-// The fields kernel (and its moments pass) on a state in a total + recolouring form, read
-// through the form's two-population reader; the same grid as the other precisions' fields
-// launches (tiled_blocks), so the host reduces the same partials.
-template <typename FORM>
-cudaError_t form_fields(typename FORM::Reader rd, void* psi, const HostParams& h, const FieldOut& fo, cudaStream_t s,
-                        int* nk) {
-  const StepT<float> p = to_step3(h);
-  moments_kernel<1, FORM><<<(unsigned)((p.N + 255) / 256), 256, 0, s>>>(rd, (float*)psi, p);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  static SmemAllowance configured;
-  const size_t sm = tiled_smem_bytes<1, float>(p.smax);
-  e = allow_smem(tiled_kernel<1, FORM, true, false>, sm, configured);
-  if (e != cudaSuccess) return e;
-  const dim3 grid((unsigned)((h.nx + Tile<1>::X - 1) / Tile<1>::X), (unsigned)((h.ny + Tile<1>::Y - 1) / Tile<1>::Y),
-                  (unsigned)((h.nz + Tile<1>::Z - 1) / Tile<1>::Z));
-  tiled_kernel<1, FORM, true, false><<<grid, dim3(Tile<1>::X, Tile<1>::Y, Tile<1>::Z), sm, s>>>(
-      rd, typename FORM::Writer{}, (const float*)psi, p, fo);
-  *nk = 2;
-  return cudaGetLastError();
-}
-}  // namespace
-
+// The fields passes on a state in a total + recolouring form, read through the form's
+// two-population reader.
 cudaError_t stream3d_form_fields(const void* f, void* psi, const HostParams& h, const FieldOut& fo, cudaStream_t s,
-                                 int* nk) {
-  if (h.half) return form_fields<TotalRecolHalf>(TotalRecolHalf::reader(f, (unsigned)h.N, rho_unit(h)), psi, h, fo, s, nk);
-  return form_fields<TotalRecol>(TotalRecol::reader(f, (unsigned)h.N), psi, h, fo, s, nk);
+                                 int* nk, void* scratch, long long rows, long long* used) {
+  const StepT<float> p = to_step3(h);
+  auto normals = [&](const float* q, Quad<float>* ng) { return launch_normals3d<float, true>(q, ng, p, s); };
+  const unsigned N = (unsigned)h.N;
+  if (h.half)
+    return site_fields<1, TotalRecolHalf>(TotalRecolHalf::reader(f, N, rho_unit(h)), (float*)psi, scratch, h, p, fo,
+                                          rows, used, nk, s, normals);
+  return site_fields<1, TotalRecol>(TotalRecol::reader(f, N), (float*)psi, scratch, h, p, fo, rows, used, nk, s,
+                                    normals);
 }
 
 cudaError_t stream3d_form_decode(const void* f, double* out, int s0, int count, long long pitch, const HostParams& h,

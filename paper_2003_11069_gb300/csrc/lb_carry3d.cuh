@@ -48,6 +48,7 @@
 
 #include "lb_kernels.cuh"
 #include "lb_march3d.cuh"
+#include "lb_sites.cuh"
 #include "lb_tma.cuh"
 
 namespace lbnci {
@@ -750,81 +751,12 @@ carry3d_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 }
 
 // ---------------------------------------------------------------------------------
-// The streaming D3Q27 step (FP32 and FP16-dev storage; lattices of whole 32 x 8 columns):
-// a moments pass writes psi (and, for a step that stores the total + recolouring form,
-// (rho_1, rho_2)); normals3d_kernel the per-site (n, |grad psi|); the collision
+// The streaming D3Q27 step (FP32 and FP16-dev storage): a moments pass writes psi (and, for a step that stores the total + recolouring form,
+// (rho_1, rho_2)); normals3d_kernel (lb_sites.cuh) the per-site (n, |grad psi|); the collision
 // (collide3d_kernel for two populations per direction, collide3t_kernel for the total form,
 // at the end of the file) then runs the near-contact ray of its site over those normals
 // (probes through L2), pulls, collides and stores, with no shared memory and no barrier, its
 // block's neighbours reading the same planes at the same time from L2.
-
-// (n, |grad psi|) of a 32 x 8 column's sites on kN3Z consecutive planes from the psi
-// array: the block keeps psi of its 34 x 10 cells (beyond a wall the mirror cell, along
-// periodic axes the image) in a shared-memory ring of four planes; the loads of plane z + 2
-// are issued before plane z is computed and stored after it, into the slot plane z - 2
-// held, so their latency overlaps the arithmetic and one barrier per plane suffices (62 us
-// per duct step against 65 us with three slots and two barriers). Every site sums its 26
-// neighbours in direction order.
-constexpr int kN3Z = 16;
-__global__ void __launch_bounds__(256) normals3d_kernel(const float* __restrict__ psi, float4* __restrict__ ng,
-                                                        StepT<float> p) {
-  constexpr int RX = 34, RXY = RX * 10, PER = (RXY + 255) / 256;
-  __shared__ float s_psi[4 * RXY];
-  const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 8, z0 = blockIdx.z * kN3Z;
-  const int nx = p.nx, ny = p.ny, nz = p.nz;
-  const int tid = threadIdx.x + 32 * threadIdx.y;
-  const int z1 = min(nz, z0 + kN3Z);
-  auto load = [&](int q, float v[PER]) {  // plane q (wrapped or mirrored) into registers
-    const int gz = p.wall_z ? clampc(q, nz) : wrapn(q, nz);
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int c = tid + 256 * k;
-      if (c < RXY) {
-        const int ly = c / RX, lx = c - ly * RX;
-        const int gx = wrapn(x0 - 1 + lx, nx);
-        const int gy = p.wall_y ? clampc(y0 - 1 + ly, ny) : wrapn(y0 - 1 + ly, ny);
-        v[k] = psi[(unsigned)gx + (unsigned)nx * ((unsigned)gy + (unsigned)ny * (unsigned)gz)];
-      }
-    }
-  };
-  auto store = [&](int q, const float v[PER]) {  // into ring slot q mod 4
-    float* dst = s_psi + ((q + 4) & 3) * RXY;
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      const int c = tid + 256 * k;
-      if (c < RXY) dst[c] = v[k];
-    }
-  };
-  {
-    float v[PER];
-    load(z0 - 1, v);
-    store(z0 - 1, v);
-    load(z0, v);
-    store(z0, v);
-    load(z0 + 1, v);
-    store(z0 + 1, v);
-  }
-  __syncthreads();
-  const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
-  const int cxy = (threadIdx.x + 1) + RX * (threadIdx.y + 1);
-  for (int z = z0; z < z1; ++z) {
-    float vn[PER];
-    const bool more = z + 1 < z1;  // plane z + 2 is needed by the next iteration
-    if (more) load(z + 2, vn);
-    const float* pm = s_psi + ((z + 3) & 3) * RXY;
-    const float* p0 = s_psi + (z & 3) * RXY;
-    const float* pp = s_psi + ((z + 1) & 3) * RXY;
-    float g[3];
-    grad_ring<float>(pm, p0, pp, RX, cxy, g);
-    float n[3];
-    const float gn = M<float>::unit(g, n);
-    ng[(unsigned)x + (unsigned)nx * ((unsigned)y + (unsigned)ny * (unsigned)z)] = make_float4(n[0], n[1], n[2], gn);
-    // plane z + 2 goes to the fourth slot, the one plane z - 2 held: every thread finished
-    // reading it before the barrier that ended the previous plane
-    if (more) store(z + 2, vn);
-    __syncthreads();
-  }
-}
 
 // psi of every site, in 32 x 8 blocks of one plane (the streaming step's moments pass for
 // FP16-dev storage): a block's sources lie within 3 planes of 34 x 10 cells, so the

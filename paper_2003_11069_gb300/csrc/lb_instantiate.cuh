@@ -4,6 +4,7 @@
 
 #include "lb_fused2d.cuh"
 #include "lb_march3d.cuh"
+#include "lb_sites.cuh"
 #include "lb_kernels.cuh"
 #include "lb_launch.h"
 
@@ -153,6 +154,9 @@ template <int LAT, typename ST>
 cudaError_t l_step(const void* fa, void* fb, void* psi, const HostParams& h, cudaStream_t s, int* nk) {
   using T = typename ST::Compute;
   const StepT<T> p = convert<T>(h);
+  if constexpr (std::is_same<T, double>::value) {
+    if (h.sites && !p.edm) return site_step64<LAT>(fa, fb, (T*)psi, h.sites, h, p, nk, s);
+  }
   if constexpr (LAT == 0) {
     *nk = 1;
     return h.spt == 4 ? launch_fused2d<ST, 4>(fa, fb, p, s) : launch_fused2d<ST, 2>(fa, fb, p, s);
@@ -166,14 +170,26 @@ cudaError_t l_step(const void* fa, void* fb, void* psi, const HostParams& h, cud
   }
 }
 
+// Fields and observables: three per-site passes through the given scratch or, without any
+// (lb_observables_noalloc, whose fixed array has no room for it), a pass for psi and the
+// tiled kernel, which recomputes the gradients of its probes.
 template <int LAT, typename ST>
-cudaError_t l_fields(const void* f, void* psi, const HostParams& h, const FieldOut& fo, cudaStream_t s, int* nk) {
+cudaError_t l_fields(const void* f, void* psi, const HostParams& h, const FieldOut& fo, cudaStream_t s, int* nk,
+                     void* scratch, long long rows, long long* used) {
   using T = typename ST::Compute;
   const StepT<T> p = convert<T>(h);
+  if (scratch) {
+    auto normals = [&](const T* q, Quad<T>* ng) {
+      if constexpr (LAT == 1 && sizeof(T) == 4) return launch_normals3d<T, true>(q, ng, p, s);
+      else return launch_site_normals<LAT, T>(q, ng, h, p, s);
+    };
+    return site_fields<LAT, ST>(ST::reader(f, (unsigned)p.N), (T*)psi, scratch, h, p, fo, rows, used, nk, s, normals);
+  }
   moments_kernel<LAT, ST><<<blocks_for(p.N, 256), 256, 0, s>>>(ST::reader(f, (unsigned)p.N), (T*)psi, p);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   *nk = 2;
+  *used = rows;
   return launch_tiled<LAT, ST, true>(f, nullptr, psi, h, p, fo, s);
 }
 
@@ -241,7 +257,11 @@ cudaError_t l_batch_step(const void* members, const int* tile0, int n, int total
 
 template <int LAT, typename ST>
 const Launchers* table() {
-  static const Launchers L = {ST::bytes, sizeof(typename ST::Compute), l_init<LAT, ST>, l_step<LAT, ST>,
+  using T = typename ST::Compute;
+  static const Launchers L = {ST::bytes, sizeof(T),
+                              [](size_t N) { return site_scratch_bytes<LAT, T>(N, true); },
+                              [](size_t N) { return sizeof(T) == 8 ? site_scratch_bytes<LAT, T>(N, false) : 0; },
+                              l_init<LAT, ST>, l_step<LAT, ST>,
                               l_fields<LAT, ST>, l_decode<LAT, ST>, l_encode<LAT, ST>,
                               sizeof(BatchMember<typename ST::Compute>), l_batch_fill<ST>, l_batch_tiles,
                               l_batch_step<LAT, ST>};

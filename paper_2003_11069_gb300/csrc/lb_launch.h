@@ -52,6 +52,8 @@ struct HostParams {
   int c3_zseg;    // planes per z segment of their collision kernel
   int stream3d;   // 1: D3Q27 steps run moments, normals and a streaming collision
   int totals;     // 1: streaming steps with Guo forcing store the total + recolouring form
+  void* sites;    // device scratch of the FP64 step's per-site passes (null: the kernels that
+                  // recompute over halos, lb_fused2d.cuh and lb_march3d.cuh)
   float rho_ref;  // reference density rho_0 of the FP16 totals (f*_i = w_i rho_0 + d_i)
   unsigned* seedw;  // device: two dither-seed words of the FP16-deviation stores
   int parity;       // state buffer the next step reads (0: the one the sim was created with)
@@ -61,12 +63,16 @@ struct HostParams {
 struct Launchers {
   size_t (*state_bytes)(size_t N);  // bytes of one population state
   size_t compute_elem;              // bytes of the arithmetic type (psi scratch elements)
+  size_t (*fields_scratch)(size_t N);  // bytes of the fields passes' per-site scratch
+  size_t (*step_scratch)(size_t N);    // bytes of the step's (HostParams::sites), 0: it takes none
   cudaError_t (*init)(void* f, const double* rho1, const double* rho2, const double* u,
                       const HostParams& p, cudaStream_t s);
   // One full step fa -> fb (psi: scratch of N compute elements). Kernels launched -> *nk.
   cudaError_t (*step)(const void* fa, void* fb, void* psi, const HostParams& p, cudaStream_t s, int* nk);
+  // Fields of a state; scratch: fields_scratch bytes, or null (slower, no scratch but psi).
+  // The observables' block sums go to fo.partials, which has `rows` rows; *used are written.
   cudaError_t (*fields)(const void* f, void* psi, const HostParams& p, const FieldOut& fo,
-                        cudaStream_t s, int* nk);
+                        cudaStream_t s, int* nk, void* scratch, long long rows, long long* used);
   // FP64 [2][Q][pitch] copies of sites [s0, s0 + count) of a state, and back.
   cudaError_t (*decode)(const void* f, double* out, int s0, int count, long long pitch, int N, cudaStream_t s);
   cudaError_t (*encode)(const double* in, void* f, int s0, int count, long long pitch, int N, cudaStream_t s);
@@ -124,22 +130,20 @@ cudaError_t carry3d_prepare(TmaMaps* m, const void* fa, const void* fb, const vo
 // the carried densities of a state no step produced (pulled from it; rings zeroed)
 cudaError_t carry3d_init(const void* f, void* carry, void* ring, void* ghost, const HostParams& h, cudaStream_t s);
 // one step from state `from` (0: buffer A, 1: buffer B) into the other; *nk = launches
-// Streaming D3Q27 step (lb_carry3d.cu) for FP32 and FP16-dev storage on lattices of whole
-// 32 x 8 columns: moments (psi), normals3d ((n, |grad psi|) into ng, N float4), collide3d
+// Streaming D3Q27 step (lb_carry3d.cu) for FP32 and FP16-dev storage: moments (psi), normals3d ((n, |grad psi|) into ng, N float4), collide3d
 // (near-contact ray, pull, collision: fa -> fb). Kernels launched -> *nk.
 // With h.totals, steps under Guo forcing store the total + recolouring form of the
 // precision (TotalRecol / TotalRecolHalf in lb_carry3d.cuh: the total populations, the rest
 // population of each component and (rho_1/rho, beta rho_1 rho_2/rho m) per site; FP16 totals
 // as deviations from w_i h.rho_ref); totals_in says that fa holds that form; rho12 (N float2)
 // carries (rho_1, rho_2) from the moments pass to the collision.
-bool stream3d_supported(const HostParams& h);
 bool stream3d_stores_totals(const HostParams& h);
 cudaError_t stream3d_step(const void* fa, void* fb, void* psi, void* ng, void* rho12, int totals_in,
                           const HostParams& h, cudaStream_t s, int* nk);
 // fields and population copies of a state in the total + recolouring form (the
 // Launchers::fields / decode of the other states)
 cudaError_t stream3d_form_fields(const void* f, void* psi, const HostParams& h, const FieldOut& fo, cudaStream_t s,
-                                 int* nk);
+                                 int* nk, void* scratch, long long rows, long long* used);
 cudaError_t stream3d_form_decode(const void* f, double* out, int s0, int count, long long pitch, const HostParams& h,
                                  cudaStream_t s);
 size_t stream3d_totals_bytes(size_t N, int half);
