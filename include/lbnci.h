@@ -115,7 +115,9 @@ typedef struct {
 } lb_obs;
 
 /* Device bytes lb_create needs when it is given a workspace (cfg->workspace): two
- * population states of the two sets f^k_i of Eq. (CGLBE) plus scratch. */
+ * population states of the two sets f^k_i of Eq. (CGLBE) plus scratch. Where a step can
+ * run without part of the scratch (lb_step_path), a workspace smaller by that part is
+ * accepted and the step takes its slower kernels; the populations are the same bits. */
 lb_status lb_workspace_size(const lb_config* cfg, size_t* bytes);
 
 /* Validate cfg, take the current CUDA device, allocate (or carve from the
@@ -185,12 +187,17 @@ const char* lb_last_error(const lb_sim* sim);
 long long lb_kernel_launches(const lb_sim* sim);
 
 /* Which kernel lb_step runs for this sim (no paper counterpart; reporting only):
- *   LB_PATH_FUSED2D  one-pass fused D2Q9 kernel (FP64; FP32 and FP16-dev when nx % 4 != 0
- *                    or LBNCI_FUSED=classic is set in the environment),
+ *   LB_PATH_FUSED2D  one-pass fused D2Q9 kernel (FP32 and FP16-dev when nx % 4 != 0 or
+ *                    LBNCI_FUSED=classic is set in the environment; FP64 with the
+ *                    exact-difference forcing) or, for FP64 with Guo forcing, moments,
+ *                    normals and collision as passes over the sites,
  *   LB_PATH_TMA2D    persistent TMA-fed D2Q9 kernel (FP32 and FP16-dev storage),
- *   LB_PATH_D3Q27    D3Q27 two-pass step: moments, then the collision kernel marching along
- *                    z (FP64; FP32 and FP16-dev when nx % 32 != 0 or ny % 8 != 0, or when
- *                    LBNCI_D3_KERNEL=march or tiled is set in the environment),
+ *   LB_PATH_D3Q27    D3Q27 step on the two-population state: for FP64, and for FP32 and
+ *                    FP16-dev when nx % 32 != 0 or ny % 8 != 0, moments, normals and
+ *                    collision as passes over the sites; where a workspace has no room for
+ *                    their scratch, for FP64 with the exact-difference forcing, or when
+ *                    LBNCI_D3_KERNEL=march or tiled is set in the environment, moments, then
+ *                    a collision kernel that keeps gradients in shared memory,
  *   LB_PATH_D3Q27_CARRY  D3Q27 single-read step (FP32 and FP16-dev, LBNCI_D3_KERNEL=carry): an
  *                    interface pass over densities the previous collision carried forward,
  *                    a ray pass, then a TMA-fed collision that reads each population once,

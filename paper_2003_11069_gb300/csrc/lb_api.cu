@@ -203,14 +203,16 @@ lb_status validate(const lb_config* c, HostParams* p, Layout* lay, long long* nb
   // LBNCI_TMA_STALL_TEST=1 makes every CTA's first wait run out after about a second.
   p->tma_stall_test = 0;
   if (const char* e = std::getenv("LBNCI_TMA_STALL_TEST")) p->tma_stall_test = std::atoi(e) == 1 ? 1 : 0;
-  // D3Q27 FP32 / FP16-dev step on lattices of whole 32 x 8 columns: the streaming step
-  // (moments, normals, collision with the ray), the fastest measured; LBNCI_D3_KERNEL=carry
-  // selects the single-read step (density carry), march or tiled the two-pass step, which
-  // the other lattices run
+  // D3Q27 FP32 / FP16-dev step: the streaming step (moments, normals, collision with the
+  // ray), the fastest measured; LBNCI_D3_KERNEL=carry selects the single-read step (density
+  // carry; lattices of whole 32 x 8 columns), march or tiled the two-pass step. Lattices of
+  // no whole columns keep the two-population state (a 150 x 66 x 66 FP32 duct: 0.106 ms per
+  // step against 0.175 ms with the marching collision, whose few columns leave CTAs short of
+  // planes and whose barriers expose every pull's latency; the states are the same bits)
   const bool col_ok = c->lattice == LB_D3Q27 && (c->precision == LB_FP32 || c->precision == LB_FP16DEV) &&
                       c->nx % 32 == 0 && c->ny % 8 == 0 && (c->wall_z || c->nz >= 2);
   p->carry3d = 0;
-  p->stream3d = col_ok ? 1 : 0;
+  p->stream3d = c->lattice == LB_D3Q27 && c->precision != LB_FP64 && (c->wall_z || c->nz >= 2) ? 1 : 0;
   // FP64 steps with Guo forcing run the per-site passes of lb_sites.cuh at every size: the
   // FP64 pipe bounds both ways, and the passes recompute nothing over halos (128 x 128: 29 us
   // per step against 117 us with the fused kernel, whose 32 tiles also leave most
@@ -226,7 +228,7 @@ lb_status validate(const lb_config* c, HostParams* p, Layout* lay, long long* nb
   // streaming steps with Guo forcing store the total + recolouring form (FP32: 128 instead
   // of 216 bytes per site; FP16-dev: 76 instead of 116), unless LBNCI_D3_STATE=pairs keeps
   // the two-population layout
-  p->totals = p->stream3d && c->forcing == 0 ? 1 : 0;
+  p->totals = p->stream3d && col_ok && c->forcing == 0 ? 1 : 0;
   if (const char* e = std::getenv("LBNCI_D3_STATE"))
     if (std::strcmp(e, "pairs") == 0) p->totals = 0;
   p->rho_ref = 1.0f;
@@ -253,11 +255,14 @@ lb_status validate(const lb_config* c, HostParams* p, Layout* lay, long long* nb
     lay->ng = off; off = align256(off + (size_t)N * 16);
     lay->hit = off; off = align256(off + (size_t)N);
   }
-  if (p->stream3d) {
+  if (p->stream3d && col_ok) {
     lay->ng = off; off = align256(off + (size_t)N * 16);
     lay->rho1 = off; off = align256(off + (size_t)N * 2 * sizeof(float));
   }
   lay->least = off;
+  if (p->stream3d && !col_ok) {
+    lay->ng = off; off = align256(off + (size_t)N * 16);
+  }
   p->sites = nullptr;
   if (sites) {
     lay->sites = off; off = align256(off + L->step_scratch((size_t)N));
@@ -435,6 +440,7 @@ lb_status lb_create(const lb_config* cfg, lb_sim** out) {
       s->p.carry3d = 0;
     cudaGetLastError();
   }
+  if (!passes && lay.ng >= lay.least) s->p.stream3d = 0;
   if (s->p.stream3d) {
     s->ng = base + lay.ng;
     s->rho1 = base + lay.rho1;
@@ -673,7 +679,8 @@ long long lb_kernel_launches(const lb_sim* s) { return s ? s->launches : 0; }
 int lb_step_path(const lb_sim* s) {
   if (!s) return -1;
   if (s->cfg.lattice == LB_D3Q27)
-    return s->p.carry3d ? LB_PATH_D3Q27_CARRY : (s->p.stream3d ? LB_PATH_D3Q27_STREAM : LB_PATH_D3Q27);
+    return s->p.carry3d ? LB_PATH_D3Q27_CARRY
+                        : (s->p.stream3d && s->p.nx % 32 == 0 && s->p.ny % 8 == 0 ? LB_PATH_D3Q27_STREAM : LB_PATH_D3Q27);
   return s->p.tma ? LB_PATH_TMA2D : LB_PATH_FUSED2D;
 }
 

@@ -219,14 +219,14 @@ cudaError_t carry3d_step(const TmaMaps& m, int from, const void* fa, void* fb, v
 }
 
 namespace {
-template <typename ST>
+template <typename ST, bool RAGGED>
 cudaError_t launch_collide3d(const void* fa, void* fb, const float4* ng, const StepT<float>& p, dim3 grid,
                              cudaStream_t s) {
   if (p.edm)
-    collide3d_kernel<ST, true><<<grid, dim3(32, 8), 0, s>>>(ST::reader(fa, (unsigned)p.N),
+    collide3d_kernel<ST, true, RAGGED><<<grid, dim3(32, 8), 0, s>>>(ST::reader(fa, (unsigned)p.N),
                                                                     ST::writer(fb, (unsigned)p.N), ng, p);
   else
-    collide3d_kernel<ST, false><<<grid, dim3(32, 8), 0, s>>>(ST::reader(fa, (unsigned)p.N),
+    collide3d_kernel<ST, false, RAGGED><<<grid, dim3(32, 8), 0, s>>>(ST::reader(fa, (unsigned)p.N),
                                                                      ST::writer(fb, (unsigned)p.N), ng, p);
   return cudaGetLastError();
 }
@@ -257,7 +257,7 @@ cudaError_t stream3d_step(const void* fa, void* fb, void* psi, void* ng, void* r
   *nk = 0;
   const bool totals_out = stream3d_stores_totals(h);
   if (totals_in && !totals_out) return cudaErrorInvalidValue;  // no step reads that form into pairs
-  const dim3 grid((unsigned)(h.nx / 32), (unsigned)(h.ny / 8), (unsigned)h.nz);
+  const dim3 grid((unsigned)((h.nx + 31) / 32), (unsigned)((h.ny + 7) / 8), (unsigned)h.nz);
   const unsigned N = (unsigned)p.N;
   const float r0 = rho_unit(h);
   float2* r12 = totals_out ? (float2*)rho12 : nullptr;
@@ -297,8 +297,13 @@ cudaError_t stream3d_step(const void* fa, void* fb, void* psi, void* ng, void* r
                   : launch_collide3t<Plain<1, float>::Reader, false>(Plain<1, float>::reader(fa, N), wr, rho12, ng, p,
                                                                       grid, s);
   } else {
-    e = h.half ? launch_collide3d<HalfDev<1>>(fa, fb, (const float4*)ng, p, grid, s)
-               : launch_collide3d<Plain<1, float>>(fa, fb, (const float4*)ng, p, grid, s);
+    const bool ragged = h.nx % 32 != 0 || h.ny % 8 != 0;
+    if (ragged)
+      e = h.half ? launch_collide3d<HalfDev<1>, true>(fa, fb, (const float4*)ng, p, grid, s)
+                 : launch_collide3d<Plain<1, float>, true>(fa, fb, (const float4*)ng, p, grid, s);
+    else
+      e = h.half ? launch_collide3d<HalfDev<1>, false>(fa, fb, (const float4*)ng, p, grid, s)
+                 : launch_collide3d<Plain<1, float>, false>(fa, fb, (const float4*)ng, p, grid, s);
   }
   if (e == cudaSuccess) ++*nk;
   return e;

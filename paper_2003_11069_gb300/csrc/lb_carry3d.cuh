@@ -205,6 +205,7 @@ __device__ __forceinline__ int nci_ray(const float4* __restrict__ ng, const floa
         return;
       }
       px = px < 0 ? px + nx : (px >= nx ? px - nx : px);
+      if (nx <= kMaxProbe) px = wrapn(px, nx);  // a probe may pass several periods
       if (!p.wall_y) py = wrapn(py, ny);
       if (!p.wall_z) pz = wrapn(pz, nz);
       q[s - 1] = ng[(unsigned)px + (unsigned)nx * ((unsigned)py + (unsigned)ny * (unsigned)pz)];
@@ -766,6 +767,7 @@ template <typename ST>
 __global__ void __launch_bounds__(256) moments3_kernel(typename ST::Reader f, float* __restrict__ psi,
                                                        float2* __restrict__ rho12, StepT<float> p) {
   const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y, z = blockIdx.z;
+  if (x >= p.nx || y >= p.ny) return;
   const int site = x + p.nx * (y + p.ny * z);
   float fin[2][27];
   pull_any<1, float>(f, x, y, z, p, fin);
@@ -776,13 +778,16 @@ __global__ void __launch_bounds__(256) moments3_kernel(typename ST::Reader f, fl
   if (rho12) rho12[site] = make_float2(r1, r2);
 }
 
-template <typename ST, bool EDM>
+// RAGGED: lattices of no whole 32 x 8 columns, whose states stay those of march3d_kernel bit
+// for bit.
+template <typename ST, bool EDM, bool RAGGED>
 __global__ void __launch_bounds__(256) collide3d_kernel(typename ST::Reader f, typename ST::Writer fout,
                                                         const float4* __restrict__ ng, StepT<float> p) {
   const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y, z = blockIdx.z;
   if constexpr (ST::kHalf)
     fout.seed = step_seed(p, p.parity, blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0 &&
                                            threadIdx.y == 0);
+  if (x >= p.nx || y >= p.ny) return;
   const int site = x + p.nx * (y + p.ny * z);
   // FP32: the pulls first, so that their loads are in flight while the ray's dependent
   // probes resolve (2.5% faster); FP16-dev: the ray first (pulls first raised its
@@ -810,7 +815,16 @@ __global__ void __launch_bounds__(256) collide3d_kernel(typename ST::Reader f, t
     if (h == s) A = p.Ah[s];
   });
   const float deltaI = 0.5f * v.w;
-  const float F[3] = {p.G[0] - A * v.x * deltaI, p.G[1] - A * v.y * deltaI, p.G[2] - A * v.z * deltaI};
+  float F[3];
+  if constexpr (RAGGED) {  // the marching kernel's roundings: F_rep, then the sum
+    F[0] = __fsub_rn(p.G[0], A * v.x * deltaI);
+    F[1] = __fsub_rn(p.G[1], A * v.y * deltaI);
+    F[2] = __fsub_rn(p.G[2], A * v.z * deltaI);
+  } else {
+    F[0] = p.G[0] - A * v.x * deltaI;
+    F[1] = p.G[1] - A * v.y * deltaI;
+    F[2] = p.G[2] - A * v.z * deltaI;
+  }
   float u[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) u[a] = M<float>::div(j[a] + 0.5f * F[a], rho);

@@ -118,6 +118,28 @@ def test_fields_and_observables(lat, nx, ny, nz, walls, precision):
             sim.step(1)
 
 
+@pytest.mark.parametrize("precision", [lbnci.LB_FP32, lbnci.LB_FP16DEV])
+@pytest.mark.parametrize("forcing", [lbnci.LB_FORCE_GUO, lbnci.LB_FORCE_EDM_DISPERSED])
+@pytest.mark.parametrize("nx,ny,nz,walls", [(33, 9, 5, (1, 1)), (31, 7, 17, (0, 1)), (70, 20, 18, (1, 0)), (5, 3, 2, (0, 0))])
+def test_ragged_ducts_equal_the_marching_step(nx, ny, nz, walls, forcing, precision, monkeypatch):
+    """Lattices of no whole 32 x 8 columns: the streaming kernels on the two-population state give
+    the marching kernel's populations (the same expressions on the same state)."""
+    f = _state(lbnci.LB_D3Q27, nx, ny, nz, 6)
+    cfg = _cfg(lbnci.LB_D3Q27, nx, ny, nz, walls, precision)
+    cfg.forcing = forcing
+    got = []
+    for mode in ("", "march"):
+        if mode:
+            monkeypatch.setenv("LBNCI_D3_KERNEL", mode)
+        else:
+            monkeypatch.delenv("LBNCI_D3_KERNEL", raising=False)
+        with lbnci.Sim(cfg) as sim:
+            sim.set_populations(f)
+            sim.step(3)
+            got.append(sim.get_populations())
+    assert np.array_equal(*got)
+
+
 def test_fields_report_bad_sites_as_before():
     """NaN, infinite and negative densities are counted, whatever path the fields take."""
     for lat, dims in ((lbnci.LB_D2Q9, (40, 24, 1)), (lbnci.LB_D3Q27, (32, 8, 4))):
