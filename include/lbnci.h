@@ -115,9 +115,11 @@ typedef struct {
 } lb_obs;
 
 /* Device bytes lb_create needs when it is given a workspace (cfg->workspace): two
- * population states of the two sets f^k_i of Eq. (CGLBE) plus scratch. Where a step can
- * run without part of the scratch (lb_step_path), a workspace smaller by that part is
- * accepted and the step takes its slower kernels; the populations are the same bits. */
+ * population states of the two sets f^k_i of Eq. (CGLBE) plus scratch. A workspace larger
+ * by 48 N + 1024 bytes (FP64 with Guo forcing) or 16 N + 1024 bytes (FP32 and FP16-dev D3Q27
+ * lattices with nx % 32 != 0 or ny % 8 != 0) also holds the per-site arrays of those steps'
+ * faster kernels, which a sim that allocates its own memory takes when it can; without
+ * them the step runs kernels that recompute over halos, to the same bits. */
 lb_status lb_workspace_size(const lb_config* cfg, size_t* bytes);
 
 /* Validate cfg, take the current CUDA device, allocate (or carve from the

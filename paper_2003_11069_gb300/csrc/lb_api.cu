@@ -355,7 +355,7 @@ lb_status lb_workspace_size(const lb_config* cfg, size_t* bytes) {
   long long nb;
   lb_status st = validate(cfg, &p, &lay, &nb);
   if (st != LB_OK) return st;
-  *bytes = lay.total;
+  *bytes = lay.least;
   return LB_OK;
 }
 

@@ -53,25 +53,23 @@ def test_fp64_passes_equal_the_one_pass_kernels(lat, nx, ny, nz, walls, monkeypa
         assert np.array_equal(out[("passes",) + k], out[("halo",) + k])
 
 
-def test_fp64_passes_need_no_larger_workspace(monkeypatch):
-    """A workspace without room for the passes' scratch still steps, to the same state."""
+@pytest.mark.parametrize("precision", [lbnci.LB_FP64, lbnci.LB_FP32])
+def test_passes_need_no_larger_workspace(precision, monkeypatch):
+    """A workspace without room for the passes' scratch still steps, to the state of one that has it
+    and of a sim that allocates its own memory."""
     monkeypatch.delenv("LBNCI_D3_KERNEL", raising=False)
     f = _state(lbnci.LB_D3Q27, 33, 9, 5, 4)
-    cfg = _cfg(lbnci.LB_D3Q27, 33, 9, 5, (1, 1), lbnci.LB_FP64)
-    full = lbnci.lb_workspace_size(cfg)
-    monkeypatch.setenv("LBNCI_D3_KERNEL", "march")
+    cfg = _cfg(lbnci.LB_D3Q27, 33, 9, 5, (1, 1), precision)
     least = lbnci.lb_workspace_size(cfg)
-    monkeypatch.delenv("LBNCI_D3_KERNEL")
-    assert least < full
     got = []
-    for n in (least, full):
+    for n in (least, least + 48 * 33 * 9 * 5 + 1024, 0):
         ws = torch.empty(n + 256, dtype=torch.uint8, device="cuda")
-        cfg.workspace, cfg.workspace_bytes = (ws.data_ptr() + 255) & ~255, n
+        cfg.workspace, cfg.workspace_bytes = ((ws.data_ptr() + 255) & ~255, n) if n else (None, 0)
         with lbnci.Sim(cfg) as sim:
             sim.set_populations(f)
             sim.step(2)
             got.append(sim.get_populations())
-    assert np.array_equal(*got)
+    assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])
 
 
 @pytest.mark.parametrize("precision", [lbnci.LB_FP64, lbnci.LB_FP32, lbnci.LB_FP16DEV])
