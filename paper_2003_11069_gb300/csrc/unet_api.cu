@@ -13,7 +13,8 @@
 
 #include "lbnci_unet.h"
 #include "unet_kernels.cuh"
-#include "unet_tc.cuh"
+#include "unet_conv.cuh"
+#include "lb_launch.h"
 
 // Error word of the tensor-core convolutions: bit 0 set when a bounded mbarrier wait
 // expired (the launch then wrote no output). Read and cleared by the calls that
@@ -115,7 +116,88 @@ size_t wgrad_bytes(const WgradPlan& w, int cin, int cout) {
   return ((size_t)w.nsplit * cout * 9 * cin + (size_t)w.nsplit * cout) * sizeof(float);
 }
 
+constexpr int kSmemMax = 227 * 1024, kSmemSm = 228 * 1024;
+
+// Partition of the tensor-memory weight gradient (conv3x3_wgrad_tma_kernel) over B images of
+// H x W positions (the low-resolution input's when up): tiles of eight rows x 32 columns
+// (four rows when up, whose stage holds four tiles of dy), as many stages as the shared
+// memory of one or two CTAs holds, and as many splits as fill the 152 multiprocessors once.
+struct WgradTmaPlan {
+  bool ok = false;
+  int BN, rowb, smem;
+  lbu::WgradTma a;
+};
+WgradTmaPlan wgrad_tma_plan(int B, int H, int W, int cin, int cout, int up) {
+  WgradTmaPlan p;
+  if (cin % 32 || cout % 32) return p;
+  p.rowb = cin % 64 == 0 ? 128 : 64;
+  p.BN = cout % 64 == 0 ? 64 : 32;
+  if (up && p.rowb != 128) return p;
+  lbu::WgradTma& a = p.a;
+  a = lbu::WgradTma{};
+  a.H = H;
+  a.W = W;
+  a.up = up;
+  a.TW = W >= 32 ? 32 : 16;
+  a.TH = std::min(H, up ? 4 : 8);
+  a.pitch = a.TW + 2;
+  a.tiles_x = (W + a.TW - 1) / a.TW;
+  a.tiles_y = (H + a.TH - 1) / a.TH;
+  a.ntile = B * a.tiles_x * a.tiles_y;
+  a.Cin = cin;
+  a.Cout = cout;
+  const int npar = up ? 4 : 1, nacc = up ? 8 : (p.rowb == 64 ? 3 : 5);
+  a.x_bytes = (((a.TH + 2) * a.pitch + 1) * p.rowb + 1023) / 1024 * 1024;
+  a.d_bytes = (a.TH * a.TW * p.BN * 2 + 1023) / 1024 * 1024;
+  const int stage = a.x_bytes + npar * a.d_bytes;
+  a.cols = 32;
+  while (a.cols < nacc * p.BN) a.cols *= 2;
+  const int occ = a.cols <= 256 && 2 * (2 * stage + 2048) <= kSmemSm ? 2 : 1;
+  a.nstage = std::min(lbu::kWgradMaxStage, (kSmemSm / occ - 3072) / stage);
+  if (a.nstage < 2) return p;
+  a.tail = std::max(a.nstage * stage, 8192);
+  // no more CTAs on a multiprocessor than its tensor memory serves
+  p.smem = std::max(a.tail + (int)sizeof(lbu::WgradTail), kSmemSm / (512 / a.cols + 1) - 1024 + 16);
+  if (p.smem > kSmemMax) return p;
+  const int blocks = (cin / (p.rowb / 2)) * (cout / p.BN);
+  a.nsplit = std::max(1, std::min(a.ntile, 152 * occ / blocks));
+  p.ok = true;
+  return p;
+}
+size_t wgrad_tma_bytes(const WgradTmaPlan& p) {
+  const lbu::WgradTma& a = p.a;
+  return p.ok ? ((size_t)a.nsplit * a.Cout * (a.up ? 16 : 9) * a.Cin + (size_t)a.nsplit * a.Cout) * sizeof(float) : 0;
+}
+// Scratch of a weight gradient by either kernel, with or without upsampled input.
+size_t wgrad_work(int B, int H, int W, int cin, int cout) {
+  size_t n = wgrad_bytes(wgrad_plan(B * H * W, cin, cout), cin, cout);
+  n = std::max(n, wgrad_tma_bytes(wgrad_tma_plan(B, H, W, cin, cout, 0)));
+  if (H % 2 == 0 && W % 2 == 0) n = std::max(n, wgrad_tma_bytes(wgrad_tma_plan(B, H / 2, W / 2, cin, cout, 1)));
+  return n;
+}
+
 thread_local std::string g_err;
+
+// One launch of conv3x3_tma_kernel: tensor maps, tile and grid of a convolution's operands.
+struct ConvPlan {
+  bool ok = false;
+  CUtensorMap mx, mw;
+  lbu::ConvTma a;
+  dim3 grid;
+  int smem = 0, BN = 0, rowb = 0;
+};
+
+// The plans of a network's launches, one per layer and direction, kept for the batch they
+// were made for: a layer's operands are the network's own buffers.
+struct ConvCache {
+  int B = -1;
+  ConvPlan p;
+};
+struct WgradCache {
+  int B = -1;
+  WgradTmaPlan p;
+  lbu::WgradMaps maps;
+};
 
 }  // namespace
 
@@ -139,6 +221,8 @@ struct lbu_net {
   float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   long long t = 0;
   long long launches = 0;
+  std::vector<ConvCache> conv_cache;    // forward of layer i: i, data gradient: layers + i
+  std::vector<WgradCache> wgrad_cache;  // layer i
   std::vector<void*> allocs;
   std::string err;
 };
@@ -178,31 +262,174 @@ int grid_for(long long work, int threads) {
   return (int)std::max<long long>(1, std::min<long long>(b, 152LL * 16));
 }
 
-template <int BN, int BK>
-cudaError_t launch_conv_tc_k(const lbu::ConvFwd& a, dim3 grid, cudaStream_t s) {
+// ------------------------------------------------------------------ tensor-core convolution
+bool encode_tiled(CUtensorMap* m, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
+                  const cuuint32_t* box, int rowb) {
+  auto fn = lbnci::encode_fn();
+  if (!fn) return false;
+  const cuuint32_t es[4] = {1, 1, 1, 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, es,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, rowb == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The tile of a convolution over B images of H x W positions (the low-resolution input's
+// when up): among tiles of 16 rows x 8 k columns (every operand row a pixel) and tiles of
+// TH rows x min(W, 126) columns (rows of the operand run through the pitched tile), those
+// whose operands fit, the one with the smallest estimated time. The estimate counts, per
+// multiprocessor, waves of resident CTAs, each wave a fixed latency (copy, first MMA,
+// drain: about 4,000 cycles) plus the CTAs' MMAs (M = 128: 32 cycles whatever N up to 128,
+// reading A from shared memory sets the rate) or their copies (about 50 bytes a cycle),
+// whichever is longer.
+bool plan_tile(int B, int H, int W, int cin, int cout, int up, ConvPlan* p) {
+  p->rowb = cin % 64 == 0 ? 128 : 64;
+  const int nchunk = cin / (p->rowb / 2), npar = up ? 4 : 1, ni = 9 * nchunk;
+  double best = 1e30;
+  auto consider = [&](int BN, int TH, int TW, bool linear) {
+    const int bstage = BN * p->rowb;
+    const int stages = std::min(std::min(ni, lbu::kConvMaxStage), std::max(3, 36864 / bstage));
+    const int pitch = TW + 2, sbo = linear ? 8 : pitch, mstart = linear ? 128 : 8;
+    const int nm = linear ? (TH * pitch - 2 + 127) / 128 : TW / 8;
+    const int ncols = nm * npar * BN;
+    if (ncols > 512 || TW + 2 > 256 || TH + 2 > 256) return;
+    int cols = 32;
+    while (cols < ncols) cols *= 2;
+    // rows of the tile in shared memory: the copy's, and what the last M tile reads beyond it
+    const int reach = (nm - 1) * mstart + 15 * sbo + 7 + 2 * pitch + 2 + 1;
+    const int rows = std::max((TH + 2) * pitch, reach);
+    const int a_stride = (rows * p->rowb + 1023) / 1024 * 1024;
+    const int body = std::max(nchunk * a_stride + stages * bstage, 2 * 128 * BN * 2);
+    const int tail = (body + 15) / 16 * 16;
+    // at most 512/cols CTAs per SM: none ever waits for another's tensor memory
+    const int smem = std::max(tail + (int)sizeof(lbu::ConvTail), kSmemSm / (512 / cols + 1) - 1024 + 16);
+    if (smem > kSmemMax) return;
+    const int occ = std::min(std::min(kSmemSm / (smem + 1024), 512 / cols), 3);
+    if (occ < 1) return;
+    const int tiles_x = (W + TW - 1) / TW, tiles_y = (H + TH - 1) / TH;
+    const double ctas = (double)B * tiles_x * tiles_y * (cout / BN);
+    const double waves = std::ceil(ctas / (152.0 * occ));
+    const double mma = (double)nm * npar * ni * (p->rowb / 32) * 32;
+    const double copy = ((double)nchunk * (TH + 2) * pitch * p->rowb + (double)ni * bstage +
+                         (double)TH * TW * npar * BN * 2) / 50.0;
+    const double cost = waves * (4000.0 + occ * std::max(mma, copy));
+    if (cost >= best) return;
+    best = cost;
+    p->BN = BN;
+    p->smem = smem;
+    p->grid = dim3((unsigned)(B * tiles_x * tiles_y), (unsigned)(cout / BN));
+    lbu::ConvTma& a = p->a;
+    a.tiles_x = tiles_x;
+    a.tiles_y = tiles_y;
+    a.TH = TH;
+    a.TW = TW;
+    a.pitch = pitch;
+    a.nm = nm;
+    a.mstart = mstart;
+    a.sbo = sbo;
+    a.linear = linear ? 1 : 0;
+    a.nchunk = nchunk;
+    a.a_stride = a_stride;
+    a.nstage = stages;
+    a.cols = cols;
+    a.tail = tail;
+  };
+  for (int BN = 128; BN >= 32; BN /= 2) {
+    if (cout % BN) continue;
+    for (int k = 1; k <= 8; k *= 2)
+      if (8 * k < W + 8) consider(BN, 16, 8 * k, false);
+    for (int TH = 1; TH <= 16 && TH <= H; ++TH) consider(BN, TH, std::min(W, 126), true);
+  }
+  return best < 1e30;
+}
+
+ConvPlan conv_plan(const bf16* x, int xs, int B, int H, int W, int cin, int up, const bf16* w, const float* bias,
+                   int relu, bf16* y, int ys, int cout, const bf16* mask, int ms) {
+  ConvPlan p;
+  if (cin % 32 || cout % 32 || xs % 8 || ys % 8 || ms % 8) return p;
+  // whole 16-byte pieces are copied, loaded and stored
+  if ((((uintptr_t)x | (uintptr_t)w | (uintptr_t)y | (uintptr_t)mask) & 15u) != 0) return p;
+  const int Hi = H >> up, Wi = W >> up;
+  if (!plan_tile(B, Hi, Wi, cin, cout, up, &p)) return p;
+  lbu::ConvTma& a = p.a;
+  a.x = x;
+  a.xs = xs;
+  a.H = Hi;
+  a.W = Wi;
+  a.up = up;
+  a.bias = bias;
+  a.relu = relu;
+  a.y = y;
+  a.ys = ys;
+  a.mask = mask;
+  a.ms = ms;
+  const cuuint32_t ch = (cuuint32_t)(p.rowb / 2);
+  const cuuint64_t dx[4] = {(cuuint64_t)cin, (cuuint64_t)Wi, (cuuint64_t)Hi, (cuuint64_t)B};
+  const cuuint64_t sx[3] = {(cuuint64_t)xs * 2, (cuuint64_t)Wi * xs * 2, (cuuint64_t)Hi * Wi * xs * 2};
+  const cuuint32_t bx[4] = {ch, (cuuint32_t)a.TW + 2, (cuuint32_t)a.TH + 2, 1};
+  const cuuint64_t dw[2] = {(cuuint64_t)9 * cin, (cuuint64_t)cout};
+  const cuuint64_t sw[1] = {(cuuint64_t)9 * cin * 2};
+  const cuuint32_t bw[2] = {ch, (cuuint32_t)p.BN};
+  p.ok = encode_tiled(&p.mx, x, 4, dx, sx, bx, p.rowb) && encode_tiled(&p.mw, w, 2, dw, sw, bw, p.rowb);
+  return p;
+}
+
+template <int BN, int ROWB>
+cudaError_t launch_conv_tma(const ConvPlan& p, int* err, cudaStream_t s) {
+  static lbnci::SmemAllowance configured;
+  cudaError_t e = lbnci::allow_smem(lbu::conv3x3_tma_kernel<BN, ROWB>, (size_t)p.smem, configured);
+  if (e != cudaSuccess) return e;
+  lbu::conv3x3_tma_kernel<BN, ROWB><<<p.grid, lbu::kConvThreads, p.smem, s>>>(p.mx, p.mw, p.a, err);
+  return cudaGetLastError();
+}
+cudaError_t launch_conv_plan(const ConvPlan& p, cudaStream_t s) {
   int* err = nullptr;
   cudaError_t e = cudaGetSymbolAddress((void**)&err, g_tc_err);
   if (e != cudaSuccess) return e;
-  constexpr int smem = lbu::tc::Smem<BN, BK>::kBytes;
-  e = cudaFuncSetAttribute(lbu::conv3x3_tc_kernel<BN, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  grid.y = a.Cout / BN;
-  lbu::conv3x3_tc_kernel<BN, BK><<<grid, lbu::kTcThreads, smem, s>>>(a, err);
-  return cudaGetLastError();
-}
-// chunks of 32 input channels (stages of 10-16 KB: three to five CTAs of 8 warps per SM)
-template <int BN>
-cudaError_t launch_conv_tc(const lbu::ConvFwd& a, dim3 grid, cudaStream_t s) {
-  return launch_conv_tc_k<BN, 32>(a, grid, s);
+  if (p.rowb == 128)
+    return p.BN == 128 ? launch_conv_tma<128, 128>(p, err, s)
+                       : (p.BN == 64 ? launch_conv_tma<64, 128>(p, err, s) : launch_conv_tma<32, 128>(p, err, s));
+  return p.BN == 128 ? launch_conv_tma<128, 64>(p, err, s)
+                     : (p.BN == 64 ? launch_conv_tma<64, 64>(p, err, s) : launch_conv_tma<32, 64>(p, err, s));
 }
 
-// LBNCI_UNET_MMA=tcgen05 selects the tensor-memory convolution (unet_tc.cuh). It computes
-// the same sums (equal to the mma.sync kernel's bit for bit on the measured layers) but is
-// slower here: 7.1 ms against 5.5 ms per training step of batch 32 at 64 x 256; the
-// mma.sync kernel stays the default.
-bool conv_on_tcgen05() {
+// LBNCI_UNET_MMA=sync selects the mma.sync convolution for every layer. It stays for the
+// layers whose input tile does not fit in shared memory (more than about 512 channels).
+bool conv_on_mma_sync() {
   const char* e = std::getenv("LBNCI_UNET_MMA");
-  return e && std::strcmp(e, "tcgen05") == 0;
+  return e && std::strcmp(e, "sync") == 0;
+}
+
+// Tensor maps of a weight gradient's operands: boxes of the tile and its ring (x) and of the
+// tile (dy; when up, one map per parity of the output pixels).
+bool wgrad_maps(lbu::WgradMaps* m, const WgradTmaPlan& p, const bf16* x, int xs, const bf16* dy, int dys, int B) {
+  const lbu::WgradTma& a = p.a;
+  const cuuint64_t W = (cuuint64_t)a.W, H = (cuuint64_t)a.H, b = (cuuint64_t)B;
+  const cuuint64_t dx[4] = {(cuuint64_t)a.Cin, W, H, b};
+  const cuuint64_t sx[3] = {(cuuint64_t)xs * 2, W * xs * 2, H * W * xs * 2};
+  const cuuint32_t bx[4] = {(cuuint32_t)p.rowb / 2, (cuuint32_t)a.TW + 2, (cuuint32_t)a.TH + 2, 1};
+  if (!encode_tiled(&m->x, x, 4, dx, sx, bx, p.rowb)) return false;
+  const int f = a.up ? 2 : 1;
+  const cuuint64_t dd[4] = {(cuuint64_t)a.Cout, W, H, b};
+  const cuuint64_t sd[3] = {(cuuint64_t)f * dys * 2, (cuuint64_t)f * f * W * dys * 2, (cuuint64_t)f * f * H * W * dys * 2};
+  const cuuint32_t bd[4] = {(cuuint32_t)p.BN, (cuuint32_t)a.TW, (cuuint32_t)a.TH, 1};
+  for (int q = 0; q < 4; ++q) {
+    const bf16* base = a.up ? dy + ((size_t)(q >> 1) * f * W + (q & 1)) * dys : dy;
+    if (!encode_tiled(&m->dy[q], base, 4, dd, sd, bd, p.BN * 2)) return false;
+  }
+  return true;
+}
+
+template <int BN, int ROWB>
+cudaError_t launch_wgrad_tma(const WgradTmaPlan& p, const lbu::WgradMaps& maps, cudaStream_t s) {
+  static lbnci::SmemAllowance configured;
+  int* err = nullptr;
+  cudaError_t e = cudaGetSymbolAddress((void**)&err, g_tc_err);
+  if (e != cudaSuccess) return e;
+  e = lbnci::allow_smem(lbu::conv3x3_wgrad_tma_kernel<BN, ROWB>, (size_t)p.smem, configured);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((unsigned)p.a.nsplit, (unsigned)(p.a.Cin / (ROWB / 2)), (unsigned)(p.a.Cout / BN));
+  lbu::conv3x3_wgrad_tma_kernel<BN, ROWB><<<grid, lbu::kConvThreads, p.smem, s>>>(maps, p.a, err);
+  return cudaGetLastError();
 }
 
 // Reports (and clears) an expired wait of a tensor-core convolution; call after a
@@ -219,19 +446,26 @@ lb_status check_tc(lbu_net* n) {
   return LB_OK;
 }
 
-// one 3x3 convolution launch (forward or data gradient)
-lb_status conv(lbu_net* n, const bf16* x, int xs, int B, int H, int W, int cin, int up, const bf16* w,
+// one 3x3 convolution launch (forward or data gradient); site: the network's cache slot
+lb_status conv(lbu_net* n, int site, const bf16* x, int xs, int B, int H, int W, int cin, int up, const bf16* w,
                const float* bias, int relu, bf16* y, int ys, int cout, const bf16* mask, int ms,
                cudaStream_t s) {
+  if (!conv_on_mma_sync()) {
+    ConvCache once;
+    ConvCache& c = n ? n->conv_cache[site] : once;
+    if (c.B != B) {
+      c.p = conv_plan(x, xs, B, H, W, cin, up, w, bias, relu, y, ys, cout, mask, ms);
+      c.B = B;
+    }
+    if (c.p.ok) {
+      cudaError_t e = launch_conv_plan(c.p, s);
+      if (n) ++n->launches;
+      return e == cudaSuccess ? LB_OK : cuda_fail(n, e, "conv3x3 (tensor memory) launch");
+    }
+  }
   lbu::ConvFwd a{x, xs, B, H, W, cin, up, w, bias, relu, y, ys, cout, mask, ms};
   const int M = B * H * W;
   dim3 grid((M + lbu::kConvBM - 1) / lbu::kConvBM, 1);
-  if (conv_on_tcgen05()) {
-    cudaError_t e = cout % 128 == 0 ? launch_conv_tc<128>(a, grid, s)
-                                    : (cout % 64 == 0 ? launch_conv_tc<64>(a, grid, s) : launch_conv_tc<32>(a, grid, s));
-    if (n) ++n->launches;
-    return e == cudaSuccess ? LB_OK : cuda_fail(n, e, "conv3x3 (tcgen05) launch");
-  }
   if (cout % 64 == 0) {
     grid.y = cout / 64;
     lbu::conv3x3_kernel<64><<<grid, 128, 0, s>>>(a);
@@ -244,9 +478,41 @@ lb_status conv(lbu_net* n, const bf16* x, int xs, int B, int H, int W, int cin, 
   return e == cudaSuccess ? LB_OK : cuda_fail(n, e, "conv3x3 launch");
 }
 
-lb_status wgrad(lbu_net* n, const bf16* x, int xs, int up, const bf16* dy, int dys, int B, int H, int W, int cin,
+lb_status wgrad(lbu_net* n, int site, const bf16* x, int xs, int up, const bf16* dy, int dys, int B, int H, int W, int cin,
                 int cout, float* work, size_t work_bytes, cudaStream_t s, float* dw_master, float* db_master,
                 int cin_true) {
+  if (!conv_on_mma_sync() && xs % 8 == 0 && dys % 8 == 0 && (((uintptr_t)x | (uintptr_t)dy) & 15u) == 0) {
+    WgradCache once;
+    WgradCache& c = n ? n->wgrad_cache[site] : once;
+    if (c.B != B) {
+      c.p = wgrad_tma_plan(B, H >> up, W >> up, cin, cout, up);
+      c.p.ok = c.p.ok && wgrad_maps(&c.maps, c.p, x, xs, dy, dys, B);
+      c.B = B;
+    }
+    WgradTmaPlan& p = c.p;
+    const lbu::WgradMaps& maps = c.maps;
+    if (p.ok && wgrad_tma_bytes(p) <= work_bytes) {
+      p.a.x = x;
+      p.a.xs = xs;
+      p.a.part = work;
+      float* bp = work + (size_t)p.a.nsplit * cout * (up ? 16 : 9) * cin;
+      p.a.bpart = db_master ? bp : nullptr;
+      cudaError_t e = p.rowb == 128 ? (p.BN == 64 ? launch_wgrad_tma<64, 128>(p, maps, s)
+                                                  : launch_wgrad_tma<32, 128>(p, maps, s))
+                                    : (p.BN == 64 ? launch_wgrad_tma<64, 64>(p, maps, s)
+                                                  : launch_wgrad_tma<32, 64>(p, maps, s));
+      if (e != cudaSuccess) return cuda_fail(n, e, "wgrad (tensor memory) launch");
+      const int n4 = cout * 9 * cin / 4;
+      int S = 1;  // threads to each group of four values: about four blocks per multiprocessor
+      while (S < 32 && 2 * S <= p.a.nsplit && (long long)n4 * S < 152LL * 4 * 256) S *= 2;
+      const int wblocks = (n4 + 256 / S - 1) / (256 / S), bblocks = db_master ? (cout + 31) / 32 : 0;
+      lbu::wgrad_reduce_tma_kernel<<<wblocks + bblocks, 256, 0, s>>>(work, bp, p.a.nsplit, cout, cin, cin_true, up, S,
+                                                                     wblocks, dw_master, db_master);
+      if (n) n->launches += 2;
+      e = cudaGetLastError();
+      return e == cudaSuccess ? LB_OK : cuda_fail(n, e, "wgrad reduction launch");
+    }
+  }
   const WgradPlan p = wgrad_plan(B * H * W, cin, cout);
   if (wgrad_bytes(p, cin, cout) > work_bytes) return fail(n, LB_EINVAL, "wgrad scratch too small");
   float* part = work;
@@ -288,10 +554,10 @@ lb_status forward_impl(lbu_net* n, int B) {
   int hs = kInPad;
   for (int l = 0; l < Lv; ++l) {
     const int C = width(n, l), H = Hl(n, l), W = Wl(n, l);
-    LBU_TRY(conv(n, h, hs, B, H, W, n->L[enc_a(l)].cin_pad, 0, WB(n, enc_a(l)), BIAS(n, enc_a(l)), 1, n->ea[l], C,
+    LBU_TRY(conv(n, enc_a(l), h, hs, B, H, W, n->L[enc_a(l)].cin_pad, 0, WB(n, enc_a(l)), BIAS(n, enc_a(l)), 1, n->ea[l], C,
                  C, nullptr, 0, s));
     if (l < Lv - 1) {
-      LBU_TRY(conv(n, n->ea[l], C, B, H, W, C, 0, WB(n, enc_b(l)), BIAS(n, enc_b(l)), 1, n->cat[l] + C, 2 * C, C,
+      LBU_TRY(conv(n, enc_b(l), n->ea[l], C, B, H, W, C, 0, WB(n, enc_b(l)), BIAS(n, enc_b(l)), 1, n->cat[l] + C, 2 * C, C,
                    nullptr, 0, s));
       const long long work = (long long)B * (H / 2) * (W / 2) * (C / 8);
       lbu::maxpool_kernel<<<grid_for(work, 256), 256, 0, s>>>(n->cat[l] + C, 2 * C, B, H, W, C, n->pool[l]);
@@ -299,7 +565,7 @@ lb_status forward_impl(lbu_net* n, int B) {
       h = n->pool[l];
       hs = C;
     } else {
-      LBU_TRY(conv(n, n->ea[l], C, B, H, W, C, 0, WB(n, enc_b(l)), BIAS(n, enc_b(l)), 1, n->db[l], C, C, nullptr,
+      LBU_TRY(conv(n, enc_b(l), n->ea[l], C, B, H, W, C, 0, WB(n, enc_b(l)), BIAS(n, enc_b(l)), 1, n->db[l], C, C, nullptr,
                    0, s));
       h = n->db[l];
       hs = C;
@@ -307,10 +573,10 @@ lb_status forward_impl(lbu_net* n, int B) {
   }
   for (int l = Lv - 2; l >= 0; --l) {
     const int C = width(n, l), H = Hl(n, l), W = Wl(n, l), k = up_i(n, l);
-    LBU_TRY(conv(n, h, hs, B, H, W, 2 * C, 1, WB(n, k), BIAS(n, k), 1, n->cat[l], 2 * C, C, nullptr, 0, s));
-    LBU_TRY(conv(n, n->cat[l], 2 * C, B, H, W, 2 * C, 0, WB(n, k + 1), BIAS(n, k + 1), 1, n->da[l], C, C, nullptr,
+    LBU_TRY(conv(n, k, h, hs, B, H, W, 2 * C, 1, WB(n, k), BIAS(n, k), 1, n->cat[l], 2 * C, C, nullptr, 0, s));
+    LBU_TRY(conv(n, k + 1, n->cat[l], 2 * C, B, H, W, 2 * C, 0, WB(n, k + 1), BIAS(n, k + 1), 1, n->da[l], C, C, nullptr,
                  0, s));
-    LBU_TRY(conv(n, n->da[l], C, B, H, W, C, 0, WB(n, k + 2), BIAS(n, k + 2), 1, n->db[l], C, C, nullptr, 0, s));
+    LBU_TRY(conv(n, k + 2, n->da[l], C, B, H, W, C, 0, WB(n, k + 2), BIAS(n, k + 2), 1, n->db[l], C, C, nullptr, 0, s));
     h = n->db[l];
     hs = C;
   }
@@ -327,6 +593,7 @@ lb_status backward_impl(lbu_net* n, int B) {
   const int Lv = n->cfg.levels;
   cudaStream_t s = n->stream;
   const int P = B * n->cfg.H * n->cfg.W;
+  const int nl = (int)n->L.size();
   float* G = n->grads;
   auto GW = [&](int i) { return G + n->L[i].w_off; };
   auto GB = [&](int i) { return G + n->L[i].b_off; };
@@ -335,7 +602,7 @@ lb_status backward_impl(lbu_net* n, int B) {
     const int hi = head_i(n), C0 = n->cfg.base;
     const int nblk = (P + lbu::kHeadPix - 1) / lbu::kHeadPix;
     lbu::head_bwd_kernel<<<nblk, 256, 0, s>>>(n->db[0], C0, WB(n, hi), n->cfg.out_ch, P, n->dy, n->gB[0], n->work);
-    lbu::head_reduce_kernel<<<1, 256, 0, s>>>(n->work, nblk, n->cfg.out_ch, C0, GW(hi), GB(hi));
+    lbu::head_reduce_kernel<<<n->cfg.out_ch * (C0 + 1), 128, 0, s>>>(n->work, nblk, n->cfg.out_ch, C0, GW(hi), GB(hi));
     n->launches += 2;
   }
   // decoder, finest level first
@@ -343,17 +610,17 @@ lb_status backward_impl(lbu_net* n, int B) {
     const int C = width(n, l), H = Hl(n, l), W = Wl(n, l), k = up_i(n, l);
     const int C1 = width(n, l + 1);
     // dec_lb: input da[l], output gradient gB[l]
-    LBU_TRY(wgrad(n, n->da[l], C, 0, n->gB[l], C, B, H, W, C, C, n->work, n->work_bytes, s, GW(k + 2), GB(k + 2), C));
-    LBU_TRY(conv(n, n->gB[l], C, B, H, W, C, 0, WT(n, k + 2), nullptr, 0, n->gA[l], C, C, n->da[l], C, s));
+    LBU_TRY(wgrad(n, k + 2, n->da[l], C, 0, n->gB[l], C, B, H, W, C, C, n->work, n->work_bytes, s, GW(k + 2), GB(k + 2), C));
+    LBU_TRY(conv(n, nl + k + 2, n->gB[l], C, B, H, W, C, 0, WT(n, k + 2), nullptr, 0, n->gA[l], C, C, n->da[l], C, s));
     // dec_la: input cat[l]
-    LBU_TRY(wgrad(n, n->cat[l], 2 * C, 0, n->gA[l], C, B, H, W, 2 * C, C, n->work, n->work_bytes, s, GW(k + 1),
+    LBU_TRY(wgrad(n, k + 1, n->cat[l], 2 * C, 0, n->gA[l], C, B, H, W, 2 * C, C, n->work, n->work_bytes, s, GW(k + 1),
                   GB(k + 1), 2 * C));
-    LBU_TRY(conv(n, n->gA[l], C, B, H, W, C, 0, WT(n, k + 1), nullptr, 0, n->gCat[l], 2 * C, 2 * C, n->cat[l],
+    LBU_TRY(conv(n, nl + k + 1, n->gA[l], C, B, H, W, C, 0, WT(n, k + 1), nullptr, 0, n->gCat[l], 2 * C, 2 * C, n->cat[l],
                  2 * C, s));
     // up_l: input = nearest upsampling of the level-(l+1) output
     const bf16* hin = n->db[l + 1];
-    LBU_TRY(wgrad(n, hin, C1, 1, n->gCat[l], 2 * C, B, H, W, C1, C, n->work, n->work_bytes, s, GW(k), GB(k), C1));
-    LBU_TRY(conv(n, n->gCat[l], 2 * C, B, H, W, C, 0, WT(n, k), nullptr, 0, n->gU[l], C1, C1, nullptr, 0, s));
+    LBU_TRY(wgrad(n, k, hin, C1, 1, n->gCat[l], 2 * C, B, H, W, C1, C, n->work, n->work_bytes, s, GW(k), GB(k), C1));
+    LBU_TRY(conv(n, nl + k, n->gCat[l], 2 * C, B, H, W, C, 0, WT(n, k), nullptr, 0, n->gU[l], C1, C1, nullptr, 0, s));
     const long long work = (long long)B * Hl(n, l + 1) * Wl(n, l + 1) * (C1 / 8);
     lbu::upsample_bwd_kernel<<<grid_for(work, 256), 256, 0, s>>>(n->gU[l], hin, n->gB[l + 1], B, Hl(n, l + 1),
                                                                  Wl(n, l + 1), C1);
@@ -375,14 +642,14 @@ lb_status backward_impl(lbu_net* n, int B) {
       g = n->gCat[l] + C;
       gs = 2 * C;
     }
-    LBU_TRY(wgrad(n, n->ea[l], C, 0, g, gs, B, H, W, C, C, n->work, n->work_bytes, s, GW(enc_b(l)), GB(enc_b(l)), C));
-    LBU_TRY(conv(n, g, gs, B, H, W, C, 0, WT(n, enc_b(l)), nullptr, 0, n->gA[l], C, C, n->ea[l], C, s));
+    LBU_TRY(wgrad(n, enc_b(l), n->ea[l], C, 0, g, gs, B, H, W, C, C, n->work, n->work_bytes, s, GW(enc_b(l)), GB(enc_b(l)), C));
+    LBU_TRY(conv(n, nl + enc_b(l), g, gs, B, H, W, C, 0, WT(n, enc_b(l)), nullptr, 0, n->gA[l], C, C, n->ea[l], C, s));
     const bf16* xin = l == 0 ? n->x0 : n->pool[l - 1];
     const int cin = n->L[enc_a(l)].cin_pad;
-    LBU_TRY(wgrad(n, xin, cin, 0, n->gA[l], C, B, H, W, cin, C, n->work, n->work_bytes, s, GW(enc_a(l)),
+    LBU_TRY(wgrad(n, enc_a(l), xin, cin, 0, n->gA[l], C, B, H, W, cin, C, n->work, n->work_bytes, s, GW(enc_a(l)),
                   GB(enc_a(l)), n->L[enc_a(l)].cin));
     if (l > 0)
-      LBU_TRY(conv(n, n->gA[l], C, B, H, W, C, 0, WT(n, enc_a(l)), nullptr, 0, n->gPool[l - 1], cin, cin, nullptr,
+      LBU_TRY(conv(n, nl + enc_a(l), n->gA[l], C, B, H, W, C, 0, WT(n, enc_a(l)), nullptr, 0, n->gPool[l - 1], cin, cin, nullptr,
                    0, s));
   }
   cudaError_t e = cudaGetLastError();
@@ -406,7 +673,7 @@ lb_status loss_impl(lbu_net* n, const float* T, const int* idx, int B, const flo
   const int blocks = std::min(n->npartial, grid_for(P, 256));
   lbu::mse_kernel<<<blocks, 256, 0, n->stream>>>(n->y, T, idx, HW, n->cfg.out_ch, P, lm[0], lm[1], lm[2], lm[3],
                                                  lm[4], lm[5], lm[6], lm[7], n->dy, n->partial);
-  lbu::sum_partials_kernel<<<1, 32, 0, n->stream>>>(n->partial, blocks, 1.0 / P, n->loss);
+  lbu::sum_partials_kernel<<<1, 256, 0, n->stream>>>(n->partial, blocks, 1.0 / P, n->loss);
   n->launches += 2;
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? LB_OK : cuda_fail(n, e, "loss launch");
@@ -474,6 +741,8 @@ lb_status lbu_create(const lbu_config* cfg, lbu_net** out) {
   cudaGetDevice(&n->device);
   n->L = layer_table(cfg);
   n->nparams = total_params(n->L);
+  n->conv_cache.resize(2 * n->L.size());
+  n->wgrad_cache.resize(n->L.size());
   const int Lv = cfg->levels, B = cfg->max_batch;
   auto bail = [&](lb_status st) {
     g_err = n->err;
@@ -541,10 +810,9 @@ lb_status lbu_create(const lbu_config* cfg, lbu_net** out) {
   // scratch: the largest wgrad partial set and the head partials
   size_t wb = 0;
   for (int l = 0; l < Lv; ++l) {
-    const int P = (int)((size_t)B * (HW >> (2 * l)));
     const int C = width(n, l);
     const int cins[4] = {l == 0 ? kInPad : width(n, l - 1), C, 2 * C, l < Lv - 1 ? width(n, l + 1) : C};
-    for (int ci : cins) wb = std::max(wb, wgrad_bytes(wgrad_plan(P, ci, C), ci, C));
+    for (int ci : cins) wb = std::max(wb, wgrad_work(B, Hl(n, l), Wl(n, l), ci, C));
   }
   const size_t nblk = ((size_t)B * HW + lbu::kHeadPix - 1) / lbu::kHeadPix;
   wb = std::max(wb, nblk * cfg->out_ch * (cfg->base + 1) * sizeof(float));
@@ -680,13 +948,13 @@ lb_status lbu_conv3x3(const unsigned short* x, int x_stride, int batch, int h, i
   if (x_stride < c_in || y_stride < c_out || x_stride % 8 || y_stride % 8)
     return fail(nullptr, LB_EINVAL, "strides: at least the channel count, multiples of 8");
   if (upsample && (h % 2 || w % 2)) return fail(nullptr, LB_EINVAL, "upsampled output must have even size");
-  return conv(nullptr, (const bf16*)x, x_stride, batch, h, w, c_in, upsample ? 1 : 0, (const bf16*)wgt, bias, relu,
+  return conv(nullptr, 0, (const bf16*)x, x_stride, batch, h, w, c_in, upsample ? 1 : 0, (const bf16*)wgt, bias, relu,
               (bf16*)y, y_stride, c_out, nullptr, 0, (cudaStream_t)stream);
 }
 
 size_t lbu_conv3x3_wgrad_work(int batch, int h, int w, int c_in, int c_out) {
   if (batch <= 0 || h <= 0 || w <= 0 || c_in <= 0 || c_out <= 0) return 0;
-  return wgrad_bytes(wgrad_plan(batch * h * w, c_in, c_out), c_in, c_out);
+  return wgrad_work(batch, h, w, c_in, c_out);
 }
 
 lb_status lbu_conv3x3_wgrad(const unsigned short* x, int x_stride, int batch, int h, int w, int c_in, int upsample,
@@ -698,7 +966,7 @@ lb_status lbu_conv3x3_wgrad(const unsigned short* x, int x_stride, int batch, in
   if (x_stride < c_in || dy_stride < c_out || x_stride % 8 || dy_stride % 8)
     return fail(nullptr, LB_EINVAL, "strides: at least the channel count, multiples of 8");
   if (upsample && (h % 2 || w % 2)) return fail(nullptr, LB_EINVAL, "upsampled output must have even size");
-  return wgrad(nullptr, (const bf16*)x, x_stride, upsample ? 1 : 0, (const bf16*)dy, dy_stride, batch, h, w, c_in,
+  return wgrad(nullptr, 0, (const bf16*)x, x_stride, upsample ? 1 : 0, (const bf16*)dy, dy_stride, batch, h, w, c_in,
                c_out, (float*)work, work_bytes, (cudaStream_t)stream, dw, db, c_in);
 }
 

@@ -1,0 +1,782 @@
+// unet_conv.cuh -- the U-Net's 3x3 convolution (forward and data gradient) on the
+// fifth-generation tensor cores, operands copied by TMA, accumulators in tensor memory.
+//
+// Implicit GEMM, D[m][n] = sum_k A[m][k] B[n][k] with m a pixel, n an output channel and
+// k = (tap, input channel). A CTA owns a tile of TH x TW pixels of one image and BN output
+// channels. Its input, the tile and a ring of one pixel with all input channels, is copied
+// once into shared memory (one TMA box per chunk of 64 or 32 channels: a pixel's chunk is a
+// 128- or 64-byte row of the swizzled K-major operand layout). Every tap then reads that
+// one copy: the operand of tap (dy, dx) starts dy pitch + dx rows further on (pitch = TW +
+// 2 pixels), so a tap costs no copy and shared memory holds each input pixel once instead
+// of nine times. 8-row groups of the 128-row operand are eight neighbouring pixels of an
+// image row; they lie `sbo` pixels apart:
+//   patch   sbo = pitch: 16 image rows x 8 columns, every row of the operand a pixel
+//   linear  sbo = 8:     128 consecutive positions of the pitched tile; the two ring
+//                        columns of each row are computed and dropped (images with too
+//                        few rows, or columns that are no multiple of eight)
+// The swizzle is a function of the shared-memory address, so a start anywhere in a
+// 1024-byte pattern reads what the copy wrote (matrix base offset 0: the patterns
+// themselves are aligned). Rows beyond the first and last image row arrive as the copy's
+// zero fill; the periodic columns beyond the first and last image column also arrive as
+// zeros and are overwritten with their images by the epilogue warps.
+//
+// Upsampled input (up = 1, nearest 2x): output pixel (2 y + py, 2 x + px) reads input row
+// floor((2 y + py + dy)/2), so each of the four parities (py, px) is a 3x3-tap sum over
+// shifts -1, 0, 1 of the low-resolution tile: four accumulators over the same operands,
+// nothing upsampled in memory.
+//
+// The weights stream through a ring of stages, one (tap, chunk) each, in k order; per stage
+// one thread issues the K = 16 MMAs of every accumulator. So each accumulator adds the
+// same K = 16 products in the same order as conv3x3_kernel's, tap by tap, channels
+// ascending, and gives the same bits.
+//
+// Warps: 0 copies, 1 issues MMAs (and owns the tensor memory), 2..9 patch the periodic
+// columns, then drain the accumulators: bias, ReLU, BF16, through shared memory so that
+// the mask's loads and the output's stores are whole lines.
+//
+// What bounds it: an MMA of M = 128, K = 16 takes about 60 cycles up to N = 128 (the fetch of
+// A), and the copy before and the drain after a tile's MMAs are hidden only by the other
+// CTA of the multiprocessor, where two fit. Measured on GB300 against the mma.sync kernel
+// (conv3x3_kernel), 32 images: 32 -> 32 channels at 64 x 256, 37 us (72 us); 256 -> 256 at
+// 8 x 32, 25 us (75 us).
+//
+// Every mbarrier wait is bounded (about a second of %globaltimer); on expiry the kernel
+// sets its error word, waits (bounded) for the copies and MMAs in flight, releases its
+// tensor memory and writes no further output.
+#pragma once
+
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <stdint.h>
+
+#include "lb_tma.cuh"
+#include "unet_kernels.cuh"
+
+namespace lbu {
+namespace tc {
+
+// Shared-memory matrix descriptor of a swizzled operand: start address, leading byte
+// offset (unused by the K-major swizzled layouts), stride byte offset between 8-row groups
+// (all in 16-byte units), version 1 (bits 46-47), layout type at bits 61-63 (2: 128-byte
+// swizzle, 4: 64-byte swizzle).
+__host__ __device__ constexpr unsigned long long desc_base(int rowb, unsigned lbo, unsigned sbo) {
+  return ((unsigned long long)((lbo >> 4) & 0x3FFFu) << 16) | ((unsigned long long)((sbo >> 4) & 0x3FFFu) << 32) |
+         (1ull << 46) | ((rowb == 128 ? 2ull : 4ull) << 61);
+}
+
+// Instruction descriptor of kind::f16: FP32 accumulator (bits 4-5 = 1), BF16 A and B (bits
+// 7-9 and 10-12 = 1), A and B K-major (bits 15, 16 = 0) or MN-major (= 1), N >> 3 at bits
+// 17-22, M >> 4 at 24-28.
+__host__ __device__ constexpr unsigned idesc_bf16(int M, int N, bool mn_major = false) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (mn_major ? (3u << 15) : 0u) | ((unsigned)(N >> 3) << 17) |
+         ((unsigned)(M >> 4) << 24);
+}
+
+__device__ __forceinline__ void tmem_alloc(unsigned* s_addr, unsigned ncols) {  // one whole warp
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_addr)),
+               "r"(ncols)
+               : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc(unsigned taddr, unsigned ncols) {  // one whole warp
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+__device__ __forceinline__ void fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+// D (tensor memory) = A B^T (+ D when accumulate), issued by the one lane whose `leader` is
+// nonzero. The whole warp runs the issue loop, so that its addresses and descriptors are
+// warp-uniform values: issued from a branch that one lane took, each MMA cost 80 to 140
+// cycles of moves between register files, three times what the tensor cores take.
+template <bool ACC>
+__device__ __forceinline__ void mma_bf16(unsigned tmem_d, unsigned long long a, unsigned long long b, unsigned idesc,
+                                         unsigned leader) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "l"(a), "l"(b), "r"(idesc), "n"(ACC ? 1 : 0), "r"(leader)
+      : "memory");
+}
+// Descriptor from its constant upper half and the lower half at a shared-memory address.
+__device__ __forceinline__ unsigned long long desc64(unsigned hi, unsigned lo) {
+  return ((unsigned long long)hi << 32) | lo;
+}
+// The K = 16 MMAs kk = 0 .. KK - 1 of one stage for G accumulators (d + g dstep), whose A
+// operands start at the descriptors lo[g]: unrolled, accumulators innermost, so that an MMA
+// costs a few instructions of the issuing warp and seldom follows one into its accumulator.
+template <int G, int KK, bool ACC>
+__device__ __forceinline__ void mma_group(unsigned d, unsigned dstep, const unsigned lo[G], unsigned hiA, unsigned loB,
+                                          unsigned hiB, unsigned idesc, unsigned leader) {
+#pragma unroll
+  for (int kk = 0; kk < KK; ++kk)
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      if (ACC || kk > 0) mma_bf16<true>(d + g * dstep, desc64(hiA, lo[g] + 2 * kk), desc64(hiB, loB + 2 * kk), idesc, leader);
+      else mma_bf16<false>(d + g * dstep, desc64(hiA, lo[g]), desc64(hiB, loB), idesc, leader);
+    }
+}
+// The mbarrier receives one arrival when every MMA the leader issued before has completed.
+__device__ __forceinline__ void mma_commit(unsigned long long* bar, unsigned leader) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)),
+      "r"(leader)
+      : "memory");
+}
+// 16 consecutive 32-bit columns of this thread's lane (shape 32x32b: lane = warp's base + lane id)
+__device__ __forceinline__ void tmem_ld16(unsigned taddr, float v[16]) {
+  unsigned r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+      "%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// Offset of 16-byte piece v of row r in a swizzled operand of ROWB-byte rows whose patterns
+// (8 rows of 128 bytes, or of 64) are aligned.
+template <int ROWB>
+__device__ __forceinline__ unsigned swizzled(int r, int v) {
+  const unsigned off = (unsigned)r * ROWB + (unsigned)v * 16u;
+  return off ^ (((off >> 7) & (ROWB == 128 ? 7u : 3u)) << 4);
+}
+
+}  // namespace tc
+
+constexpr int kConvThreads = 320;  // copy warp, MMA warp, eight epilogue warps
+constexpr int kConvEpiThreads = 256;
+
+struct ConvTma {
+  const bf16* x;      // input, for the periodic columns
+  int xs, H, W;       // input pixel stride and image: the grid of positions
+  int up;             // 1: the output is 2H x 2W
+  int tiles_x, tiles_y, TH, TW, pitch;
+  int nm, mstart, sbo;  // M tiles (per parity), positions between their starts, between 8-row groups
+  int linear;         // position p of M tile m: (p / pitch, p % pitch), else (l / 8, 8 m + l % 8)
+  int nchunk;         // chunks of ROWB/2 input channels
+  int a_stride;       // bytes of a chunk's tile in shared memory
+  int nstage;         // ring stages of the weights
+  int cols;           // tensor-memory columns (a power of two)
+  int tail;           // offset of the ConvTail behind the tile, the ring and the output staging
+  const float* bias;
+  int relu;
+  bf16* y;
+  int ys;
+  const bf16* mask;
+  int ms;
+};
+
+constexpr int kConvMaxStage = 24;
+struct ConvTail {
+  unsigned long long bar_a, bar_p, bar_d, bar_full[kConvMaxStage], bar_empty[kConvMaxStage];
+  unsigned tmem;
+  int fail;
+  float bias[128];
+};
+
+template <int BN, int ROWB>
+__global__ void __launch_bounds__(kConvThreads, 3)
+conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w, ConvTma a,
+                   int* err) {
+  constexpr int CH = ROWB / 2, KK = CH / 16;  // channels and K = 16 MMAs of a chunk
+  constexpr int BBYTES = BN * ROWB;
+  constexpr unsigned IDESC = tc::idesc_bf16(128, BN);
+  extern __shared__ __align__(1024) unsigned char sm[];  // no static shared memory: it starts the window
+  ConvTail& t = *reinterpret_cast<ConvTail*>(sm + a.tail);
+  unsigned char* const sA = sm;
+  unsigned char* const sB = sm + a.nchunk * a.a_stride;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tx = blockIdx.x % a.tiles_x, ty = (blockIdx.x / a.tiles_x) % a.tiles_y;
+  const int b = blockIdx.x / (a.tiles_x * a.tiles_y);
+  const int x0 = tx * a.TW, y0 = ty * a.TH, n0 = blockIdx.y * BN;
+  const int ni = 9 * a.nchunk, ST = a.nstage;
+
+  if (tid == 0) {
+    lbnci::mbar_init(&t.bar_a, 1);
+    lbnci::mbar_init(&t.bar_p, kConvEpiThreads / 32);
+    lbnci::mbar_init(&t.bar_d, 2);
+    for (int s = 0; s < ST; ++s) {
+      lbnci::mbar_init(&t.bar_full[s], 1);
+      lbnci::mbar_init(&t.bar_empty[s], 1);
+    }
+    t.fail = (smem_u32(sm) & 1023u) ? 2 : 0;  // the patterns need the alignment: report, do nothing
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) tc::tmem_alloc(&t.tmem, (unsigned)a.cols);
+  if (tid < BN) t.bias[tid] = a.bias ? a.bias[n0 + tid] : 0.f;
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const unsigned tmem = t.tmem;
+  const bool aligned = t.fail == 0;
+
+  if (!aligned) {
+    // nothing was started
+  } else if (warp == 0) {
+    if (lane == 0) {  // copies: the input tile, then the weights through the ring
+      lbnci::mbar_expect_tx(&t.bar_a, (unsigned)(a.nchunk * ROWB * (a.TW + 2) * (a.TH + 2)));
+      for (int k = 0; k < a.nchunk; ++k)
+        lbnci::tma_load_4d(sA + k * a.a_stride, &map_x, k * CH, x0 - 1, y0 - 1, b, &t.bar_a);
+      int issued = 0;
+      for (int i = 0; i < ni; ++i) {
+        const int s = i % ST, u = i / ST;
+        if (u > 0 && !lbnci::mbar_wait(&t.bar_empty[s], (unsigned)((u - 1) & 1))) {
+          atomicOr(&t.fail, 1);
+          break;
+        }
+        lbnci::mbar_expect_tx(&t.bar_full[s], BBYTES);
+        lbnci::tma_load_2d(sB + s * BBYTES, &map_w, i * CH, n0, &t.bar_full[s]);
+        issued = i + 1;
+      }
+      // before the CTA may end: every copy has landed (bounded; each was waited for by the
+      // MMA warp unless a wait ran out)
+      lbnci::mbar_wait(&t.bar_a, 0u);
+      for (int i = issued > ST ? issued - ST : 0; i < issued; ++i)
+        lbnci::mbar_wait(&t.bar_full[i % ST], (unsigned)((i / ST) & 1));
+    }
+  } else if (warp == 1) {  // MMAs: the whole warp, lane 0 issues
+    const unsigned leader = lane == 0;
+    bool bad = __any_sync(~0u, !lbnci::mbar_wait(&t.bar_a, 0u) || !lbnci::mbar_wait(&t.bar_p, 0u));
+    const unsigned long long dA = tc::desc_base(ROWB, 16u, (unsigned)(a.sbo * ROWB));
+    const unsigned long long dB = tc::desc_base(ROWB, 16u, 8u * ROWB);
+    const unsigned hiA = (unsigned)(dA >> 32), hiB = (unsigned)(dB >> 32);
+    // lower halves in 16-byte units: addresses below 256 KB never carry out of their field
+    const unsigned loA0 = (unsigned)dA + (smem_u32(sA) >> 4), loB0 = (unsigned)dB + (smem_u32(sB) >> 4);
+    const unsigned mstep = (unsigned)(a.mstart * ROWB) >> 4;
+    unsigned ph = 0u;
+    int s = 0;
+    auto stage = [&](int tap, int k, auto ACC) {
+      constexpr bool acc = decltype(ACC)::value;
+      const int dy = tap / 3 - 1, dx = tap % 3 - 1;
+      const unsigned lb = loB0 + (unsigned)(s * (BBYTES >> 4)), la = loA0 + (unsigned)((k * a.a_stride) >> 4);
+      auto at = [&](int oy, int ox) { return la + (unsigned)((((oy + 1) * a.pitch + ox + 1) * ROWB) >> 4); };
+      if (a.up) {
+        // the four parities of an upsampled input: low-resolution row and column
+        // floor((parity + tap)/2)
+        unsigned lo[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) lo[q] = at(((q >> 1) + dy) >> 1, ((q & 1) + dx) >> 1);
+        for (int m = 0; m < a.nm; ++m) {
+          tc::mma_group<4, KK, acc>(tmem + m * BN, (unsigned)(a.nm * BN), lo, hiA, lb, hiB, IDESC, leader);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) lo[q] += mstep;
+        }
+      } else {
+        unsigned lo[4];
+        lo[0] = at(dy, dx);
+        lo[1] = lo[0] + mstep;
+        lo[2] = lo[1] + mstep;
+        lo[3] = lo[2] + mstep;
+        int m = 0;
+        for (; m + 4 <= a.nm; m += 4) {
+          tc::mma_group<4, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC, leader);
+#pragma unroll
+          for (int g = 0; g < 4; ++g) lo[g] += 4 * mstep;
+        }
+        if (a.nm - m == 3) tc::mma_group<3, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC, leader);
+        else if (a.nm - m == 2) tc::mma_group<2, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC, leader);
+        else if (a.nm - m == 1) tc::mma_group<1, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC, leader);
+      }
+      tc::mma_commit(&t.bar_empty[s], leader);
+      if (++s == ST) {
+        s = 0;
+        ph ^= 1u;
+      }
+    };
+    for (int tap = 0; tap < 9 && !bad; ++tap)
+      for (int k = 0; k < a.nchunk; ++k) {
+        bad = __any_sync(~0u, !lbnci::mbar_wait(&t.bar_full[s], ph));
+        if (bad) break;
+        tc::fence_after_sync();
+        if (tap == 0 && k == 0) stage(tap, k, std::false_type{});
+        else stage(tap, k, std::true_type{});
+      }
+    if (lane == 0) {
+      if (bad) atomicOr(&t.fail, 1);
+    }
+    tc::mma_commit(&t.bar_d, leader);
+    if (lane == 0) lbnci::mbar_arrive(&t.bar_d);
+  } else {
+    const int et = tid - 64;
+    {  // the periodic images of the columns beyond the image: pieces of 16 bytes
+      const int vpp = a.nchunk * (ROWB / 16);
+      const int left = x0 == 0 ? 1 : 0, right = x0 + a.TW >= a.W ? 1 : 0;
+      const int ncol = left + right, count = ncol * (a.TH + 2) * vpp;
+      bool ok = true;
+      constexpr int U = 4;
+      for (int e0 = 0; e0 < count && ok; e0 += U * kConvEpiThreads) {
+        uint4 v[U];
+        int dst[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+          const int e = e0 + j * kConvEpiThreads + et;
+          dst[j] = -1;
+          if (e < count) {
+            const int px = e / vpp, p = e - px * vpp;
+            const int row = px / ncol, col = px - row * ncol;
+            const int yy = y0 - 1 + row;
+            if (yy >= 0 && yy < a.H) {
+              const bool lft = left && col == 0;
+              v[j] = *reinterpret_cast<const uint4*>(a.x + ((size_t)(b * a.H + yy) * a.W + (lft ? a.W - 1 : 0)) * a.xs +
+                                                     p * 8);
+              const int r = row * a.pitch + (lft ? 0 : a.W - x0 + 1);
+              const int k = p / (ROWB / 16);
+              dst[j] = k * a.a_stride + (int)tc::swizzled<ROWB>(r, p - k * (ROWB / 16));
+            }
+          }
+        }
+        if (e0 == 0) ok = lbnci::mbar_wait(&t.bar_a, 0u);  // the copy's zeros have landed
+        if (ok) {
+#pragma unroll
+          for (int j = 0; j < U; ++j)
+            if (dst[j] >= 0) *reinterpret_cast<uint4*>(sA + dst[j]) = v[j];
+        }
+      }
+      if (!ok) atomicOr(&t.fail, 1);
+      lbnci::fence_async_smem();  // these writes -> the tensor cores' reads
+      __syncwarp();
+      if (lane == 0) lbnci::mbar_arrive(&t.bar_p);
+    }
+    // drain: group g of four warps takes accumulators g, g + 2, ...
+    const bool done = lbnci::mbar_wait(&t.bar_d, 0u);
+    if (!done) atomicOr(&t.fail, 1);
+    tc::fence_after_sync();
+    if (done && *(volatile int*)&t.fail == 0) {
+      const int g = (warp - 2) >> 2, quad = warp & 3, l = quad * 32 + lane, gt = et & 127;
+      unsigned char* const stg = sm + g * (128 * BN * 2);
+      constexpr int NV = BN / 8;                      // 16-byte pieces of a pixel's output
+      auto piece = [](int r, int v) {                 // bank-conflict-free place of piece v of row r
+        return r * (BN * 2) + ((v ^ ((BN == 32 ? r >> 1 : r) & (NV < 8 ? NV - 1 : 7))) << 4);
+      };
+      const int nacc = a.nm * (a.up ? 4 : 1), Wo = a.W << a.up, Ho = a.H << a.up;
+      for (int q = g; q < nacc; q += 2) {
+        const int par = a.up ? q / a.nm : 0, m = q - par * a.nm;
+        auto out_row = [&](int r0) {  // output pixel of operand row r0, -1: none
+          int r, c;
+          if (a.linear) {
+            const int pos = m * a.mstart + r0;
+            r = pos / a.pitch;
+            c = pos - r * a.pitch;
+          } else {
+            r = r0 >> 3;
+            c = 8 * m + (r0 & 7);
+          }
+          const int yy = y0 + r, xx = x0 + c;
+          if (!(r < a.TH && c < a.TW && yy < a.H && xx < a.W)) return -1;
+          return a.up ? (b * Ho + 2 * yy + (par >> 1)) * Wo + 2 * xx + (par & 1) : (b * Ho + yy) * Wo + xx;
+        };
+        // this thread's pieces k = 0 .. NV - 1 of the tile: row (128 k + gt) / NV, piece gt % NV.
+        // The first four masks are in flight while the accumulator is drained.
+        constexpr int UB = NV < 4 ? NV : 4;
+        int orow[UB];
+        uint4 mk[UB];
+        auto fetch = [&](int k0) {
+#pragma unroll
+          for (int k = 0; k < UB; ++k) {
+            orow[k] = out_row(((k0 + k) * 128 + gt) / NV);
+            if (a.mask && orow[k] >= 0)
+              mk[k] = *reinterpret_cast<const uint4*>(a.mask + (size_t)orow[k] * a.ms + n0 + (gt % NV) * 8);
+          }
+        };
+        fetch(0);
+        const unsigned taddr = tmem + (unsigned)(q * BN) + ((unsigned)(quad * 32) << 16);
+#pragma unroll
+        for (int c0 = 0; c0 < BN; c0 += 16) {
+          float acc[16];
+          tc::tmem_ld16(taddr + (unsigned)c0, acc);
+          V8 o[2];
+#pragma unroll
+          for (int j = 0; j < 16; j += 2) {
+            float v0 = acc[j] + t.bias[c0 + j], v1 = acc[j + 1] + t.bias[c0 + j + 1];
+            if (a.relu) {
+              v0 = fmaxf(v0, 0.f);
+              v1 = fmaxf(v1, 0.f);
+            }
+            o[j >> 3].h[(j & 7) >> 1] = __floats2bfloat162_rn(v0, v1);
+          }
+          *reinterpret_cast<uint4*>(stg + piece(l, c0 / 8)) = o[0].u;
+          *reinterpret_cast<uint4*>(stg + piece(l, c0 / 8 + 1)) = o[1].u;
+        }
+        asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory");
+#pragma unroll
+        for (int k0 = 0; k0 < NV; k0 += UB) {
+          if (k0 > 0) fetch(k0);
+#pragma unroll
+          for (int k = 0; k < UB; ++k) {
+            if (orow[k] < 0) continue;
+            V8 o;
+            o.u = *reinterpret_cast<const uint4*>(stg + piece(((k0 + k) * 128 + gt) / NV, gt % NV));
+            if (a.mask) {
+              V8 w;
+              w.u = mk[k];
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const float2 mf = __bfloat1622float2(w.h[j]);
+                if (!(mf.x > 0.f)) o.h[j].x = __float2bfloat16_rn(0.f);
+                if (!(mf.y > 0.f)) o.h[j].y = __float2bfloat16_rn(0.f);
+              }
+            }
+            *reinterpret_cast<uint4*>(a.y + (size_t)orow[k] * a.ys + n0 + (gt % NV) * 8) = o.u;
+          }
+        }
+        asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory");
+      }
+    }
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  __syncwarp();
+  if (warp == 1) tc::tmem_dealloc(tmem, (unsigned)a.cols);
+  if (tid == 0 && t.fail) atomicOr(err, t.fail);
+}
+
+// ------------------------------------------------------------------ weight gradient
+// dw[o][t][c] = sum_p dy[p][o] xpad[p + t][c] as a GEMM with the pixels as K: both operands
+// are MN-major (channels contiguous), so the copied tiles are used as they arrive: x as the
+// tile and its ring of one pixel (CH = ROWB/2 channels, the chunk blockIdx.y), dy as the
+// tile (BN channels, block blockIdx.z). Shifting x by a tap is again only a start address,
+// and M = 128 holds several taps: the operand's blocks of CH channels lie `leading byte
+// offset` apart, which may be one pixel:
+//   CH = 32  3 accumulators, dy = -1, 0, 1; blocks dx = -1, 0, 1 (and 2, dropped)
+//   CH = 64  5 accumulators of two taps each, (0, 1), (2, 3), ... (8, dropped)
+//   up       the input is low-resolution and dy is copied per parity (py, px) of the output
+//            pixels; a parity meets only the shifts (py - 1, py) x (px - 1, px), so 4 x 2
+//            accumulators of two neighbouring shifts hold everything, and the reduction
+//            adds the parities' parts of each tap.
+// CTA (s, k, n) takes the tiles of split s and writes its partial sums; the epilogue warps
+// patch the periodic columns of x stage by stage, sum dy for the bias (chunk 0) and drain
+// the accumulators. Sums run over the same pixels as in conv3x3_wgrad_kernel with shorter
+// chains (more splits).
+struct WgradTma {
+  const bf16* x;
+  int xs, H, W;       // position grid: the image of x
+  int up;
+  int tiles_x, tiles_y, ntile, nsplit;
+  int TH, TW, pitch;
+  int x_bytes, d_bytes;  // shared memory of a stage: the x tile, one dy tile (four when up)
+  int nstage, cols, tail;
+  int Cin, Cout;
+  float* part;        // [nsplit][Cout][9 Cin], up: [nsplit][Cout][16 Cin]
+  float* bpart;       // [nsplit][Cout] or null
+};
+struct WgradMaps {
+  CUtensorMap x, dy[4];  // dy: all pixels, or the pixels of each parity 2 py + px
+};
+constexpr int kWgradMaxStage = 4;
+struct WgradTail {
+  unsigned long long bar_d, bar_full[kWgradMaxStage], bar_patched[kWgradMaxStage], bar_empty[kWgradMaxStage];
+  unsigned tmem;
+  int fail;
+};
+
+template <int BN, int ROWB>
+__global__ void __launch_bounds__(kConvThreads, 2)
+conv3x3_wgrad_tma_kernel(const __grid_constant__ WgradMaps maps, WgradTma a, int* err) {
+  constexpr int CH = ROWB / 2, DROW = BN * 2;
+  constexpr unsigned IDESC = tc::idesc_bf16(128, BN, true);
+  extern __shared__ __align__(1024) unsigned char sm[];
+  WgradTail& t = *reinterpret_cast<WgradTail*>(sm + a.tail);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int split = blockIdx.x, c0 = blockIdx.y * CH, n0 = blockIdx.z * BN;
+  const int t0 = (int)((long long)a.ntile * split / a.nsplit), t1 = (int)((long long)a.ntile * (split + 1) / a.nsplit);
+  const int nt = t1 - t0, ST = a.nstage, npar = a.up ? 4 : 1;
+  const int stage_bytes = a.x_bytes + npar * a.d_bytes;
+
+  if (tid == 0) {
+    lbnci::mbar_init(&t.bar_d, 2);
+    for (int s = 0; s < ST; ++s) {
+      lbnci::mbar_init(&t.bar_full[s], 1);
+      lbnci::mbar_init(&t.bar_patched[s], kConvEpiThreads / 32);
+      lbnci::mbar_init(&t.bar_empty[s], 1 + kConvEpiThreads / 32);
+    }
+    t.fail = (smem_u32(sm) & 1023u) ? 2 : 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) tc::tmem_alloc(&t.tmem, (unsigned)a.cols);
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const unsigned tmem = t.tmem;
+  const bool aligned = t.fail == 0;
+  auto origin = [&](int i, int& b, int& y0, int& x0) {
+    const int tt = t0 + i;
+    x0 = (tt % a.tiles_x) * a.TW;
+    y0 = ((tt / a.tiles_x) % a.tiles_y) * a.TH;
+    b = tt / (a.tiles_x * a.tiles_y);
+  };
+
+  if (!aligned) {
+  } else if (warp == 0) {
+    if (lane == 0) {  // copies
+      int issued = 0;
+      for (int i = 0; i < nt; ++i) {
+        const int s = i % ST, u = i / ST;
+        if (u > 0 && !lbnci::mbar_wait(&t.bar_empty[s], (unsigned)((u - 1) & 1))) {
+          atomicOr(&t.fail, 1);
+          break;
+        }
+        int b, y0, x0;
+        origin(i, b, y0, x0);
+        unsigned char* sx = sm + s * stage_bytes;
+        lbnci::mbar_expect_tx(&t.bar_full[s],
+                              (unsigned)(ROWB * (a.TW + 2) * (a.TH + 2) + npar * DROW * a.TW * a.TH));
+        lbnci::tma_load_4d(sx, &maps.x, c0, x0 - 1, y0 - 1, b, &t.bar_full[s]);
+        for (int q = 0; q < npar; ++q)
+          lbnci::tma_load_4d(sx + a.x_bytes + q * a.d_bytes, &maps.dy[q], n0, x0, y0, b, &t.bar_full[s]);
+        issued = i + 1;
+      }
+      for (int i = issued > ST ? issued - ST : 0; i < issued; ++i)
+        lbnci::mbar_wait(&t.bar_full[i % ST], (unsigned)((i / ST) & 1));
+    }
+  } else if (warp == 1) {  // MMAs: the whole warp, lane 0 issues
+    const unsigned leader = lane == 0;
+    bool bad = false;
+    const unsigned long long dB = tc::desc_base(DROW, 16u, 8u * DROW);
+    const unsigned hiA = (unsigned)(tc::desc_base(ROWB, 16u, 8u * ROWB) >> 32), hiB = (unsigned)(dB >> 32);
+    const unsigned base = smem_u32(sm) >> 4;
+    const int kx = a.TW / 16;
+    // A descriptors of the accumulators relative to the pixel's own position: start (the
+    // shift) and leading byte offset (to the next block of channels), lower half
+    constexpr int NA = ROWB == 64 ? 3 : 8;
+    unsigned rel[NA];
+    if constexpr (ROWB == 64) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) rel[j] = (unsigned)((j * a.pitch * 64) >> 4) + (4u << 16);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        if (a.up) {  // parity j >> 1, shift row j & 1
+          const int q = j >> 1;
+          rel[j] = (unsigned)((((q >> 1) + (j & 1)) * a.pitch + (q & 1)) * 8) + (8u << 16);
+        } else {  // taps 2j and 2j + 1
+          const int o0 = (2 * j / 3) * a.pitch + (2 * j) % 3, o1 = ((2 * j + 1) / 3) * a.pitch + (2 * j + 1) % 3;
+          rel[j] = (unsigned)(o0 * 8) + ((unsigned)((j < 4 ? o1 - o0 : 1) * 8) << 16);
+        }
+      }
+    }
+    const unsigned dpar = (unsigned)(a.d_bytes >> 4);
+    unsigned ph = 0u;
+    int s = 0;
+    auto block = [&](unsigned ua, unsigned ub, auto ACC) {  // the MMAs of K = 16 pixels of a row
+      constexpr bool acc = decltype(ACC)::value;
+      if (ROWB == 128 && a.up) {
+#pragma unroll
+        for (int j = 0; j < NA; ++j)
+          tc::mma_bf16<acc>(tmem + j * BN, tc::desc64(hiA, ua + rel[j]), tc::desc64(hiB, ub + (unsigned)(j >> 1) * dpar),
+                            IDESC, leader);
+      } else {
+#pragma unroll
+        for (int j = 0; j < (ROWB == 64 ? 3 : 5); ++j)
+          tc::mma_bf16<acc>(tmem + j * BN, tc::desc64(hiA, ua + rel[j]), tc::desc64(hiB, ub), IDESC, leader);
+      }
+    };
+    for (int i = 0; i < nt; ++i) {
+      bad = __any_sync(~0u, !lbnci::mbar_wait(&t.bar_full[s], ph) || !lbnci::mbar_wait(&t.bar_patched[s], ph));
+      if (bad) break;
+      tc::fence_after_sync();
+      const unsigned ux = base + (unsigned)((s * stage_bytes) >> 4);
+      const unsigned ud = ux + (unsigned)(a.x_bytes >> 4) + (unsigned)dB;
+      for (int r = 0; r < a.TH; ++r) {
+        unsigned ua = ux + (unsigned)((r * a.pitch * ROWB) >> 4), ub = ud + (unsigned)((r * a.TW * DROW) >> 4);
+        for (int c = 0; c < kx; ++c) {
+          if (i == 0 && r == 0 && c == 0) block(ua, ub, std::false_type{});
+          else block(ua, ub, std::true_type{});
+          ua += ROWB;  // 16 pixels of ROWB bytes, in 16-byte units
+          ub += DROW;
+        }
+      }
+      tc::mma_commit(&t.bar_empty[s], leader);
+      if (++s == ST) {
+        s = 0;
+        ph ^= 1u;
+      }
+    }
+    if (lane == 0 && bad) atomicOr(&t.fail, 1);
+    tc::mma_commit(&t.bar_d, leader);
+    if (lane == 0) lbnci::mbar_arrive(&t.bar_d);
+  } else {
+    const int et = tid - 64;
+    constexpr int VX = ROWB / 16, VD = DROW / 16, DR = kConvEpiThreads / VD;
+    const bool do_bias = a.bpart != nullptr && blockIdx.y == 0;
+    float bs[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    bool ok = true;
+    for (int i = 0; i < nt && ok; ++i) {
+      const int s = i % ST;
+      const unsigned ph = (unsigned)((i / ST) & 1);
+      int b, y0, x0;
+      origin(i, b, y0, x0);
+      unsigned char* sx = sm + s * stage_bytes;
+      const int left = x0 == 0 ? 1 : 0, right = x0 + a.TW >= a.W ? 1 : 0;
+      const int ncol = left + right, count = ncol * (a.TH + 2) * VX;
+      constexpr int U = 2;
+      uint4 v[U];
+      int dst[U];
+      for (int e0 = 0; e0 < count || e0 == 0; e0 += U * kConvEpiThreads) {
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+          const int e = e0 + j * kConvEpiThreads + et;
+          dst[j] = -1;
+          if (e < count) {
+            const int px = e / VX, p = e - px * VX;
+            const int row = px / ncol, col = px - row * ncol;
+            const int yy = y0 - 1 + row;
+            if (yy >= 0 && yy < a.H) {
+              const bool lft = left && col == 0;
+              v[j] = *reinterpret_cast<const uint4*>(a.x + ((size_t)(b * a.H + yy) * a.W + (lft ? a.W - 1 : 0)) * a.xs +
+                                                     c0 + p * 8);
+              dst[j] = (int)tc::swizzled<ROWB>(row * a.pitch + (lft ? 0 : a.W - x0 + 1), p);
+            }
+          }
+        }
+        if (e0 == 0) ok = lbnci::mbar_wait(&t.bar_full[s], ph);
+        if (!ok) break;
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+          if (dst[j] >= 0) *reinterpret_cast<uint4*>(sx + dst[j]) = v[j];
+      }
+      lbnci::fence_async_smem();
+      __syncwarp();
+      if (lane == 0) lbnci::mbar_arrive(&t.bar_patched[s]);
+      if (do_bias && ok)
+        for (int q = 0; q < npar; ++q)
+          for (int r = et / VD; r < a.TH * a.TW; r += DR) {
+            V8 d;
+            d.u = *reinterpret_cast<const uint4*>(sx + a.x_bytes + q * a.d_bytes + tc::swizzled<DROW>(r, et % VD));
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float2 f = __bfloat1622float2(d.h[j]);
+              bs[2 * j] += f.x;
+              bs[2 * j + 1] += f.y;
+            }
+          }
+      __syncwarp();
+      if (lane == 0) lbnci::mbar_arrive(&t.bar_empty[s]);
+    }
+    if (!ok) atomicOr(&t.fail, 1);
+    if (!lbnci::mbar_wait(&t.bar_d, 0u)) {
+      ok = false;
+      atomicOr(&t.fail, 1);
+    }
+    tc::fence_after_sync();
+    asm volatile("bar.sync 1, 256;" ::: "memory");  // every epilogue warp is past the stages
+    if (ok && *(volatile int*)&t.fail == 0) {
+      if (do_bias) {  // thread sums, added in thread order
+        float* red = reinterpret_cast<float*>(sm);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) red[(et / VD) * BN + (et % VD) * 8 + j] = bs[j];
+      }
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      if (do_bias && et < BN) {
+        const float* red = reinterpret_cast<const float*>(sm);
+        float v = 0.f;
+        for (int r = 0; r < DR; ++r) v += red[r * BN + et];
+        a.bpart[(size_t)split * a.Cout + n0 + et] = v;
+      }
+      const int g = (warp - 2) >> 2, quad = warp & 3, l = quad * 32 + lane;
+      const int blk = l / CH, ci = c0 + l % CH;  // block of the operand's M rows, input channel
+      const int nacc = a.up ? 8 : (ROWB == 64 ? 3 : 5), nk = a.up ? 16 : 9;
+      for (int q = g; q < nacc; q += 2) {
+        int k = -1;  // row block of the partial sums: the tap, or (parity, shift)
+        if (a.up) k = blk < 2 ? 2 * q + blk : -1;
+        else if (ROWB == 64) k = blk < 3 ? 3 * q + blk : -1;
+        else k = 2 * q + blk < 9 ? 2 * q + blk : -1;
+        float* out = a.part + ((size_t)split * a.Cout + n0) * nk * a.Cin + (size_t)(k < 0 ? 0 : k) * a.Cin + ci;
+        const unsigned taddr = tmem + (unsigned)(q * BN) + ((unsigned)(quad * 32) << 16);
+#pragma unroll
+        for (int j0 = 0; j0 < BN; j0 += 16) {
+          float acc[16];
+          tc::tmem_ld16(taddr + (unsigned)j0, acc);
+          if (k >= 0) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) out[(size_t)(j0 + j) * nk * a.Cin] = acc[j];
+          }
+        }
+      }
+    }
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  __syncwarp();
+  if (warp == 1) tc::tmem_dealloc(tmem, (unsigned)a.cols);
+  if (tid == 0 && t.fail) atomicOr(err, t.fail);
+}
+
+// Sum the split partials: dw[o][t][c] for c < cin_true (master layout [Cout][3][3][cin_true])
+// and db[o] (the last blocks). A block takes 256 / S groups of four consecutive values, S
+// threads to each (thread k the splits k, k + S, ...; their sums added in thread order), S
+// so large that the grid fills the multiprocessors: whole lines are read, every load of a
+// thread is independent. up: a tap's sum also runs over the four parities, each at the
+// shift floor((parity + tap)/2) the tap has there.
+__global__ void __launch_bounds__(256) wgrad_reduce_tma_kernel(const float* __restrict__ part,
+                                                               const float* __restrict__ bpart, int nsplit, int Cout,
+                                                               int Cin, int cin_true, int up, int S, int wblocks,
+                                                               float* __restrict__ dw, float* __restrict__ db) {
+  __shared__ float4 s[256];
+  if ((int)blockIdx.x >= wblocks) {  // 32 output channels of the bias, eight threads to each
+    float* sb = reinterpret_cast<float*>(s);
+    const int o = ((int)blockIdx.x - wblocks) * 32 + (threadIdx.x & 31), share = threadIdx.x >> 5;
+    float v = 0.f;
+    if (o < Cout) {
+#pragma unroll 4
+      for (int z = share; z < nsplit; z += 8) v += bpart[(size_t)z * Cout + o];
+    }
+    sb[threadIdx.x] = v;
+    __syncthreads();
+    if (share == 0 && o < Cout) {
+      float r = 0.f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) r += sb[k * 32 + threadIdx.x];
+      db[o] = r;
+    }
+    return;
+  }
+  const int V = 256 / S, vec = threadIdx.x % V, share = threadIdx.x / V;
+  const int nk = up ? 16 : 9, c4 = Cin / 4, n4 = Cout * 9 * c4;
+  const int i = blockIdx.x * V + vec;
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  int c = 0, tap = 0, o = 0;
+  if (i < n4) {
+    c = (i % c4) * 4;
+    const int r = i / c4;
+    tap = r % 9;
+    o = r / 9;
+    const size_t stride = (size_t)Cout * nk * Cin;
+    const int dy = tap / 3 - 1, dx = tap % 3 - 1;
+    for (int q = 0; q < (up ? 4 : 1); ++q) {
+      const int py = q >> 1, px = q & 1;
+      // shift row py - 1 + sy, column px - 1 + sx
+      const int k = up ? 4 * q + 2 * (((py + dy) >> 1) - py + 1) + (((px + dx) >> 1) - px + 1) : tap;
+      const float* p = part + ((size_t)o * nk + k) * Cin + c;
+#pragma unroll 4
+      for (int z = share; z < nsplit; z += S) {
+        const float4 w = *reinterpret_cast<const float4*>(p + (size_t)z * stride);
+        v.x += w.x;
+        v.y += w.y;
+        v.z += w.z;
+        v.w += w.w;
+      }
+    }
+  }
+  s[threadIdx.x] = v;
+  __syncthreads();
+  if (share == 0 && i < n4) {
+    for (int k = 1; k < S; ++k) {
+      const float4 w = s[k * V + vec];
+      v.x += w.x;
+      v.y += w.y;
+      v.z += w.z;
+      v.w += w.w;
+    }
+    float* out = dw + ((size_t)o * 9 + tap) * cin_true + c;
+    if (c < cin_true) out[0] = v.x;
+    if (c + 1 < cin_true) out[1] = v.y;
+    if (c + 2 < cin_true) out[2] = v.z;
+    if (c + 3 < cin_true) out[3] = v.w;
+  }
+}
+
+}  // namespace lbu

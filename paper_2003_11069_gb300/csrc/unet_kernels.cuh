@@ -545,67 +545,97 @@ __global__ void mse_kernel(const float* __restrict__ y, const float* __restrict_
   if (threadIdx.x == 0) partial[blockIdx.x] = red[0];
 }
 
-__global__ void sum_partials_kernel(const double* __restrict__ partial, int n, double scale, double* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0.0;
-    for (int i = 0; i < n; ++i) s += partial[i];
-    *out = s * scale;
+// One block: thread t adds partials t, t + 256, ..., then a fixed tree.
+__global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restrict__ partial, int n, double scale,
+                                                           double* __restrict__ out) {
+  __shared__ double s[256];
+  double v = 0.0;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n; i += 256) v += partial[i];
+  s[threadIdx.x] = v;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
+    __syncthreads();
   }
+  if (threadIdx.x == 0) *out = s[0] * scale;
 }
 
 // Head backward. dx[p][c] = bf16(sum_j dy[p][j] wh[j][c]) where x[p][c] > 0, else 0;
 // per block of kHeadPix pixels the partial sums of dW[j][c] = sum_p dy[p][j] x[p][c] and
-// db[j] = sum_p dy[p][j] go to part[block][nout (C + 1)].
-constexpr int kHeadPix = 1024;
-__global__ void head_bwd_kernel(const bf16* __restrict__ x, int C, const bf16* __restrict__ wh, int nout, int P,
-                                const float* __restrict__ dy, bf16* __restrict__ dx, float* __restrict__ part) {
-  __shared__ float sw[kMaxOut * kMaxHeadIn];
-  for (int i = threadIdx.x; i < nout * C; i += blockDim.x) sw[i] = __bfloat162float(wh[i]);
-  __syncthreads();
+// db[j] = sum_p dy[p][j] go to part[block][nout (C + 1)]. A warp takes every eighth pixel of
+// the block, a lane one channel (of each 32): rows of x and dx are whole lines, dy[p] is
+// one broadcast, the sums stay in registers until the block's eight warps are added in
+// order. (32 images of 64 x 256, 32 channels: 74 us, 90 us with one thread per output
+// summing the block's pixels.)
+constexpr int kHeadPix = 512;
+__global__ void __launch_bounds__(256) head_bwd_kernel(const bf16* __restrict__ x, int C, const bf16* __restrict__ wh,
+                                                       int nout, int P, const float* __restrict__ dy,
+                                                       bf16* __restrict__ dx, float* __restrict__ part) {
+  __shared__ float red[8][kMaxOut + 1][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int p0 = blockIdx.x * kHeadPix, p1 = min(p0 + kHeadPix, P);
-  for (int p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-    float d[kMaxOut];
-    for (int j = 0; j < nout; ++j) d[j] = dy[(size_t)p * nout + j];
-    for (int c0 = 0; c0 < C; c0 += 8) {
-      V8 v, o;
-      v.u = *reinterpret_cast<const uint4*>(x + (size_t)p * C + c0);
+  float* out = part + (size_t)blockIdx.x * nout * (C + 1);
+  for (int c0 = 0; c0 < C; c0 += 32) {
+    float w[kMaxOut], sw[kMaxOut], sb[kMaxOut];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 f = __bfloat1622float2(v.h[e]);
-        float s0 = 0.f, s1 = 0.f;
-        for (int j = 0; j < nout; ++j) {
-          s0 = fmaf(d[j], sw[j * C + c0 + 2 * e], s0);
-          s1 = fmaf(d[j], sw[j * C + c0 + 2 * e + 1], s1);
+    for (int j = 0; j < kMaxOut; ++j) {
+      w[j] = j < nout ? __bfloat162float(wh[j * C + c0 + lane]) : 0.f;
+      sw[j] = 0.f;
+      sb[j] = 0.f;
+    }
+#pragma unroll 4
+    for (int p = p0 + warp; p < p1; p += 8) {
+      const float xv = __bfloat162float(x[(size_t)p * C + c0 + lane]);
+      float s = 0.f;
+#pragma unroll
+      for (int j = 0; j < kMaxOut; ++j)
+        if (j < nout) {
+          const float d = dy[(size_t)p * nout + j];
+          s = fmaf(d, w[j], s);
+          sw[j] = fmaf(d, xv, sw[j]);
+          sb[j] += d;
         }
-        o.h[e] = __floats2bfloat162_rn(f.x > 0.f ? s0 : 0.f, f.y > 0.f ? s1 : 0.f);
+      dx[(size_t)p * C + c0 + lane] = __float2bfloat16_rn(xv > 0.f ? s : 0.f);
+    }
+#pragma unroll
+    for (int j = 0; j < kMaxOut; ++j)
+      if (j < nout) {
+        red[warp][j][lane] = sw[j];
+        if (lane == 0) red[warp][j][32] = sb[j];
       }
-      *reinterpret_cast<uint4*>(dx + (size_t)p * C + c0) = o.u;
+    __syncthreads();
+    for (int o = threadIdx.x; o < nout * 33; o += 256) {
+      const int j = o / 33, l = o % 33;
+      float v = 0.f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v += red[k][j][l];
+      if (l < 32) out[j * (C + 1) + c0 + l] = v;
+      else if (c0 == 0) out[j * (C + 1) + C] = v;
     }
-  }
-  const int nw = nout * (C + 1);
-  for (int o = threadIdx.x; o < nw; o += blockDim.x) {
-    const int j = o / (C + 1), c = o % (C + 1);
-    float s = 0.f;
-    for (int p = p0; p < p1; ++p) {
-      const float xv = c < C ? __bfloat162float(x[(size_t)p * C + c]) : 1.f;
-      s = fmaf(dy[(size_t)p * nout + j], xv, s);
-    }
-    part[(size_t)blockIdx.x * nw + o] = s;
+    __syncthreads();
   }
 }
 
-// Sum head partials in block order into the master gradient: dW [nout][C] then db [nout].
-__global__ void head_reduce_kernel(const float* __restrict__ part, int nblk, int nout, int C, float* __restrict__ dw,
-                                   float* __restrict__ db) {
-  const int nw = nout * (C + 1);
-  for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < nw; o += gridDim.x * blockDim.x) {
-    float s = 0.f;
-    for (int z = 0; z < nblk; ++z) s += part[(size_t)z * nw + o];
+// Sum head partials into the master gradient, one block per value (thread t adds blocks t, t
+// + 128, ..., then a fixed tree): dW [nout][C] then db [nout].
+__global__ void __launch_bounds__(128) head_reduce_kernel(const float* __restrict__ part, int nblk, int nout, int C,
+                                                          float* __restrict__ dw, float* __restrict__ db) {
+  __shared__ float s[128];
+  const int nw = nout * (C + 1), o = blockIdx.x;
+  float v = 0.f;
+#pragma unroll 4
+  for (int z = threadIdx.x; z < nblk; z += 128) v += part[(size_t)z * nw + o];
+  s[threadIdx.x] = v;
+  __syncthreads();
+  for (int h = 64; h > 0; h >>= 1) {
+    if (threadIdx.x < h) s[threadIdx.x] += s[threadIdx.x + h];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) {
     const int j = o / (C + 1), c = o % (C + 1);
-    if (c < C)
-      dw[j * C + c] = s;
-    else
-      db[j] = s;
+    if (c < C) dw[j * C + c] = s[0];
+    else db[j] = s[0];
   }
 }
 
