@@ -133,7 +133,7 @@ size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 // kErrSlot, the kernels' error word (an int), in slot kErrSlot + 1 the two tile
 // counters of the TMA step kernel (ints), and in slot kErrSlot + 2 the two dither-seed
 // words of the FP16-deviation stores (StepT::seedw).
-constexpr int kErrSlot = 12;
+static_assert(lbnci::kErrSlot == 12, "result area");
 
 struct Layout {
   size_t fa, fb, psi, partials, result, carry, ring, ghost, ng, hit, rho1, sites;
@@ -293,20 +293,28 @@ lb_status run_fields(lb_sim* s, const FieldOut& outs, size_t staged = 0) {
   const size_t need = s->L->fields_scratch((size_t)s->p.N);
   void* scratch = need + staged <= state ? (void*)((unsigned char*)s->fb + (state - need)) : nullptr;
   long long rows = s->nblocks;
+  if (scratch) {  // the fields pass adds its own sums and writes them to the pinned result
+    fo.out = s->host_result;
+    fo.ticket = (unsigned*)(s->result + kErrSlot + 3);
+    fo.err = s->errflag;
+    fo.ens = s->ens_flag;
+  }
   cudaError_t e = s->totals_state
                       ? stream3d_form_fields(s->fa, s->psi, s->p, fo, s->stream, &nk, scratch, s->nblocks, &rows)
                       : s->L->fields(s->fa, s->psi, s->p, fo, s->stream, &nk, scratch, s->nblocks, &rows);
-  s->launches += nk + 1;
+  s->launches += nk + (scratch ? 0 : 1);
   if (e != cudaSuccess) return cuda_fail(s, e, "fields launch");
-  e = reduce_partials(s->partials, rows, s->result, s->stream);
-  if (e != cudaSuccess) return cuda_fail(s, e, "reduce launch");
-  e = cudaMemcpyAsync(s->host_result, s->result, 16 * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
-  if (e != cudaSuccess) return cuda_fail(s, e, "result copy");
+  if (!scratch) {
+    e = reduce_partials(s->partials, rows, s->result, s->stream);
+    if (e != cudaSuccess) return cuda_fail(s, e, "reduce launch");
+    e = cudaMemcpyAsync(s->host_result, s->result, 16 * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
+    if (e != cudaSuccess) return cuda_fail(s, e, "result copy");
+  }
   e = cudaStreamSynchronize(s->stream);
   if (e != cudaSuccess) return cuda_fail(s, e, "stream synchronize");
   int flag = 0;
   std::memcpy(&flag, &s->host_result[kErrSlot], sizeof(flag));
-  if (s->ens_flag) {  // the batched step reports into its ensemble's word
+  if (s->ens_flag && !scratch) {  // the batched step reports into its ensemble's word
     int ef = 0;
     e = cudaMemcpy(&ef, s->ens_flag, sizeof(ef), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(s, e, "ensemble flag copy");
@@ -537,7 +545,8 @@ lb_status lb_fields(lb_sim* s, double* rho1, double* rho2, double* psi, double* 
   if (!s) return fail(nullptr, LB_EINVAL, "sim is NULL");
   const long long N = s->p.N;
   if (on_device) {
-    FieldOut fo{rho1, rho2, psi, grad, frep, hit, u, nullptr};
+    FieldOut fo{};
+    fo.rho1 = rho1; fo.rho2 = rho2; fo.psi = psi; fo.grad = grad; fo.frep = frep; fo.hit = hit; fo.u = u;
     lb_status st = run_fields(s, fo);
     if (st != LB_OK) return st;
     return s->host_result[9] > 0 ? fail(s, LB_ENUMERIC, "non-finite or non-positive density at %.0f sites", s->host_result[9]) : LB_OK;

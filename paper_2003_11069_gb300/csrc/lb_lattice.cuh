@@ -91,8 +91,16 @@ struct FieldOut {
   int* hit;
   double* u;     // [3][N]
   double* partials;  // [blocks][kRedSlots] reductions
+  // where the reductions end (or null: the caller adds the partials): kRedSlots values, then,
+  // in slot kErrSlot, the error words err and ens (either may be null) or'ed into an int;
+  // ticket: a device counter, zero between launches
+  double* out;
+  unsigned* ticket;
+  const int* err;
+  const int* ens;
 };
 
+constexpr int kErrSlot = 12;  // of a result area of 16 doubles
 constexpr int kRedSlots = 10;  // mass1, mass2, P_x, P_y, P_z, flux, flux_disp, n_if, n_nci, n_bad
 
 // Thread-block tile of the tiled (fields and 3D step) kernels.

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <utility>
 
 #include "lb_lattice.cuh"
 
@@ -35,6 +36,33 @@ cudaError_t allow_smem(K kernel, size_t bytes, SmemAllowance& a) {
   }
   return e;
 }
+
+// Programmatic dependent launch of a chain of kernels on one stream: a launch may be
+// scheduled, and its blocks may start, as soon as every block of the kernel before it has
+// started (pdl_begin) or ended. pdl_begin waits for that kernel's completion (its writes
+// visible) before anything of the chain's memory is touched, so results and order are those
+// of plain launches; what overlaps is the launch latency and the last blocks' tail. Every
+// kernel launched this way begins with pdl_begin (which does nothing after a plain launch).
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, std::forward<A>(args)...);
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+#endif
 
 // Everything a launcher needs, in FP64; each instantiation converts it to its own
 // arithmetic type once per call.

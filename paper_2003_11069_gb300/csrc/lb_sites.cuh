@@ -77,6 +77,7 @@ __global__ void __launch_bounds__(256) site_moments_kernel(typename ST::Reader f
                                                            SiteScratch<typename ST::Compute> sc,
                                                            StepT<typename ST::Compute> p) {
   using T = typename ST::Compute;
+  if (WITHJ) pdl_begin();
   const SiteIdx s = site_of(p);
   if (s.x >= p.nx || s.y >= p.ny) return;
   T fin[2][Lattice<LAT>::Q];
@@ -155,6 +156,7 @@ __device__ __forceinline__ T unit_site(const T g[3], T n[3]) {
 template <int LAT, typename T>
 __global__ void __launch_bounds__(256) site_normals_kernel(const T* __restrict__ psi, Quad<T>* __restrict__ ng,
                                                            StepT<T> p) {
+  pdl_begin();
   const SiteIdx s = site_of(p);
   if (s.x >= p.nx || s.y >= p.ny) return;
   T g[3], n[3];
@@ -191,6 +193,7 @@ __global__ void __launch_bounds__(256) normals3d_kernel(const T* __restrict__ ps
                                                         StepT<T> p) {
   constexpr int RX = 34, RXY = RX * 10, PER = (RXY + 255) / 256;
   __shared__ T s_psi[4 * RXY];
+  pdl_begin();
   const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 8, z0 = blockIdx.z * kN3Z;
   const int nx = p.nx, ny = p.ny, nz = p.nz;
   const int tid = threadIdx.x + 32 * threadIdx.y;
@@ -252,7 +255,8 @@ __global__ void __launch_bounds__(256) normals3d_kernel(const T* __restrict__ ps
 template <typename T, bool FIELDS = false>
 cudaError_t launch_normals3d(const T* psi, Quad<T>* ng, const StepT<T>& p, cudaStream_t s) {
   const dim3 grid((unsigned)((p.nx + 31) / 32), (unsigned)((p.ny + 7) / 8), (unsigned)((p.nz + kN3Z - 1) / kN3Z));
-  normals3d_kernel<T, FIELDS><<<grid, dim3(32, 8), 0, s>>>(psi, ng, p);
+  if constexpr (FIELDS) return launch_pdl(normals3d_kernel<T, true>, grid, dim3(32, 8), 0, s, psi, ng, p);
+  normals3d_kernel<T, false><<<grid, dim3(32, 8), 0, s>>>(psi, ng, p);
   return cudaGetLastError();
 }
 
@@ -324,6 +328,7 @@ template <int LAT, typename T>
 __global__ void __launch_bounds__(kFieldThreads) site_fields_kernel(const T* __restrict__ psi, SiteScratch<T> sc,
                                                                     StepT<T> p, FieldOut fo) {
   constexpr int D = Lattice<LAT>::D;
+  pdl_begin();
   const unsigned N = (unsigned)p.N, nx = (unsigned)p.nx, ny = (unsigned)p.ny;
   double m1 = 0.0, m2 = 0.0, P[3] = {0.0, 0.0, 0.0}, qd = 0.0;
   unsigned nif = 0, nnci = 0, nbad = 0;
@@ -414,6 +419,34 @@ __global__ void __launch_bounds__(kFieldThreads) site_fields_kernel(const T* __r
     }
     fo.partials[(size_t)blockIdx.x * kRedSlots + q] = v;
   }
+  if (!fo.out) return;
+  // the block that draws the last ticket adds the blocks' sums: thread t the elements t, t +
+  // 250, ... of the flat array (all of slot t mod 10), then each slot's 25 sums in order
+  static_assert(kRedSlots == 10 && kFieldThreads >= 250, "25 threads to each slot");
+  __shared__ unsigned last;
+  __shared__ double fin[250];
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicInc(fo.ticket, gridDim.x - 1) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (threadIdx.x < 250) {
+    const unsigned n = gridDim.x * kRedSlots;
+    double v = 0.0;
+#pragma unroll 8
+    for (unsigned e = threadIdx.x; e < n; e += 250) v += __ldcg(fo.partials + e);
+    fin[threadIdx.x] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < kRedSlots) {
+    double v = 0.0;
+#pragma unroll
+    for (int k = 0; k < 25; ++k) v += fin[threadIdx.x + k * kRedSlots];
+    fo.out[threadIdx.x] = v;
+  }
+  if (threadIdx.x == 32)
+    *reinterpret_cast<int*>(fo.out + kErrSlot) = (fo.err ? *fo.err : 0) | (fo.ens ? *fo.ens : 0);
 }
 
 // ------------------------------------------------------------------ FP64 collision
@@ -550,8 +583,7 @@ inline unsigned site_field_blocks(const HostParams& h, long long rows) {
 template <int LAT, typename T>
 cudaError_t launch_site_normals(const T* psi, Quad<T>* ng, const HostParams& h, const StepT<T>& p, cudaStream_t s) {
   const dim3 b = site_block<T>(h);
-  site_normals_kernel<LAT, T><<<site_grid(h, b), b, 0, s>>>(psi, ng, p);
-  return cudaGetLastError();
+  return launch_pdl(site_normals_kernel<LAT, T>, site_grid(h, b), b, 0, s, psi, ng, p);
 }
 
 // The FP64 step with Guo forcing: moments, normals, collision.
@@ -569,7 +601,10 @@ cudaError_t site_step64(const void* fa, void* fb, double* psi, void* scratch, co
   return cudaGetLastError();
 }
 
-// The observables and fields of a state: three passes. ng is filled by `normals` (the
+// The observables and fields of a state: three passes, launched programmatically: on a small
+// lattice the launches are most of the time. (The step's passes are launched plainly: blocks
+// of the next pass that wait on an SM unbalance the FP64 pipes of a 128 x 128 lattice, 46
+// us per step instead of 29, and cost the 512 x 128 x 128 FP16-dev duct 4%.) ng is filled by `normals` (the
 // lattice's own normals pass). rows: partial sums the caller has room for; *used: written.
 template <int LAT, typename ST, typename Normals>
 cudaError_t site_fields(typename ST::Reader f, typename ST::Compute* psi, void* scratch, const HostParams& h,
@@ -578,15 +613,13 @@ cudaError_t site_fields(typename ST::Reader f, typename ST::Compute* psi, void* 
   using T = typename ST::Compute;
   const SiteScratch<T> sc = site_scratch<LAT, T>(scratch, (size_t)p.N);
   const dim3 b = site_block<T>(h);
-  site_moments_kernel<LAT, ST, true><<<site_grid(h, b), b, 0, s>>>(f, psi, sc, p);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(site_moments_kernel<LAT, ST, true>, site_grid(h, b), b, 0, s, f, psi, sc, p);
   if (e == cudaSuccess) e = normals(psi, sc.ng);
   if (e != cudaSuccess) return e;
   const unsigned nb = site_field_blocks(h, rows);
-  site_fields_kernel<LAT, T><<<nb, kFieldThreads, 0, s>>>(psi, sc, p, fo);
   *used = nb;
   *nk = 3;
-  return cudaGetLastError();
+  return launch_pdl(site_fields_kernel<LAT, T>, dim3(nb), dim3(kFieldThreads), 0, s, (const T*)psi, sc, p, fo);
 }
 
 }  // namespace lbnci
