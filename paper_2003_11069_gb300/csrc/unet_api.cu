@@ -178,11 +178,13 @@ size_t wgrad_work(int B, int H, int W, int cin, int cout) {
 
 thread_local std::string g_err;
 
-// One launch of conv3x3_tma_kernel: tensor maps, tile and grid of a convolution's operands.
+// One launch of conv3x3_tma_kernel or, rows, conv3x3_rows_kernel: tensor maps, tile and grid
+// of a convolution's operands.
 struct ConvPlan {
-  bool ok = false;
+  bool ok = false, rows = false;
   CUtensorMap mx, mw;
   lbu::ConvTma a;
+  lbu::ConvRows r;
   dim3 grid;
   int smem = 0, BN = 0, rowb = 0;
 };
@@ -277,11 +279,11 @@ bool encode_tiled(CUtensorMap* m, const void* base, int rank, const cuuint64_t* 
 // when up): among tiles of 16 rows x 8 k columns (every operand row a pixel) and tiles of
 // TH rows x min(W, 126) columns (rows of the operand run through the pitched tile), those
 // whose operands fit, the one with the smallest estimated time. The estimate counts, per
-// multiprocessor, waves of resident CTAs, each wave a fixed latency (copy, first MMA,
-// drain: about 4,000 cycles) plus the CTAs' MMAs (M = 128: 32 cycles whatever N up to 128,
-// reading A from shared memory sets the rate) or their copies (about 50 bytes a cycle),
-// whichever is longer.
-bool plan_tile(int B, int H, int W, int cin, int cout, int up, ConvPlan* p) {
+// multiprocessor, waves of resident CTAs; a wave takes the first copy (about 2,000 cycles),
+// the MMAs (32 + N/4 cycles each, the operands' bytes) or the copies (about 50 bytes a
+// cycle), whichever is longer, and the drain (30 cycles a column of a group's accumulators,
+// 50 with a mask); two CTAs overlap one's drain with the other's MMAs.
+bool plan_tile(int B, int H, int W, int cin, int cout, int up, bool mask, ConvPlan* p) {
   p->rowb = cin % 64 == 0 ? 128 : 64;
   const int nchunk = cin / (p->rowb / 2), npar = up ? 4 : 1, ni = 9 * nchunk;
   double best = 1e30;
@@ -308,10 +310,12 @@ bool plan_tile(int B, int H, int W, int cin, int cout, int up, ConvPlan* p) {
     const int tiles_x = (W + TW - 1) / TW, tiles_y = (H + TH - 1) / TH;
     const double ctas = (double)B * tiles_x * tiles_y * (cout / BN);
     const double waves = std::ceil(ctas / (152.0 * occ));
-    const double mma = (double)nm * npar * ni * (p->rowb / 32) * 32;
+    const double mma = (double)nm * npar * ni * (p->rowb / 32) * (32 + BN / 4);
     const double copy = ((double)nchunk * (TH + 2) * pitch * p->rowb + (double)ni * bstage +
                          (double)TH * TW * npar * BN * 2) / 50.0;
-    const double cost = waves * (4000.0 + occ * std::max(mma, copy));
+    const double drain = ((nm * npar + 1) / 2) * (mask ? 50.0 : 30.0) * BN;
+    const double cost = waves * (2000.0 + (occ > 1 ? std::max(drain + std::max(mma, copy), occ * std::max(mma, copy))
+                                                    : drain + std::max(mma, copy)));
     if (cost >= best) return;
     best = cost;
     p->BN = BN;
@@ -342,6 +346,64 @@ bool plan_tile(int B, int H, int W, int cin, int cout, int up, ConvPlan* p) {
   return best < 1e30;
 }
 
+// Strips of conv3x3_rows_kernel over B images of H x W positions: wide images (at most a third
+// of the 128-column strips beyond the image) whose weights for BN output channels and three
+// input rows fit in shared memory. Two CTAs per multiprocessor where they fit, and the number
+// of output rows per CTA with the smallest estimated time: waves of CTAs, each the longer of
+// its MMAs (32 + N/4 cycles, N/2 above N = 128), its copies and its drain, and about 4,000
+// cycles to start and end.
+bool plan_rows(int B, int H, int W, int cin, int cout, int up, bool mask, ConvPlan* p) {
+  const int tiles_x = (W + 127) / 128;
+  if (W < 64 || 4 * W < 3 * tiles_x * 128) return false;
+  const int rowb = cin % 64 == 0 ? 128 : 64, nchunk = cin / (rowb / 2), npx = up ? 2 : 1, Ho = H << up;
+  const int cstride = (130 * rowb + 1023) / 1024 * 1024;
+  double best = 1e30;
+  for (int BN = cout % 64 == 0 ? 64 : 32; BN >= 32; BN /= 2)
+    for (int occ = 2; occ >= 1; --occ) {
+      const int cols = 512 / occ;
+      const int R = std::min(lbu::kRowsMaxSlot, cols / (npx * BN)) & ~1;
+      if (R < 4) continue;
+      const int weights = 9 * nchunk * BN * rowb, staging = 2 * 128 * BN * 2;
+      const int room = kSmemSm / occ - 1024 - (int)sizeof(lbu::RowsTail) - 16 - weights - staging;
+      const int nrow = std::min(lbu::kRowsMaxStage, room / (nchunk * cstride));
+      if (nrow < 3) continue;
+      const double n3 = 3 * BN, mma = 3.0 * nchunk * (rowb / 32) * npx * (n3 <= 128 ? 32 + n3 / 4 : n3 / 2);
+      for (int TH = 2; TH <= Ho; TH += 2) {
+        if (TH > 2 && TH - 2 >= Ho) break;
+        const int th = std::min(TH, Ho), tiles_h = (Ho + th - 1) / th;
+        const double ctas = (double)B * tiles_x * tiles_h * (cout / BN);
+        const double waves = std::ceil(ctas / (152.0 * occ));
+        const double bytes = (double)(th / npx + 2) * nchunk * 130 * rowb + weights + (double)th * 128 * npx * BN * 2;
+        const double drain = th / 2.0 * npx * BN * (mask ? 40.0 : 30.0);
+        const double cost = waves * (4000.0 + weights / 50.0 + std::max(std::max(occ * (th + 2) * mma, occ * bytes / 50.0), drain));
+        if (cost >= best) continue;
+        best = cost;
+        p->BN = BN;
+        p->rowb = rowb;
+        lbu::ConvRows& r = p->r;
+        r.H = H;
+        r.W = W;
+        r.up = up;
+        r.tiles_x = tiles_x;
+        r.tiles_h = tiles_h;
+        r.TH = th;
+        r.nchunk = nchunk;
+        r.cstride = cstride;
+        r.nrow = nrow;
+        r.R = R;
+        r.cols = cols;
+        r.w_off = nrow * nchunk * cstride;
+        r.stg_off = r.w_off + weights;
+        r.tail = r.stg_off + staging;
+        // no more CTAs per SM than tensor memory serves
+        p->smem = std::max(r.tail + (int)sizeof(lbu::RowsTail), kSmemSm / (occ + 1) - 1024 + 16);
+        p->grid = dim3((unsigned)(B * tiles_x * tiles_h), (unsigned)(cout / BN));
+      }
+    }
+  p->rows = best < 1e30;
+  return p->rows;
+}
+
 ConvPlan conv_plan(const bf16* x, int xs, int B, int H, int W, int cin, int up, const bf16* w, const float* bias,
                    int relu, bf16* y, int ys, int cout, const bf16* mask, int ms) {
   ConvPlan p;
@@ -349,7 +411,21 @@ ConvPlan conv_plan(const bf16* x, int xs, int B, int H, int W, int cin, int up, 
   // whole 16-byte pieces are copied, loaded and stored
   if ((((uintptr_t)x | (uintptr_t)w | (uintptr_t)y | (uintptr_t)mask) & 15u) != 0) return p;
   const int Hi = H >> up, Wi = W >> up;
-  if (!plan_tile(B, Hi, Wi, cin, cout, up, &p)) return p;
+  if (plan_rows(B, Hi, Wi, cin, cout, up, mask != nullptr, &p)) {
+    lbu::ConvRows& r = p.r;
+    r.x = x;
+    r.xs = xs;
+    r.bias = bias;
+    r.relu = relu;
+    r.y = y;
+    r.ys = ys;
+    r.mask = mask;
+    r.ms = ms;
+    p.a.TW = 128;
+    p.a.TH = -1;  // boxes of one row
+  } else if (!plan_tile(B, Hi, Wi, cin, cout, up, mask != nullptr, &p)) {
+    return p;
+  }
   lbu::ConvTma& a = p.a;
   a.x = x;
   a.xs = xs;
@@ -381,10 +457,21 @@ cudaError_t launch_conv_tma(const ConvPlan& p, int* err, cudaStream_t s) {
   lbu::conv3x3_tma_kernel<BN, ROWB><<<p.grid, lbu::kConvThreads, p.smem, s>>>(p.mx, p.mw, p.a, err);
   return cudaGetLastError();
 }
+template <int BN, int ROWB>
+cudaError_t launch_conv_rows(const ConvPlan& p, int* err, cudaStream_t s) {
+  static lbnci::SmemAllowance configured;
+  cudaError_t e = lbnci::allow_smem(lbu::conv3x3_rows_kernel<BN, ROWB>, (size_t)p.smem, configured);
+  if (e != cudaSuccess) return e;
+  lbu::conv3x3_rows_kernel<BN, ROWB><<<p.grid, lbu::kRowsThreads, p.smem, s>>>(p.mx, p.mw, p.r, err);
+  return cudaGetLastError();
+}
 cudaError_t launch_conv_plan(const ConvPlan& p, cudaStream_t s) {
   int* err = nullptr;
   cudaError_t e = cudaGetSymbolAddress((void**)&err, g_tc_err);
   if (e != cudaSuccess) return e;
+  if (p.rows)
+    return p.rowb == 128 ? (p.BN == 64 ? launch_conv_rows<64, 128>(p, err, s) : launch_conv_rows<32, 128>(p, err, s))
+                         : (p.BN == 64 ? launch_conv_rows<64, 64>(p, err, s) : launch_conv_rows<32, 64>(p, err, s));
   if (p.rowb == 128)
     return p.BN == 128 ? launch_conv_tma<128, 128>(p, err, s)
                        : (p.BN == 64 ? launch_conv_tma<64, 128>(p, err, s) : launch_conv_tma<32, 128>(p, err, s));

@@ -84,17 +84,26 @@ __device__ __forceinline__ void tmem_dealloc(unsigned taddr, unsigned ncols) {  
 __device__ __forceinline__ void fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// D (tensor memory) = A B^T (+ D when accumulate), issued by the one lane whose `leader` is
-// nonzero. The whole warp runs the issue loop, so that its addresses and descriptors are
-// warp-uniform values: issued from a branch that one lane took, each MMA cost 80 to 140
-// cycles of moves between register files, three times what the tensor cores take.
+// D (tensor memory) = A B^T (+ D when ACC), run by a whole warp and issued by the lane that
+// elect.sync picks (always the same one). With the whole warp in the issue loop its
+// addresses are warp-uniform values, and the elected predicate needs no per-lane branch.
+// Cycles per MMA of M = 128, K = 16, measured: 40, 48, 56, 64, 96 and 127 for N = 32, 64, 96,
+// 128, 192 and 256, that is the operands' bytes at 128 a cycle up to N = 128, then the tensor
+// cores' rate; a predicate from the lane number gave 50 to 72 up to N = 128, and a branch that
+// one lane takes around descriptors built with run-time multiplications 80 to 250.
 template <bool ACC>
-__device__ __forceinline__ void mma_bf16(unsigned tmem_d, unsigned long long a, unsigned long long b, unsigned idesc,
-                                         unsigned leader) {
+__device__ __forceinline__ void mma_bf16(unsigned tmem_d, unsigned long long a, unsigned long long b, unsigned idesc) {
   asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "{\n\t.reg .pred p, q;\n\t.reg .b32 x;\n\tsetp.ne.b32 p, %4, 0;\n\telect.sync x|q, 0xffffffff;\n\t"
       "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(a), "l"(b), "r"(idesc), "n"(ACC ? 1 : 0), "r"(leader)
+      "l"(a), "l"(b), "r"(idesc), "n"(ACC ? 1 : 0)
+      : "memory");
+}
+// The mbarrier receives one arrival when every MMA issued before has completed (whole warp).
+__device__ __forceinline__ void mma_commit(unsigned long long* bar) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t.reg .b32 x;\n\telect.sync x|q, 0xffffffff;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar))
       : "memory");
 }
 // Descriptor from its constant upper half and the lower half at a shared-memory address.
@@ -106,36 +115,41 @@ __device__ __forceinline__ unsigned long long desc64(unsigned hi, unsigned lo) {
 // costs a few instructions of the issuing warp and seldom follows one into its accumulator.
 template <int G, int KK, bool ACC>
 __device__ __forceinline__ void mma_group(unsigned d, unsigned dstep, const unsigned lo[G], unsigned hiA, unsigned loB,
-                                          unsigned hiB, unsigned idesc, unsigned leader) {
+                                          unsigned hiB, unsigned idesc) {
 #pragma unroll
   for (int kk = 0; kk < KK; ++kk)
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      if (ACC || kk > 0) mma_bf16<true>(d + g * dstep, desc64(hiA, lo[g] + 2 * kk), desc64(hiB, loB + 2 * kk), idesc, leader);
-      else mma_bf16<false>(d + g * dstep, desc64(hiA, lo[g]), desc64(hiB, loB), idesc, leader);
+      if (ACC || kk > 0) mma_bf16<true>(d + g * dstep, desc64(hiA, lo[g] + 2 * kk), desc64(hiB, loB + 2 * kk), idesc);
+      else mma_bf16<false>(d + g * dstep, desc64(hiA, lo[g]), desc64(hiB, loB), idesc);
     }
 }
-// The mbarrier receives one arrival when every MMA the leader issued before has completed.
-__device__ __forceinline__ void mma_commit(unsigned long long* bar, unsigned leader) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
-      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)),
-      "r"(leader)
-      : "memory");
-}
-// 16 consecutive 32-bit columns of this thread's lane (shape 32x32b: lane = warp's base + lane id)
+// 16 or 32 consecutive 32-bit columns of this thread's lane (shape 32x32b: lane = warp's base
+// + lane id); tmem_wait before the values are used.
 __device__ __forceinline__ void tmem_ld16(unsigned taddr, float v[16]) {
-  unsigned r[16];
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
       "%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
+        "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
       : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
+__device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_ld32(unsigned taddr, float v[32]) {
+  tmem_ld16(taddr, v);
+  tmem_ld16(taddr + 16u, v + 16);
+  tmem_wait();
+}
+
+// Zeros to 16 columns of this thread's lane; tmem_wait_st before they are relied on.
+__device__ __forceinline__ void tmem_zero16(unsigned taddr) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, "
+      "%1};" ::"r"(taddr),
+      "r"(0u)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // Offset of 16-byte piece v of row r in a swizzled operand of ROWB-byte rows whose patterns
 // (8 rows of 128 bytes, or of 64) are aligned.
@@ -146,6 +160,18 @@ __device__ __forceinline__ unsigned swizzled(int r, int v) {
 }
 
 }  // namespace tc
+
+// Named barrier of n threads that also says whether `ok` held for all of them.
+__device__ __forceinline__ bool bar_all(int id, int n, bool ok) {
+  int r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %3, 0;\n\tbarrier.cta.red.and.pred q, %1, %2, p;\n\t"
+      "selp.b32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"(id), "r"(n), "r"((int)ok)
+      : "memory");
+  return r != 0;
+}
 
 constexpr int kConvThreads = 320;  // copy warp, MMA warp, eight epilogue warps
 constexpr int kConvEpiThreads = 256;
@@ -175,11 +201,11 @@ struct ConvTail {
   unsigned long long bar_a, bar_p, bar_d, bar_full[kConvMaxStage], bar_empty[kConvMaxStage];
   unsigned tmem;
   int fail;
-  float bias[128];
+  alignas(16) float bias[128];
 };
 
 template <int BN, int ROWB>
-__global__ void __launch_bounds__(kConvThreads, 3)
+__global__ void __launch_bounds__(kConvThreads, 2)
 conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w, ConvTma a,
                    int* err) {
   constexpr int CH = ROWB / 2, KK = CH / 16;  // channels and K = 16 MMAs of a chunk
@@ -238,8 +264,7 @@ conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       for (int i = issued > ST ? issued - ST : 0; i < issued; ++i)
         lbnci::mbar_wait(&t.bar_full[i % ST], (unsigned)((i / ST) & 1));
     }
-  } else if (warp == 1) {  // MMAs: the whole warp, lane 0 issues
-    const unsigned leader = lane == 0;
+  } else if (warp == 1) {  // MMAs: the whole warp runs the loop
     bool bad = __any_sync(~0u, !lbnci::mbar_wait(&t.bar_a, 0u) || !lbnci::mbar_wait(&t.bar_p, 0u));
     const unsigned long long dA = tc::desc_base(ROWB, 16u, (unsigned)(a.sbo * ROWB));
     const unsigned long long dB = tc::desc_base(ROWB, 16u, 8u * ROWB);
@@ -249,7 +274,7 @@ conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     const unsigned mstep = (unsigned)(a.mstart * ROWB) >> 4;
     unsigned ph = 0u;
     int s = 0;
-    auto stage = [&](int tap, int k, auto ACC) {
+    auto stage = [&](int tap, int k, auto ACC) {  // (a converged warp: __any_sync before it)
       constexpr bool acc = decltype(ACC)::value;
       const int dy = tap / 3 - 1, dx = tap % 3 - 1;
       const unsigned lb = loB0 + (unsigned)(s * (BBYTES >> 4)), la = loA0 + (unsigned)((k * a.a_stride) >> 4);
@@ -261,7 +286,7 @@ conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
 #pragma unroll
         for (int q = 0; q < 4; ++q) lo[q] = at(((q >> 1) + dy) >> 1, ((q & 1) + dx) >> 1);
         for (int m = 0; m < a.nm; ++m) {
-          tc::mma_group<4, KK, acc>(tmem + m * BN, (unsigned)(a.nm * BN), lo, hiA, lb, hiB, IDESC, leader);
+          tc::mma_group<4, KK, acc>(tmem + m * BN, (unsigned)(a.nm * BN), lo, hiA, lb, hiB, IDESC);
 #pragma unroll
           for (int q = 0; q < 4; ++q) lo[q] += mstep;
         }
@@ -273,15 +298,15 @@ conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         lo[3] = lo[2] + mstep;
         int m = 0;
         for (; m + 4 <= a.nm; m += 4) {
-          tc::mma_group<4, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC, leader);
+          tc::mma_group<4, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC);
 #pragma unroll
           for (int g = 0; g < 4; ++g) lo[g] += 4 * mstep;
         }
-        if (a.nm - m == 3) tc::mma_group<3, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC, leader);
-        else if (a.nm - m == 2) tc::mma_group<2, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC, leader);
-        else if (a.nm - m == 1) tc::mma_group<1, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC, leader);
+        if (a.nm - m == 3) tc::mma_group<3, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC);
+        else if (a.nm - m == 2) tc::mma_group<2, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC);
+        else if (a.nm - m == 1) tc::mma_group<1, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC);
       }
-      tc::mma_commit(&t.bar_empty[s], leader);
+      tc::mma_commit(&t.bar_empty[s]);
       if (++s == ST) {
         s = 0;
         ph ^= 1u;
@@ -298,7 +323,7 @@ conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     if (lane == 0) {
       if (bad) atomicOr(&t.fail, 1);
     }
-    tc::mma_commit(&t.bar_d, leader);
+    tc::mma_commit(&t.bar_d);
     if (lane == 0) lbnci::mbar_arrive(&t.bar_d);
   } else {
     const int et = tid - 64;
@@ -341,43 +366,50 @@ conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       __syncwarp();
       if (lane == 0) lbnci::mbar_arrive(&t.bar_p);
     }
+    const int Wo = a.W << a.up, Ho = a.H << a.up, nacc = a.nm * (a.up ? 4 : 1);
+    auto out_row = [&](int m, int par, int r0) {  // output pixel of operand row r0, -1: none
+      int r, c;
+      if (a.linear) {
+        const int pos = m * a.mstart + r0;
+        r = pos / a.pitch;
+        c = pos - r * a.pitch;
+      } else {
+        r = r0 >> 3;
+        c = 8 * m + (r0 & 7);
+      }
+      const int yy = y0 + r, xx = x0 + c;
+      if (!(r < a.TH && c < a.TW && yy < a.H && xx < a.W)) return -1;
+      return a.up ? (b * Ho + 2 * yy + (par >> 1)) * Wo + 2 * xx + (par & 1) : (b * Ho + yy) * Wo + xx;
+    };
+    if (a.mask)  // the mask's lines into L2 while the MMAs run
+      for (int e = et; e < nacc * 128; e += kConvEpiThreads) {
+        const int row = out_row((e >> 7) % a.nm, (e >> 7) / a.nm, e & 127);
+        if (row >= 0)
+          for (int j = 0; j < BN; j += 64)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(a.mask + (size_t)row * a.ms + n0 + j));
+      }
     // drain: group g of four warps takes accumulators g, g + 2, ...
     const bool done = lbnci::mbar_wait(&t.bar_d, 0u);
     if (!done) atomicOr(&t.fail, 1);
     tc::fence_after_sync();
-    if (done && *(volatile int*)&t.fail == 0) {
+    if (bar_all(1, kConvEpiThreads, done && *(volatile int*)&t.fail == 0)) {
       const int g = (warp - 2) >> 2, quad = warp & 3, l = quad * 32 + lane, gt = et & 127;
       unsigned char* const stg = sm + g * (128 * BN * 2);
       constexpr int NV = BN / 8;                      // 16-byte pieces of a pixel's output
       auto piece = [](int r, int v) {                 // bank-conflict-free place of piece v of row r
         return r * (BN * 2) + ((v ^ ((BN == 32 ? r >> 1 : r) & (NV < 8 ? NV - 1 : 7))) << 4);
       };
-      const int nacc = a.nm * (a.up ? 4 : 1), Wo = a.W << a.up, Ho = a.H << a.up;
       for (int q = g; q < nacc; q += 2) {
         const int par = a.up ? q / a.nm : 0, m = q - par * a.nm;
-        auto out_row = [&](int r0) {  // output pixel of operand row r0, -1: none
-          int r, c;
-          if (a.linear) {
-            const int pos = m * a.mstart + r0;
-            r = pos / a.pitch;
-            c = pos - r * a.pitch;
-          } else {
-            r = r0 >> 3;
-            c = 8 * m + (r0 & 7);
-          }
-          const int yy = y0 + r, xx = x0 + c;
-          if (!(r < a.TH && c < a.TW && yy < a.H && xx < a.W)) return -1;
-          return a.up ? (b * Ho + 2 * yy + (par >> 1)) * Wo + 2 * xx + (par & 1) : (b * Ho + yy) * Wo + xx;
-        };
         // this thread's pieces k = 0 .. NV - 1 of the tile: row (128 k + gt) / NV, piece gt % NV.
-        // The first four masks are in flight while the accumulator is drained.
-        constexpr int UB = NV < 4 ? NV : 4;
+        // The first masks are in flight while the accumulator is drained.
+        constexpr int UB = NV < 8 ? 4 : 8;
         int orow[UB];
         uint4 mk[UB];
         auto fetch = [&](int k0) {
 #pragma unroll
           for (int k = 0; k < UB; ++k) {
-            orow[k] = out_row(((k0 + k) * 128 + gt) / NV);
+            orow[k] = out_row(m, par, ((k0 + k) * 128 + gt) / NV);
             if (a.mask && orow[k] >= 0)
               mk[k] = *reinterpret_cast<const uint4*>(a.mask + (size_t)orow[k] * a.ms + n0 + (gt % NV) * 8);
           }
@@ -385,21 +417,24 @@ conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         fetch(0);
         const unsigned taddr = tmem + (unsigned)(q * BN) + ((unsigned)(quad * 32) << 16);
 #pragma unroll
-        for (int c0 = 0; c0 < BN; c0 += 16) {
-          float acc[16];
-          tc::tmem_ld16(taddr + (unsigned)c0, acc);
-          V8 o[2];
+        for (int c0 = 0; c0 < BN; c0 += 32) {
+          float acc[32];
+          tc::tmem_ld32(taddr + (unsigned)c0, acc);
 #pragma unroll
-          for (int j = 0; j < 16; j += 2) {
-            float v0 = acc[j] + t.bias[c0 + j], v1 = acc[j + 1] + t.bias[c0 + j + 1];
+          for (int v = 0; v < 4; ++v) {
+            const float4 b0 = *reinterpret_cast<const float4*>(&t.bias[c0 + 8 * v]);
+            const float4 b1 = *reinterpret_cast<const float4*>(&t.bias[c0 + 8 * v + 4]);
+            float r[8] = {acc[8 * v] + b0.x,     acc[8 * v + 1] + b0.y, acc[8 * v + 2] + b0.z, acc[8 * v + 3] + b0.w,
+                          acc[8 * v + 4] + b1.x, acc[8 * v + 5] + b1.y, acc[8 * v + 6] + b1.z, acc[8 * v + 7] + b1.w};
             if (a.relu) {
-              v0 = fmaxf(v0, 0.f);
-              v1 = fmaxf(v1, 0.f);
+#pragma unroll
+              for (int j = 0; j < 8; ++j) r[j] = fmaxf(r[j], 0.f);
             }
-            o[j >> 3].h[(j & 7) >> 1] = __floats2bfloat162_rn(v0, v1);
+            V8 o;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) o.h[j] = __floats2bfloat162_rn(r[2 * j], r[2 * j + 1]);
+            *reinterpret_cast<uint4*>(stg + piece(l, c0 / 8 + v)) = o.u;
           }
-          *reinterpret_cast<uint4*>(stg + piece(l, c0 / 8)) = o[0].u;
-          *reinterpret_cast<uint4*>(stg + piece(l, c0 / 8 + 1)) = o[1].u;
         }
         asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory");
 #pragma unroll
@@ -422,6 +457,289 @@ conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             }
             *reinterpret_cast<uint4*>(a.y + (size_t)orow[k] * a.ys + n0 + (gt % NV) * 8) = o.u;
           }
+        }
+        asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory");
+      }
+    }
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  __syncwarp();
+  if (warp == 1) tc::tmem_dealloc(tmem, (unsigned)a.cols);
+  if (tid == 0 && t.fail) atomicOr(err, t.fail);
+}
+
+// ------------------------------------------------------------------ wide images, few channels
+// The same convolution for 32 or 64 output channels on wide images, row by row. An MMA's
+// operand fetch (128 rows of A) costs as much for N = 32 as the products of N = 96, so here
+// one MMA multiplies an input row, shifted by dx, with the weights of the three dy at once
+// (N = 3 BN, the weights stacked dy = +1, 0, -1) into the accumulators of the three output
+// rows h = v - 1, v, v + 1 it contributes to, which lie side by side in tensor memory.
+// Input rows go by in order, so every output row still adds dy = -1, 0, +1, dx, channels in
+// the order of conv3x3_kernel: the same bits. A CTA takes 128 columns of TH output rows: the
+// weights stay in shared memory, input rows pass through a ring (each copied once), output
+// rows through a ring of R accumulators; a row is drained while the next ones are computed.
+//
+// up: virtual input row V of the upsampled image is row V >> 1 of the input, taken twice;
+// output columns 2 x + px have accumulators of their own (px = 0, 1), reading the input
+// column shifted by floor((px + dx)/2).
+//
+// An accumulator starts from zeros that the draining warps store (a row's first MMA shares
+// its instruction with two rows that accumulate); 0 + a is a.
+//
+// Warps: 0 copies, 1 issues MMAs, 2..9 drain (two groups of four, alternate rows), 10 patches
+// the periodic columns.
+constexpr int kRowsThreads = 352, kRowsMaxStage = 8, kRowsMaxSlot = 16;
+struct ConvRows {
+  const bf16* x;
+  int xs, H, W, up;        // input image
+  int tiles_x, tiles_h, TH;  // strips of 128 columns, groups of TH output rows
+  int nchunk, cstride;     // chunks of ROWB/2 channels; bytes of a row's chunk in shared memory
+  int nrow, R;             // ring stages (input rows), accumulator slots (output rows, even)
+  int w_off, stg_off, tail;
+  int cols;
+  const float* bias;
+  int relu;
+  bf16* y;
+  int ys;
+  const bf16* mask;
+  int ms;
+};
+struct RowsTail {
+  unsigned long long bar_w, bar_full[kRowsMaxStage], bar_patched[kRowsMaxStage], bar_empty[kRowsMaxStage];
+  unsigned long long bar_row[kRowsMaxSlot], bar_free[kRowsMaxSlot];
+  unsigned tmem;
+  int fail;
+  alignas(16) float bias[64];
+};
+
+template <int BN, int ROWB>
+__global__ void __launch_bounds__(kRowsThreads, 2)
+conv3x3_rows_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w, ConvRows a,
+                    int* err) {
+  constexpr int CH = ROWB / 2, KK = CH / 16, WB = BN * ROWB, XW = 130;
+  extern __shared__ __align__(1024) unsigned char sm[];
+  RowsTail& t = *reinterpret_cast<RowsTail*>(sm + a.tail);
+  unsigned char* const sW = sm + a.w_off;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tx = blockIdx.x % a.tiles_x, th = (blockIdx.x / a.tiles_x) % a.tiles_h;
+  const int b = blockIdx.x / (a.tiles_x * a.tiles_h);
+  const int x0 = tx * 128, h0 = th * a.TH, n0 = blockIdx.y * BN;
+  const int Ho = a.H << a.up, Wo = a.W << a.up, npx = a.up ? 2 : 1;
+  const int nh = min(a.TH, Ho - h0);
+  const int first = a.up ? (h0 >> 1) - 1 : h0 - 1, nin = a.up ? (nh >> 1) + 2 : nh + 2;
+  const int row_bytes = a.nchunk * a.cstride;
+
+  if (tid == 0) {
+    lbnci::mbar_init(&t.bar_w, 1);
+    for (int s = 0; s < a.nrow; ++s) {
+      lbnci::mbar_init(&t.bar_full[s], 1);
+      lbnci::mbar_init(&t.bar_patched[s], 1);
+      lbnci::mbar_init(&t.bar_empty[s], 1);
+    }
+    for (int s = 0; s < a.R; ++s) {
+      lbnci::mbar_init(&t.bar_row[s], 1);
+      lbnci::mbar_init(&t.bar_free[s], 4);
+    }
+    t.fail = (smem_u32(sm) & 1023u) ? 2 : 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) tc::tmem_alloc(&t.tmem, (unsigned)a.cols);
+  if (tid < BN) t.bias[tid] = a.bias ? a.bias[n0 + tid] : 0.f;
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const unsigned tmem = t.tmem;
+  const bool aligned = t.fail == 0;
+
+  if (!aligned) {
+    // nothing was started
+  } else if (warp == 0) {
+    if (lane == 0) {  // copies: the weights (dx, chunk, dy = +1, 0, -1), then the rows
+      lbnci::mbar_expect_tx(&t.bar_w, (unsigned)(9 * a.nchunk * WB));
+      for (int dxi = 0; dxi < 3; ++dxi)
+        for (int k = 0; k < a.nchunk; ++k)
+          for (int j = 0; j < 3; ++j)
+            lbnci::tma_load_2d(sW + ((dxi * a.nchunk + k) * 3 + j) * WB, &map_w,
+                               (((2 - j) * 3 + dxi) * a.nchunk + k) * CH, n0, &t.bar_w);
+      int issued = 0;
+      for (int i = 0; i < nin; ++i) {
+        const int s = i % a.nrow, u = i / a.nrow;
+        if (u > 0 && !lbnci::mbar_wait(&t.bar_empty[s], (unsigned)((u - 1) & 1))) {
+          atomicOr(&t.fail, 1);
+          break;
+        }
+        lbnci::mbar_expect_tx(&t.bar_full[s], (unsigned)(a.nchunk * XW * ROWB));
+        for (int k = 0; k < a.nchunk; ++k)
+          lbnci::tma_load_4d(sm + s * row_bytes + k * a.cstride, &map_x, k * CH, x0 - 1, first + i, b, &t.bar_full[s]);
+        issued = i + 1;
+      }
+      lbnci::mbar_wait(&t.bar_w, 0u);  // every copy has landed before the CTA may end (bounded)
+      for (int i = issued > a.nrow ? issued - a.nrow : 0; i < issued; ++i)
+        lbnci::mbar_wait(&t.bar_full[i % a.nrow], (unsigned)((i / a.nrow) & 1));
+    }
+  } else if (warp == 1) {  // MMAs: the whole warp runs the loop
+    const unsigned long long d0 = tc::desc_base(ROWB, 16u, 8u * ROWB);
+    const unsigned hi = (unsigned)(d0 >> 32);
+    const unsigned loA = (unsigned)d0 + (smem_u32(sm) >> 4), loW = (unsigned)d0 + (smem_u32(sW) >> 4);
+    bool bad = __any_sync(~0u, !lbnci::mbar_wait(&t.bar_w, 0u));
+    int s = 0;
+    unsigned ph = 0u;
+    for (int i = 0; i < nin && !bad; ++i) {
+      bad = __any_sync(~0u, !lbnci::mbar_wait(&t.bar_full[s], ph) || !lbnci::mbar_wait(&t.bar_patched[s], ph));
+      if (bad) break;
+      tc::fence_after_sync();
+      const unsigned la = loA + (unsigned)((s * row_bytes) >> 4);
+      for (int pass = 0; pass < npx; ++pass) {
+        const int v = a.up ? 2 * (i - 1) + pass : i - 1;  // virtual input row, relative to h0
+        if (v < -1 || v > nh) continue;
+        const int lo = max(0, v - 1), hi_row = min(nh - 1, v + 1), n = hi_row - lo + 1;
+        if (hi_row == v + 1) {  // a new output row: its slot is drained and zeroed
+          bad = __any_sync(~0u, !lbnci::mbar_wait(&t.bar_free[hi_row % a.R], (unsigned)((hi_row / a.R) & 1)));
+          if (bad) break;
+          tc::fence_after_sync();
+        }
+        // rows lo .. hi_row in slots; beyond the last slot they continue at slot 0
+        const int slot = lo % a.R, n1 = min(n, a.R - slot), n2 = n - n1, j0 = lo - (v - 1);
+        auto rows = [&](int sl, int j, int nn) {
+          const unsigned id = tc::idesc_bf16(128, 0) | ((unsigned)(nn * BN / 8) << 17);
+          // dx outermost, then channels: the order of the taps
+#pragma unroll
+          for (int dxi = 0; dxi < 3; ++dxi)
+            for (int k = 0; k < a.nchunk; ++k) {
+              const unsigned lw = loW + (unsigned)((((dxi * a.nchunk + k) * 3 + j) * WB) >> 4);
+              const unsigned lk = la + (unsigned)((k * a.cstride) >> 4);
+              for (int px = 0; px < npx; ++px) {
+                const int ox = a.up ? (px + dxi - 1) >> 1 : dxi - 1;
+                const unsigned lr = lk + (unsigned)(((ox + 1) * ROWB) >> 4);
+                const unsigned d = tmem + (unsigned)((px * a.R + sl) * BN);
+#pragma unroll
+                for (int kk = 0; kk < KK; ++kk)
+                  tc::mma_bf16<true>(d, tc::desc64(hi, lr + 2 * kk), tc::desc64(hi, lw + 2 * kk), id);
+              }
+            }
+        };
+        rows(slot, j0, n1);
+        if (n2 > 0) rows(0, j0 + n1, n2);
+        if (v >= 1) tc::mma_commit(&t.bar_row[(v - 1) % a.R]);  // output row v - 1 is complete
+      }
+      tc::mma_commit(&t.bar_empty[s]);
+      if (++s == a.nrow) {
+        s = 0;
+        ph ^= 1u;
+      }
+    }
+    if (lane == 0 && bad) atomicOr(&t.fail, 1);
+    // the MMAs issued are done before tensor memory is released: the last row's barrier below
+  } else if (warp == 10) {  // the periodic images of the columns beyond the image
+    const int left = x0 == 0 ? 1 : 0, right = x0 + 128 >= a.W ? 1 : 0, ncol = left + right;
+    const int vpp = a.nchunk * (ROWB / 16), count = ncol * vpp;
+    bool ok = true;
+    for (int i = 0; i < nin && ok; ++i) {
+      const int s = i % a.nrow, yy = first + i;
+      const bool in = yy >= 0 && yy < a.H;
+      for (int e0 = 0; e0 < count || e0 == 0; e0 += 64) {
+        uint4 v[2];
+        int dst[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int e = e0 + 32 * j + lane;
+          dst[j] = -1;
+          if (in && e < count) {
+            const int col = e / vpp, p = e - col * vpp, k = p / (ROWB / 16);
+            const bool lft = left && col == 0;
+            v[j] = *reinterpret_cast<const uint4*>(a.x + ((size_t)(b * a.H + yy) * a.W + (lft ? a.W - 1 : 0)) * a.xs + p * 8);
+            dst[j] = s * row_bytes + k * a.cstride +
+                     (int)tc::swizzled<ROWB>(lft ? 0 : a.W - x0 + 1, p - k * (ROWB / 16));
+          }
+        }
+        if (e0 == 0) ok = __all_sync(~0u, lbnci::mbar_wait(&t.bar_full[s], (unsigned)((i / a.nrow) & 1)));
+        if (!ok) break;
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+          if (dst[j] >= 0) *reinterpret_cast<uint4*>(sm + dst[j]) = v[j];
+      }
+      lbnci::fence_async_smem();
+      __syncwarp();
+      if (lane == 0) {
+        if (!ok) atomicOr(&t.fail, 1);
+        lbnci::mbar_arrive(&t.bar_patched[s]);
+      }
+    }
+  } else {  // drain
+    const int g = (warp - 2) >> 2, quad = warp & 3, l = quad * 32 + lane, gt = (tid - 64) & 127;
+    const unsigned tq = tmem + ((unsigned)(quad * 32) << 16);
+    auto zero = [&](int slot) {  // this warp's lanes of a slot's accumulators
+      for (int px = 0; px < npx; ++px)
+#pragma unroll
+        for (int c0 = 0; c0 < BN; c0 += 16) tc::tmem_zero16(tq + (unsigned)((px * a.R + slot) * BN + c0));
+      tc::tmem_wait_st();
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) lbnci::mbar_arrive(&t.bar_free[slot]);
+    };
+    for (int s = g; s < a.R; s += 2) zero(s);
+    unsigned char* const stg = sm + a.stg_off + g * (128 * BN * 2);
+    constexpr int NV = BN / 8;
+    auto piece = [](int r, int v) { return r * (BN * 2) + ((v ^ ((BN == 32 ? r >> 1 : r) & (NV - 1))) << 4); };
+    bool ok = true;
+    for (int h = g; h < nh && ok; h += 2) {
+      const int slot = h % a.R;
+      for (int px = 0; px < npx; ++px) {
+        // this thread's pieces: row (128 k + gt) / NV, piece gt % NV; the masks are in flight
+        // while the row is awaited
+        int orow[NV];
+        uint4 mk[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+          const int x = x0 + (k * 128 + gt) / NV;
+          orow[k] = x < a.W ? (b * Ho + h0 + h) * Wo + (a.up ? 2 * x + px : x) : -1;
+          if (a.mask && orow[k] >= 0)
+            mk[k] = *reinterpret_cast<const uint4*>(a.mask + (size_t)orow[k] * a.ms + n0 + (gt % NV) * 8);
+        }
+        if (px == 0) {
+          ok = lbnci::mbar_wait(&t.bar_row[slot], (unsigned)((h / a.R) & 1));
+          if (!ok) atomicOr(&t.fail, 1);
+          tc::fence_after_sync();
+        }
+#pragma unroll
+        for (int c0 = 0; c0 < BN; c0 += 32) {
+          float acc[32];
+          tc::tmem_ld32(tq + (unsigned)((px * a.R + slot) * BN + c0), acc);
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            const float4 b0 = *reinterpret_cast<const float4*>(&t.bias[c0 + 8 * v]);
+            const float4 b1 = *reinterpret_cast<const float4*>(&t.bias[c0 + 8 * v + 4]);
+            float r[8] = {acc[8 * v] + b0.x,     acc[8 * v + 1] + b0.y, acc[8 * v + 2] + b0.z, acc[8 * v + 3] + b0.w,
+                          acc[8 * v + 4] + b1.x, acc[8 * v + 5] + b1.y, acc[8 * v + 6] + b1.z, acc[8 * v + 7] + b1.w};
+            if (a.relu) {
+#pragma unroll
+              for (int j = 0; j < 8; ++j) r[j] = fmaxf(r[j], 0.f);
+            }
+            V8 o;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) o.h[j] = __floats2bfloat162_rn(r[2 * j], r[2 * j + 1]);
+            *reinterpret_cast<uint4*>(stg + piece(l, c0 / 8 + v)) = o.u;
+          }
+        }
+        if (px == npx - 1 && h + a.R < nh) zero(slot);  // for row h + R
+        ok = bar_all(1 + g, 128, ok);
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+          if (orow[k] < 0 || !ok) continue;
+          V8 o;
+          o.u = *reinterpret_cast<const uint4*>(stg + piece((k * 128 + gt) / NV, gt % NV));
+          if (a.mask) {
+            V8 w;
+            w.u = mk[k];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const float2 mf = __bfloat1622float2(w.h[j]);
+              if (!(mf.x > 0.f)) o.h[j].x = __float2bfloat16_rn(0.f);
+              if (!(mf.y > 0.f)) o.h[j].y = __float2bfloat16_rn(0.f);
+            }
+          }
+          *reinterpret_cast<uint4*>(a.y + (size_t)orow[k] * a.ys + n0 + (gt % NV) * 8) = o.u;
         }
         asm volatile("bar.sync %0, 128;" ::"r"(1 + g) : "memory");
       }
@@ -532,8 +850,7 @@ conv3x3_wgrad_tma_kernel(const __grid_constant__ WgradMaps maps, WgradTma a, int
       for (int i = issued > ST ? issued - ST : 0; i < issued; ++i)
         lbnci::mbar_wait(&t.bar_full[i % ST], (unsigned)((i / ST) & 1));
     }
-  } else if (warp == 1) {  // MMAs: the whole warp, lane 0 issues
-    const unsigned leader = lane == 0;
+  } else if (warp == 1) {  // MMAs: the whole warp runs the loop
     bool bad = false;
     const unsigned long long dB = tc::desc_base(DROW, 16u, 8u * DROW);
     const unsigned hiA = (unsigned)(tc::desc_base(ROWB, 16u, 8u * ROWB) >> 32), hiB = (unsigned)(dB >> 32);
@@ -567,11 +884,11 @@ conv3x3_wgrad_tma_kernel(const __grid_constant__ WgradMaps maps, WgradTma a, int
 #pragma unroll
         for (int j = 0; j < NA; ++j)
           tc::mma_bf16<acc>(tmem + j * BN, tc::desc64(hiA, ua + rel[j]), tc::desc64(hiB, ub + (unsigned)(j >> 1) * dpar),
-                            IDESC, leader);
+                            IDESC);
       } else {
 #pragma unroll
         for (int j = 0; j < (ROWB == 64 ? 3 : 5); ++j)
-          tc::mma_bf16<acc>(tmem + j * BN, tc::desc64(hiA, ua + rel[j]), tc::desc64(hiB, ub), IDESC, leader);
+          tc::mma_bf16<acc>(tmem + j * BN, tc::desc64(hiA, ua + rel[j]), tc::desc64(hiB, ub), IDESC);
       }
     };
     for (int i = 0; i < nt; ++i) {
@@ -589,14 +906,14 @@ conv3x3_wgrad_tma_kernel(const __grid_constant__ WgradMaps maps, WgradTma a, int
           ub += DROW;
         }
       }
-      tc::mma_commit(&t.bar_empty[s], leader);
+      tc::mma_commit(&t.bar_empty[s]);
       if (++s == ST) {
         s = 0;
         ph ^= 1u;
       }
     }
     if (lane == 0 && bad) atomicOr(&t.fail, 1);
-    tc::mma_commit(&t.bar_d, leader);
+    tc::mma_commit(&t.bar_d);
     if (lane == 0) lbnci::mbar_arrive(&t.bar_d);
   } else {
     const int et = tid - 64;
@@ -662,8 +979,8 @@ conv3x3_wgrad_tma_kernel(const __grid_constant__ WgradMaps maps, WgradTma a, int
       atomicOr(&t.fail, 1);
     }
     tc::fence_after_sync();
-    asm volatile("bar.sync 1, 256;" ::: "memory");  // every epilogue warp is past the stages
-    if (ok && *(volatile int*)&t.fail == 0) {
+    // every epilogue warp is past the stages
+    if (bar_all(1, kConvEpiThreads, ok && *(volatile int*)&t.fail == 0)) {
       if (do_bias) {  // thread sums, added in thread order
         float* red = reinterpret_cast<float*>(sm);
 #pragma unroll
@@ -687,12 +1004,12 @@ conv3x3_wgrad_tma_kernel(const __grid_constant__ WgradMaps maps, WgradTma a, int
         float* out = a.part + ((size_t)split * a.Cout + n0) * nk * a.Cin + (size_t)(k < 0 ? 0 : k) * a.Cin + ci;
         const unsigned taddr = tmem + (unsigned)(q * BN) + ((unsigned)(quad * 32) << 16);
 #pragma unroll
-        for (int j0 = 0; j0 < BN; j0 += 16) {
-          float acc[16];
-          tc::tmem_ld16(taddr + (unsigned)j0, acc);
+        for (int j0 = 0; j0 < BN; j0 += 32) {
+          float acc[32];
+          tc::tmem_ld32(taddr + (unsigned)j0, acc);
           if (k >= 0) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) out[(size_t)(j0 + j) * nk * a.Cin] = acc[j];
+            for (int j = 0; j < 32; ++j) out[(size_t)(j0 + j) * nk * a.Cin] = acc[j];
           }
         }
       }
