@@ -42,7 +42,8 @@ cudaError_t allow_smem(K kernel, size_t bytes, SmemAllowance& a) {
 // started (pdl_begin) or ended. pdl_begin waits for that kernel's completion (its writes
 // visible) before anything of the chain's memory is touched, so results and order are those
 // of plain launches; what overlaps is the launch latency and the last blocks' tail. Every
-// kernel launched this way begins with pdl_begin (which does nothing after a plain launch).
+// kernel launched this way begins with pdl_begin or pdl_enter (which do nothing after a plain
+// launch).
 template <typename... P, typename... A>
 cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -61,6 +62,17 @@ cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cuda
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// The same with the next launch released only after the wait: when a kernel's blocks start,
+// every kernel before its predecessor has completed. What a block does before pdl_enter may
+// therefore read what the predecessor does not write (a network's weights), and blocks that
+// hold tensor memory at the wait never keep it from a block that has yet to start. Measured
+// on the U-Net's chains of 5 to 60 us kernels (setup, barrier initialisation, tensor-memory
+// allocation and the first weights overlap the kernel before): batch-8 forward of 23 launches
+// 289 -> 239 us, batch-32 training step of 86 launches 1771 -> 1587 us.
+__device__ __forceinline__ void pdl_enter() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 #endif
 

@@ -450,33 +450,41 @@ ConvPlan conv_plan(const bf16* x, int xs, int B, int H, int W, int cin, int up, 
 }
 
 template <int BN, int ROWB>
-cudaError_t launch_conv_tma(const ConvPlan& p, int* err, cudaStream_t s) {
+cudaError_t launch_conv_tma(const ConvPlan& p, int* err, cudaStream_t s, bool chained) {
   static lbnci::SmemAllowance configured;
   cudaError_t e = lbnci::allow_smem(lbu::conv3x3_tma_kernel<BN, ROWB>, (size_t)p.smem, configured);
   if (e != cudaSuccess) return e;
+  if (chained)
+    return lbnci::launch_pdl(lbu::conv3x3_tma_kernel<BN, ROWB>, dim3(p.grid), dim3(lbu::kConvThreads), p.smem, s, p.mx,
+                             p.mw, p.a, err);
   lbu::conv3x3_tma_kernel<BN, ROWB><<<p.grid, lbu::kConvThreads, p.smem, s>>>(p.mx, p.mw, p.a, err);
   return cudaGetLastError();
 }
 template <int BN, int ROWB>
-cudaError_t launch_conv_rows(const ConvPlan& p, int* err, cudaStream_t s) {
+cudaError_t launch_conv_rows(const ConvPlan& p, int* err, cudaStream_t s, bool chained) {
   static lbnci::SmemAllowance configured;
   cudaError_t e = lbnci::allow_smem(lbu::conv3x3_rows_kernel<BN, ROWB>, (size_t)p.smem, configured);
   if (e != cudaSuccess) return e;
+  if (chained)
+    return lbnci::launch_pdl(lbu::conv3x3_rows_kernel<BN, ROWB>, dim3(p.grid), dim3(lbu::kRowsThreads), p.smem, s, p.mx,
+                             p.mw, p.r, err);
   lbu::conv3x3_rows_kernel<BN, ROWB><<<p.grid, lbu::kRowsThreads, p.smem, s>>>(p.mx, p.mw, p.r, err);
   return cudaGetLastError();
 }
-cudaError_t launch_conv_plan(const ConvPlan& p, cudaStream_t s) {
+// chained: the launch follows a kernel of the network on its stream (whose wait the weights
+// precede), so it may start while that one drains; a single convolution takes no part in it.
+cudaError_t launch_conv_plan(const ConvPlan& p, cudaStream_t s, bool chained) {
   int* err = nullptr;
   cudaError_t e = cudaGetSymbolAddress((void**)&err, g_tc_err);
   if (e != cudaSuccess) return e;
   if (p.rows)
-    return p.rowb == 128 ? (p.BN == 64 ? launch_conv_rows<64, 128>(p, err, s) : launch_conv_rows<32, 128>(p, err, s))
-                         : (p.BN == 64 ? launch_conv_rows<64, 64>(p, err, s) : launch_conv_rows<32, 64>(p, err, s));
+    return p.rowb == 128 ? (p.BN == 64 ? launch_conv_rows<64, 128>(p, err, s, chained) : launch_conv_rows<32, 128>(p, err, s, chained))
+                         : (p.BN == 64 ? launch_conv_rows<64, 64>(p, err, s, chained) : launch_conv_rows<32, 64>(p, err, s, chained));
   if (p.rowb == 128)
-    return p.BN == 128 ? launch_conv_tma<128, 128>(p, err, s)
-                       : (p.BN == 64 ? launch_conv_tma<64, 128>(p, err, s) : launch_conv_tma<32, 128>(p, err, s));
-  return p.BN == 128 ? launch_conv_tma<128, 64>(p, err, s)
-                     : (p.BN == 64 ? launch_conv_tma<64, 64>(p, err, s) : launch_conv_tma<32, 64>(p, err, s));
+    return p.BN == 128 ? launch_conv_tma<128, 128>(p, err, s, chained)
+                       : (p.BN == 64 ? launch_conv_tma<64, 128>(p, err, s, chained) : launch_conv_tma<32, 128>(p, err, s, chained));
+  return p.BN == 128 ? launch_conv_tma<128, 64>(p, err, s, chained)
+                     : (p.BN == 64 ? launch_conv_tma<64, 64>(p, err, s, chained) : launch_conv_tma<32, 64>(p, err, s, chained));
 }
 
 // LBNCI_UNET_MMA=sync selects the mma.sync convolution for every layer. It stays for the
@@ -515,7 +523,7 @@ cudaError_t launch_wgrad_tma(const WgradTmaPlan& p, const lbu::WgradMaps& maps, 
   e = lbnci::allow_smem(lbu::conv3x3_wgrad_tma_kernel<BN, ROWB>, (size_t)p.smem, configured);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)p.a.nsplit, (unsigned)(p.a.Cin / (ROWB / 2)), (unsigned)(p.a.Cout / BN));
-  lbu::conv3x3_wgrad_tma_kernel<BN, ROWB><<<grid, lbu::kConvThreads, p.smem, s>>>(maps, p.a, err);
+  lbnci::launch_pdl(lbu::conv3x3_wgrad_tma_kernel<BN, ROWB>, dim3(grid), dim3(lbu::kConvThreads), p.smem, s, maps, p.a, err);
   return cudaGetLastError();
 }
 
@@ -545,7 +553,7 @@ lb_status conv(lbu_net* n, int site, const bf16* x, int xs, int B, int H, int W,
       c.B = B;
     }
     if (c.p.ok) {
-      cudaError_t e = launch_conv_plan(c.p, s);
+      cudaError_t e = launch_conv_plan(c.p, s, n != nullptr);
       if (n) ++n->launches;
       return e == cudaSuccess ? LB_OK : cuda_fail(n, e, "conv3x3 (tensor memory) launch");
     }
@@ -593,7 +601,7 @@ lb_status wgrad(lbu_net* n, int site, const bf16* x, int xs, int up, const bf16*
       int S = 1;  // threads to each group of four values: about four blocks per multiprocessor
       while (S < 32 && 2 * S <= p.a.nsplit && (long long)n4 * S < 152LL * 4 * 256) S *= 2;
       const int wblocks = (n4 + 256 / S - 1) / (256 / S), bblocks = db_master ? (cout + 31) / 32 : 0;
-      lbu::wgrad_reduce_tma_kernel<<<wblocks + bblocks, 256, 0, s>>>(work, bp, p.a.nsplit, cout, cin, cin_true, up, S,
+      lbnci::launch_pdl(lbu::wgrad_reduce_tma_kernel, dim3(wblocks + bblocks), dim3(256), 0, s, work, bp, p.a.nsplit, cout, cin, cin_true, up, S,
                                                                      wblocks, dw_master, db_master);
       if (n) n->launches += 2;
       e = cudaGetLastError();
@@ -647,7 +655,7 @@ lb_status forward_impl(lbu_net* n, int B) {
       LBU_TRY(conv(n, enc_b(l), n->ea[l], C, B, H, W, C, 0, WB(n, enc_b(l)), BIAS(n, enc_b(l)), 1, n->cat[l] + C, 2 * C, C,
                    nullptr, 0, s));
       const long long work = (long long)B * (H / 2) * (W / 2) * (C / 8);
-      lbu::maxpool_kernel<<<grid_for(work, 256), 256, 0, s>>>(n->cat[l] + C, 2 * C, B, H, W, C, n->pool[l]);
+      lbnci::launch_pdl(lbu::maxpool_kernel, dim3(grid_for(work, 256)), dim3(256), 0, s, n->cat[l] + C, 2 * C, B, H, W, C, n->pool[l]);
       ++n->launches;
       h = n->pool[l];
       hs = C;
@@ -669,7 +677,7 @@ lb_status forward_impl(lbu_net* n, int B) {
   }
   const int hi = head_i(n);
   const int P = B * n->cfg.H * n->cfg.W;
-  lbu::head_fwd_kernel<<<grid_for(P, 256), 256, 0, s>>>(n->db[0], n->cfg.base, WB(n, hi), BIAS(n, hi),
+  lbnci::launch_pdl(lbu::head_fwd_kernel, dim3(grid_for(P, 256)), dim3(256), 0, s, n->db[0], n->cfg.base, WB(n, hi), BIAS(n, hi),
                                                         n->cfg.out_ch, P, n->y);
   ++n->launches;
   cudaError_t e = cudaGetLastError();
@@ -688,8 +696,8 @@ lb_status backward_impl(lbu_net* n, int B) {
   {
     const int hi = head_i(n), C0 = n->cfg.base;
     const int nblk = (P + lbu::kHeadPix - 1) / lbu::kHeadPix;
-    lbu::head_bwd_kernel<<<nblk, 256, 0, s>>>(n->db[0], C0, WB(n, hi), n->cfg.out_ch, P, n->dy, n->gB[0], n->work);
-    lbu::head_reduce_kernel<<<n->cfg.out_ch * (C0 + 1), 128, 0, s>>>(n->work, nblk, n->cfg.out_ch, C0, GW(hi), GB(hi));
+    lbnci::launch_pdl(lbu::head_bwd_kernel, dim3(nblk), dim3(256), 0, s, n->db[0], C0, WB(n, hi), n->cfg.out_ch, P, n->dy, n->gB[0], n->work);
+    lbnci::launch_pdl(lbu::head_reduce_kernel, dim3(n->cfg.out_ch * (C0 + 1)), dim3(128), 0, s, n->work, nblk, n->cfg.out_ch, C0, GW(hi), GB(hi));
     n->launches += 2;
   }
   // decoder, finest level first
@@ -709,7 +717,7 @@ lb_status backward_impl(lbu_net* n, int B) {
     LBU_TRY(wgrad(n, k, hin, C1, 1, n->gCat[l], 2 * C, B, H, W, C1, C, n->work, n->work_bytes, s, GW(k), GB(k), C1));
     LBU_TRY(conv(n, nl + k, n->gCat[l], 2 * C, B, H, W, C, 0, WT(n, k), nullptr, 0, n->gU[l], C1, C1, nullptr, 0, s));
     const long long work = (long long)B * Hl(n, l + 1) * Wl(n, l + 1) * (C1 / 8);
-    lbu::upsample_bwd_kernel<<<grid_for(work, 256), 256, 0, s>>>(n->gU[l], hin, n->gB[l + 1], B, Hl(n, l + 1),
+    lbnci::launch_pdl(lbu::upsample_bwd_kernel, dim3(grid_for(work, 256)), dim3(256), 0, s, n->gU[l], hin, n->gB[l + 1], B, Hl(n, l + 1),
                                                                  Wl(n, l + 1), C1);
     ++n->launches;
   }
@@ -723,7 +731,7 @@ lb_status backward_impl(lbu_net* n, int B) {
       gs = C;
     } else {
       const long long work = (long long)B * (H / 2) * (W / 2) * (C / 8);
-      lbu::maxpool_bwd_kernel<<<grid_for(work, 256), 256, 0, s>>>(n->cat[l] + C, 2 * C, n->gPool[l],
+      lbnci::launch_pdl(lbu::maxpool_bwd_kernel, dim3(grid_for(work, 256)), dim3(256), 0, s, n->cat[l] + C, 2 * C, n->gPool[l],
                                                                   n->gCat[l] + C, 2 * C, B, H, W, C);
       ++n->launches;
       g = n->gCat[l] + C;
@@ -747,7 +755,7 @@ lb_status refresh(lbu_net* n) {
   size_t maxn = 0;
   for (auto& l : n->L) maxn = std::max(maxn, (size_t)l.cout * l.taps * l.cin_pad);
   dim3 grid((unsigned)std::min<size_t>((maxn + 255) / 256, 1024), (unsigned)n->L.size());
-  lbu::refresh_weights_kernel<<<grid, 256, 0, n->stream>>>(n->Ldev, n->params, n->wb, n->wt);
+  lbnci::launch_pdl(lbu::refresh_weights_kernel, dim3(grid), dim3(256), 0, n->stream, n->Ldev, n->params, n->wb, n->wt);
   ++n->launches;
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? LB_OK : cuda_fail(n, e, "refresh launch");
@@ -758,9 +766,9 @@ lb_status loss_impl(lbu_net* n, const float* T, const int* idx, int B, const flo
   float lm[8];
   for (int j = 0; j < 8; ++j) lm[j] = (lam && j < n->cfg.out_ch) ? lam[j] : 1.f;
   const int blocks = std::min(n->npartial, grid_for(P, 256));
-  lbu::mse_kernel<<<blocks, 256, 0, n->stream>>>(n->y, T, idx, HW, n->cfg.out_ch, P, lm[0], lm[1], lm[2], lm[3],
+  lbnci::launch_pdl(lbu::mse_kernel, dim3(blocks), dim3(256), 0, n->stream, n->y, T, idx, HW, n->cfg.out_ch, P, lm[0], lm[1], lm[2], lm[3],
                                                  lm[4], lm[5], lm[6], lm[7], n->dy, n->partial);
-  lbu::sum_partials_kernel<<<1, 256, 0, n->stream>>>(n->partial, blocks, 1.0 / P, n->loss);
+  lbnci::launch_pdl(lbu::sum_partials_kernel, dim3(1), dim3(256), 0, n->stream, n->partial, blocks, 1.0 / P, n->loss);
   n->launches += 2;
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? LB_OK : cuda_fail(n, e, "loss launch");
@@ -768,7 +776,7 @@ lb_status loss_impl(lbu_net* n, const float* T, const int* idx, int B, const flo
 
 lb_status pack(lbu_net* n, const float* X, const int* idx, int B) {
   const long long work = (long long)B * n->cfg.H * n->cfg.W * (kInPad / 8);
-  lbu::pack_input_kernel<<<grid_for(work, 256), 256, 0, n->stream>>>(X, idx, B, n->cfg.H * n->cfg.W, n->cfg.in_ch,
+  lbnci::launch_pdl(lbu::pack_input_kernel, dim3(grid_for(work, 256)), dim3(256), 0, n->stream, X, idx, B, n->cfg.H * n->cfg.W, n->cfg.in_ch,
                                                                      kInPad, n->x0);
   ++n->launches;
   cudaError_t e = cudaGetLastError();
@@ -1011,7 +1019,7 @@ lb_status lbu_train_step(lbu_net* n, const float* X, const float* T, const int* 
   ++n->t;
   const float c1 = (float)(1.0 / (1.0 - std::pow((double)n->b1, (double)n->t)));
   const float c2 = (float)(1.0 / (1.0 - std::pow((double)n->b2, (double)n->t)));
-  lbu::adam_kernel<<<grid_for(n->nparams, 256), 256, 0, n->stream>>>(n->params, n->grads, n->m, n->v, n->nparams,
+  lbnci::launch_pdl(lbu::adam_kernel, dim3(grid_for(n->nparams, 256)), dim3(256), 0, n->stream, n->params, n->grads, n->m, n->v, n->nparams,
                                                                     lr, n->b1, n->b2, n->eps, c1, c2);
   ++n->launches;
   LBU_CUDA(n, cudaGetLastError());

@@ -239,6 +239,14 @@ conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   tc::fence_after_sync();
   const unsigned tmem = t.tmem;
   const bool aligned = t.fail == 0;
+  auto weights = [&](int i) {
+    const int s = i % ST;
+    lbnci::mbar_expect_tx(&t.bar_full[s], BBYTES);
+    lbnci::tma_load_2d(sB + s * BBYTES, &map_w, i * CH, n0, &t.bar_full[s]);
+  };
+  if (aligned && tid == 0)  // the first weights, which no kernel of the chain writes, ahead of the wait
+    for (int i = 0; i < ST; ++i) weights(i);
+  lbnci::pdl_enter();
 
   if (!aligned) {
     // nothing was started
@@ -247,15 +255,14 @@ conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       lbnci::mbar_expect_tx(&t.bar_a, (unsigned)(a.nchunk * ROWB * (a.TW + 2) * (a.TH + 2)));
       for (int k = 0; k < a.nchunk; ++k)
         lbnci::tma_load_4d(sA + k * a.a_stride, &map_x, k * CH, x0 - 1, y0 - 1, b, &t.bar_a);
-      int issued = 0;
-      for (int i = 0; i < ni; ++i) {
+      int issued = ST;
+      for (int i = ST; i < ni; ++i) {
         const int s = i % ST, u = i / ST;
-        if (u > 0 && !lbnci::mbar_wait(&t.bar_empty[s], (unsigned)((u - 1) & 1))) {
+        if (!lbnci::mbar_wait(&t.bar_empty[s], (unsigned)((u - 1) & 1))) {
           atomicOr(&t.fail, 1);
           break;
         }
-        lbnci::mbar_expect_tx(&t.bar_full[s], BBYTES);
-        lbnci::tma_load_2d(sB + s * BBYTES, &map_w, i * CH, n0, &t.bar_full[s]);
+        weights(i);
         issued = i + 1;
       }
       // before the CTA may end: every copy has landed (bounded; each was waited for by the
@@ -551,17 +558,21 @@ conv3x3_rows_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
   tc::fence_after_sync();
   const unsigned tmem = t.tmem;
   const bool aligned = t.fail == 0;
+  if (aligned && tid == 0) {
+    // the weights (dx, chunk, dy = +1, 0, -1), which no kernel of the chain writes, ahead of the wait
+    lbnci::mbar_expect_tx(&t.bar_w, (unsigned)(9 * a.nchunk * WB));
+    for (int dxi = 0; dxi < 3; ++dxi)
+      for (int k = 0; k < a.nchunk; ++k)
+        for (int j = 0; j < 3; ++j)
+          lbnci::tma_load_2d(sW + ((dxi * a.nchunk + k) * 3 + j) * WB, &map_w,
+                             (((2 - j) * 3 + dxi) * a.nchunk + k) * CH, n0, &t.bar_w);
+  }
+  lbnci::pdl_enter();
 
   if (!aligned) {
     // nothing was started
   } else if (warp == 0) {
-    if (lane == 0) {  // copies: the weights (dx, chunk, dy = +1, 0, -1), then the rows
-      lbnci::mbar_expect_tx(&t.bar_w, (unsigned)(9 * a.nchunk * WB));
-      for (int dxi = 0; dxi < 3; ++dxi)
-        for (int k = 0; k < a.nchunk; ++k)
-          for (int j = 0; j < 3; ++j)
-            lbnci::tma_load_2d(sW + ((dxi * a.nchunk + k) * 3 + j) * WB, &map_w,
-                               (((2 - j) * 3 + dxi) * a.nchunk + k) * CH, n0, &t.bar_w);
+    if (lane == 0) {  // copies of the rows
       int issued = 0;
       for (int i = 0; i < nin; ++i) {
         const int s = i % a.nrow, u = i / a.nrow;
@@ -820,6 +831,7 @@ conv3x3_wgrad_tma_kernel(const __grid_constant__ WgradMaps maps, WgradTma a, int
   tc::fence_after_sync();
   const unsigned tmem = t.tmem;
   const bool aligned = t.fail == 0;
+  lbnci::pdl_enter();
   auto origin = [&](int i, int& b, int& y0, int& x0) {
     const int tt = t0 + i;
     x0 = (tt % a.tiles_x) * a.TW;
@@ -1033,6 +1045,7 @@ __global__ void __launch_bounds__(256) wgrad_reduce_tma_kernel(const float* __re
                                                                int Cin, int cin_true, int up, int S, int wblocks,
                                                                float* __restrict__ dw, float* __restrict__ db) {
   __shared__ float4 s[256];
+  lbnci::pdl_enter();
   if ((int)blockIdx.x >= wblocks) {  // 32 output channels of the bias, eight threads to each
     float* sb = reinterpret_cast<float*>(s);
     const int o = ((int)blockIdx.x - wblocks) * 32 + (threadIdx.x & 31), share = threadIdx.x >> 5;

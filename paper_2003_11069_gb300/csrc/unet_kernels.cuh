@@ -15,6 +15,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "lb_launch.h"
+
 namespace lbu {
 
 using bf16 = __nv_bfloat16;
@@ -331,6 +333,7 @@ union V8 {
 // FP32 X[n][HW][cin] (samples idx[b], or b) -> BF16 [b][HW][cpad], zero padded
 __global__ void pack_input_kernel(const float* __restrict__ X, const int* __restrict__ idx, int B, int HW, int cin,
                                   int cpad, bf16* __restrict__ out) {
+  lbnci::pdl_enter();
   const int groups = cpad / 8;
   const long total = (long)B * HW * groups;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
@@ -356,6 +359,7 @@ __global__ void pack_input_kernel(const float* __restrict__ X, const int* __rest
 // Ties go to the first element in window order (0,0), (0,1), (1,0), (1,1).
 __global__ void maxpool_kernel(const bf16* __restrict__ in, int is, int B, int H, int W, int C,
                                bf16* __restrict__ out) {
+  lbnci::pdl_enter();
   const int h = H / 2, w = W / 2, groups = C / 8;
   const long total = (long)B * h * w * groups;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
@@ -390,6 +394,7 @@ __global__ void maxpool_kernel(const bf16* __restrict__ in, int is, int B, int H
 // g[q] = bf16(g[q] + (q is the window's argmax ? dp : 0)) where act[q] > 0, else 0.
 __global__ void maxpool_bwd_kernel(const bf16* __restrict__ act, int as, const bf16* __restrict__ dp, bf16* g, int gs,
                                    int B, int H, int W, int C) {
+  lbnci::pdl_enter();
   const int h = H / 2, w = W / 2, groups = C / 8;
   const long total = (long)B * h * w * groups;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
@@ -456,6 +461,7 @@ __global__ void maxpool_bwd_kernel(const bf16* __restrict__ act, int as, const b
 // du [B][2h][2w][C], act and out [B][h][w][C], all contiguous.
 __global__ void upsample_bwd_kernel(const bf16* __restrict__ du, const bf16* __restrict__ act, bf16* __restrict__ out,
                                     int B, int h, int w, int C) {
+  lbnci::pdl_enter();
   const int groups = C / 8, H = 2 * h, W = 2 * w;
   const long total = (long)B * h * w * groups;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < total; i += (long)gridDim.x * blockDim.x) {
@@ -492,6 +498,7 @@ constexpr int kMaxOut = 8, kMaxHeadIn = 256;
 // y[p][j] = b[j] + sum_c wh[j][c] x[p][c]; x BF16 [P][C], wh BF16 [nout][C], y FP32
 __global__ void head_fwd_kernel(const bf16* __restrict__ x, int C, const bf16* __restrict__ wh,
                                 const float* __restrict__ bh, int nout, int P, float* __restrict__ y) {
+  lbnci::pdl_enter();
   __shared__ float sw[kMaxOut * kMaxHeadIn];
   for (int i = threadIdx.x; i < nout * C; i += blockDim.x) sw[i] = __bfloat162float(wh[i]);
   __syncthreads();
@@ -522,6 +529,7 @@ __global__ void head_fwd_kernel(const bf16* __restrict__ x, int C, const bf16* _
 __global__ void mse_kernel(const float* __restrict__ y, const float* __restrict__ T, const int* __restrict__ idx,
                            int HW, int nout, int P, float lam0, float lam1, float lam2, float lam3, float lam4,
                            float lam5, float lam6, float lam7, float* __restrict__ dy, double* __restrict__ partial) {
+  lbnci::pdl_enter();
   const float lam[8] = {lam0, lam1, lam2, lam3, lam4, lam5, lam6, lam7};
   double s = 0.0;
   const float scale = 2.f / (float)P;
@@ -548,6 +556,7 @@ __global__ void mse_kernel(const float* __restrict__ y, const float* __restrict_
 // One block: thread t adds partials t, t + 256, ..., then a fixed tree.
 __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restrict__ partial, int n, double scale,
                                                            double* __restrict__ out) {
+  lbnci::pdl_enter();
   __shared__ double s[256];
   double v = 0.0;
 #pragma unroll 4
@@ -572,6 +581,7 @@ constexpr int kHeadPix = 512;
 __global__ void __launch_bounds__(256) head_bwd_kernel(const bf16* __restrict__ x, int C, const bf16* __restrict__ wh,
                                                        int nout, int P, const float* __restrict__ dy,
                                                        bf16* __restrict__ dx, float* __restrict__ part) {
+  lbnci::pdl_enter();
   __shared__ float red[8][kMaxOut + 1][33];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int p0 = blockIdx.x * kHeadPix, p1 = min(p0 + kHeadPix, P);
@@ -621,6 +631,7 @@ __global__ void __launch_bounds__(256) head_bwd_kernel(const bf16* __restrict__ 
 // + 128, ..., then a fixed tree): dW [nout][C] then db [nout].
 __global__ void __launch_bounds__(128) head_reduce_kernel(const float* __restrict__ part, int nblk, int nout, int C,
                                                           float* __restrict__ dw, float* __restrict__ db) {
+  lbnci::pdl_enter();
   __shared__ float s[128];
   const int nw = nout * (C + 1), o = blockIdx.x;
   float v = 0.f;
@@ -650,6 +661,7 @@ struct LayerDev {
 // Master FP32 weights -> BF16 kernel layouts (padded input channels are zero).
 __global__ void refresh_weights_kernel(const LayerDev* __restrict__ L, const float* __restrict__ master,
                                        bf16* __restrict__ wb, bf16* __restrict__ wt) {
+  lbnci::pdl_enter();
   const LayerDev d = L[blockIdx.y];
   const long n = (long)d.cout * d.taps * d.cin_pad;
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
@@ -665,6 +677,7 @@ __global__ void refresh_weights_kernel(const LayerDev* __restrict__ L, const flo
 __global__ void adam_kernel(float* __restrict__ theta, const float* __restrict__ g, float* __restrict__ m,
                             float* __restrict__ v, long long n, float lr, float b1, float b2, float eps, float c1,
                             float c2) {
+  lbnci::pdl_enter();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi;
