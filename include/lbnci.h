@@ -189,10 +189,11 @@ const char* lb_last_error(const lb_sim* sim);
 long long lb_kernel_launches(const lb_sim* sim);
 
 /* Which kernel lb_step runs for this sim (no paper counterpart; reporting only):
- *   LB_PATH_FUSED2D  one-pass fused D2Q9 kernel (FP32 and FP16-dev when nx % 4 != 0 or
- *                    LBNCI_FUSED=classic is set in the environment; FP64 with the
- *                    exact-difference forcing) or, for FP64 with Guo forcing, moments,
- *                    normals and collision as passes over the sites,
+ *   LB_PATH_FUSED2D  moments, normals and collision as passes over the sites (FP64 with Guo
+ *                    forcing, FP32 and FP16-dev when nx % 4 != 0) or, where a workspace has no
+ *                    room for their scratch, for FP64 with the exact-difference forcing, or
+ *                    when LBNCI_FUSED=classic is set in the environment, the one-pass fused
+ *                    D2Q9 kernel,
  *   LB_PATH_TMA2D    persistent TMA-fed D2Q9 kernel (FP32 and FP16-dev storage),
  *   LB_PATH_D3Q27    D3Q27 step on the two-population state: for FP64, and for FP32 and
  *                    FP16-dev when nx % 32 != 0 or ny % 8 != 0, moments, normals and

@@ -214,13 +214,17 @@ lb_status validate(const lb_config* c, HostParams* p, Layout* lay, long long* nb
   p->carry3d = 0;
   p->stream3d = c->lattice == LB_D3Q27 && c->precision != LB_FP64 && (c->wall_z || c->nz >= 2) ? 1 : 0;
   // FP64 steps with Guo forcing run the per-site passes of lb_sites.cuh at every size: the
-  // FP64 pipe bounds both ways, and the passes recompute nothing over halos (128 x 128: 29 us
+  // FP64 pipe bounds both ways, and the passes recompute nothing over halos (128 x 128: 23 us
   // per step against 117 us with the fused kernel, whose 32 tiles also leave most
   // multiprocessors idle; 128 x 48 x 48 duct: 0.64 ms against 1.40 ms with the march).
+  // So do D2Q9 FP32 and FP16-dev steps of lattices the TMA maps cannot describe (nx % 4 != 0):
+  // faster than the fused kernel at every size measured, 37 x 19 to 8190 x 1024 (1030 x 131,
+  // exact difference forcing: 12.7 us against 16.4 us; figures at site_collide2d_kernel).
   // An environment variable that names another kernel selects that one.
   bool sites = c->precision == LB_FP64 && c->forcing == 0;
   if (c->lattice == LB_D3Q27) sites = sites && !std::getenv("LBNCI_D3_KERNEL");
-  else sites = sites && !std::getenv("LBNCI_FUSED_SPT") && !std::getenv("LBNCI_FUSED");
+  else sites = (sites || (c->precision != LB_FP64 && c->nx % 4 != 0)) && !std::getenv("LBNCI_FUSED_SPT") &&
+               !std::getenv("LBNCI_FUSED");
   if (const char* e = std::getenv("LBNCI_D3_KERNEL")) {
     if (std::strcmp(e, "march") == 0 || std::strcmp(e, "tiled") == 0) p->stream3d = 0;
     if (std::strcmp(e, "carry") == 0 && col_ok) { p->carry3d = 1; p->stream3d = 0; }

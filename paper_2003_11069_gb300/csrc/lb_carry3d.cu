@@ -246,8 +246,8 @@ namespace {
 template <typename RD, bool TOTALS, typename WR>
 cudaError_t launch_collide3t(RD rd, WR wr, const void* rho12, const void* ng, const StepT<float>& p, dim3 grid,
                              cudaStream_t s) {
-  collide3t_kernel<RD, TOTALS, WR><<<grid, dim3(32, 8), 0, s>>>(rd, wr, (const float2*)rho12, (const float4*)ng, p);
-  return cudaGetLastError();
+  return launch_pdl(collide3t_kernel<RD, TOTALS, WR>, grid, dim3(32, 8), 0, s, rd, wr, (const float2*)rho12,
+                    (const float4*)ng, p);
 }
 }  // namespace
 
@@ -266,24 +266,31 @@ cudaError_t stream3d_step(const void* fa, void* fb, void* psi, void* ng, void* r
   // blocks of 256 consecutive sites; the total forms: the recolouring coefficients, about
   // two thirds of whose sectors hit L1); the two-population FP32 state has none and keeps
   // the flat kernel (the same time)
+  // Steps from one total form to the next are chained programmatically (384 x 96 x 96 FP32:
+  // 305 -> 300 us, 512 x 128 x 128 FP16-dev: 683 -> 681 us); those on pairs keep plain
+  // launches (a 150 x 66 x 66 lattice: 106 us, 113 us when chained, the next pass's blocks
+  // taking their places on the multiprocessors unevenly).
+  const dim3 b3(32, 8);
+  cudaError_t e;
   if (totals_in && h.half) {
-    moments3_kernel<TotalRecolHalf><<<grid, dim3(32, 8), 0, s>>>(TotalRecolHalf::reader(fa, N, r0), (float*)psi,
-                                                                 r12, p);
+    e = launch_pdl(moments3_kernel<TotalRecolHalf>, grid, b3, 0, s, TotalRecolHalf::reader(fa, N, r0), (float*)psi, r12,
+                   p);
   } else if (totals_in) {
-    moments3_kernel<TotalRecol><<<grid, dim3(32, 8), 0, s>>>(TotalRecol::reader(fa, N), (float*)psi, r12, p);
+    e = launch_pdl(moments3_kernel<TotalRecol>, grid, b3, 0, s, TotalRecol::reader(fa, N), (float*)psi, r12, p);
   } else if (h.half) {
-    moments3_kernel<HalfDev<1>><<<grid, dim3(32, 8), 0, s>>>(HalfDev<1>::reader(fa, N), (float*)psi, r12, p);
+    moments3_kernel<HalfDev<1>><<<grid, b3, 0, s>>>(HalfDev<1>::reader(fa, N), (float*)psi, r12, p);
+    e = cudaGetLastError();
   } else if (totals_out) {
-    moments3_kernel<Plain<1, float>><<<grid, dim3(32, 8), 0, s>>>(Plain<1, float>::reader(fa, N), (float*)psi, r12,
-                                                                  p);
+    moments3_kernel<Plain<1, float>><<<grid, b3, 0, s>>>(Plain<1, float>::reader(fa, N), (float*)psi, r12, p);
+    e = cudaGetLastError();
   } else {
     const unsigned nb = (unsigned)((p.N + 255) / 256);
     moments_kernel<1, Plain<1, float>><<<nb, 256, 0, s>>>(Plain<1, float>::reader(fa, N), (float*)psi, p);
+    e = cudaGetLastError();
   }
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   ++*nk;
-  e = launch_normals3d<float>((const float*)psi, (Quad<float>*)ng, p, s);
+  e = launch_normals3d<float>((const float*)psi, (Quad<float>*)ng, p, s, totals_in);
   if (e != cudaSuccess) return e;
   ++*nk;
   if (totals_out && h.half) {

@@ -792,6 +792,7 @@ __device__ __forceinline__ void prefetch_state(const RD&, const StepT<float>&) {
 template <typename ST>
 __global__ void __launch_bounds__(256) moments3_kernel(typename ST::Reader f, float* __restrict__ psi,
                                                        float2* __restrict__ rho12, StepT<float> p) {
+  pdl_enter();
   const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y, z = blockIdx.z;
   prefetch_state(f, p);
   if (x >= p.nx || y >= p.ny) return;
@@ -1244,6 +1245,7 @@ __device__ __forceinline__ void collide_totals_dev(const float d[27], float rho1
 template <typename RD, bool TOTALS, typename WR>
 __global__ void __launch_bounds__(256, 4) collide3t_kernel(RD f, WR fout, const float2* __restrict__ rho12,
                                                            const float4* __restrict__ ng, StepT<float> p) {
+  pdl_enter();
   const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y, z = blockIdx.z;
   const unsigned site = (unsigned)x + (unsigned)p.nx * ((unsigned)y + (unsigned)p.ny * (unsigned)z);
   if constexpr (std::is_same<WR, TotalRecolHalf::Writer>::value)

@@ -157,6 +157,9 @@ cudaError_t l_step(const void* fa, void* fb, void* psi, const HostParams& h, cud
   if constexpr (std::is_same<T, double>::value) {
     if (h.sites && !p.edm) return site_step64<LAT>(fa, fb, (T*)psi, h.sites, h, p, nk, s);
   }
+  if constexpr (LAT == 0 && std::is_same<T, float>::value) {
+    if (h.sites) return site_step2d<ST>(fa, fb, (T*)psi, h.sites, h, p, nk, s);
+  }
   if constexpr (LAT == 0) {
     *nk = 1;
     return h.spt == 4 ? launch_fused2d<ST, 4>(fa, fb, p, s) : launch_fused2d<ST, 2>(fa, fb, p, s);
@@ -260,7 +263,7 @@ const Launchers* table() {
   using T = typename ST::Compute;
   static const Launchers L = {ST::bytes, sizeof(T),
                               [](size_t N) { return site_scratch_bytes<LAT, T>(N, true); },
-                              [](size_t N) { return sizeof(T) == 8 ? site_scratch_bytes<LAT, T>(N, false) : 0; },
+                              [](size_t N) { return sizeof(T) == 8 || LAT == 0 ? site_scratch_bytes<LAT, T>(N, false) : 0; },
                               l_init<LAT, ST>, l_step<LAT, ST>,
                               l_fields<LAT, ST>, l_decode<LAT, ST>, l_encode<LAT, ST>,
                               sizeof(BatchMember<typename ST::Compute>), l_batch_fill<ST>, l_batch_tiles,

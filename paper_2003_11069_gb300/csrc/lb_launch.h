@@ -38,12 +38,11 @@ cudaError_t allow_smem(K kernel, size_t bytes, SmemAllowance& a) {
 }
 
 // Programmatic dependent launch of a chain of kernels on one stream: a launch may be
-// scheduled, and its blocks may start, as soon as every block of the kernel before it has
-// started (pdl_begin) or ended. pdl_begin waits for that kernel's completion (its writes
-// visible) before anything of the chain's memory is touched, so results and order are those
-// of plain launches; what overlaps is the launch latency and the last blocks' tail. Every
-// kernel launched this way begins with pdl_begin or pdl_enter (which do nothing after a plain
-// launch).
+// scheduled, and its blocks may start, once every block of the kernel before it has passed
+// pdl_enter or ended. pdl_enter waits for that kernel's completion (its writes visible) before
+// anything of the chain's memory is touched, so results and order are those of plain
+// launches; what overlaps is the launch latency and the last blocks' tail. Every kernel
+// launched this way begins with pdl_enter, which does nothing after a plain launch.
 template <typename... P, typename... A>
 cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -59,15 +58,14 @@ cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cuda
   return cudaLaunchKernelEx(&cfg, k, std::forward<A>(args)...);
 }
 #ifdef __CUDACC__
-__device__ __forceinline__ void pdl_begin() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-// The same with the next launch released only after the wait: when a kernel's blocks start,
-// every kernel before its predecessor has completed. What a block does before pdl_enter may
-// therefore read what the predecessor does not write (a network's weights), and blocks that
-// hold tensor memory at the wait never keep it from a block that has yet to start. Measured
-// on the U-Net's chains of 5 to 60 us kernels (setup, barrier initialisation, tensor-memory
+// The next launch is released only after the wait: when a kernel's blocks start, every kernel
+// before its predecessor has completed, and blocks that wait take room from one kernel at
+// most. (Released before the wait, the waiting blocks unbalanced the FP64 pipes of a 128 x
+// 128 lattice, 46 us per step against 29 us with plain launches and 23 us like this; a 1030 x
+// 131 FP32 step 12.2 us against 16.5 us and 10.4 us.) What a block does before pdl_enter may
+// read what the predecessor does not write (a network's weights), and blocks that hold
+// tensor memory at the wait never keep it from a block that has yet to start. Measured on
+// the U-Net's chains of 5 to 60 us kernels (setup, barrier initialisation, tensor-memory
 // allocation and the first weights overlap the kernel before): batch-8 forward of 23 launches
 // 289 -> 239 us, batch-32 training step of 86 launches 1771 -> 1587 us.
 __device__ __forceinline__ void pdl_enter() {
@@ -92,8 +90,8 @@ struct HostParams {
   int c3_zseg;    // planes per z segment of their collision kernel
   int stream3d;   // 1: D3Q27 steps run moments, normals and a streaming collision
   int totals;     // 1: streaming steps with Guo forcing store the total + recolouring form
-  void* sites;    // device scratch of the FP64 step's per-site passes (null: the kernels that
-                  // recompute over halos, lb_fused2d.cuh and lb_march3d.cuh)
+  void* sites;    // device scratch of a step of per-site passes (lb_sites.cuh; null: the kernels
+                  // that recompute over halos, lb_fused2d.cuh and lb_march3d.cuh)
   float rho_ref;  // reference density rho_0 of the FP16 totals (f*_i = w_i rho_0 + d_i)
   unsigned* seedw;  // device: two dither-seed words of the FP16-deviation stores
   int parity;       // state buffer the next step reads (0: the one the sim was created with)

@@ -9,12 +9,15 @@
 //                         the block sums of the observables
 //   site_collide64_kernel the near-contact ray, the totals f_i^1 + f_i^2 and the FP64
 //                         collision (Guo forcing)
+//   site_collide2d_kernel the near-contact ray and the D2Q9 collision in FP32 arithmetic
+//                         (FP32 and FP16-deviation storage, either forcing)
 //
 // Measured on GB300 (lb_observables with psi and u on the device, before -> after): FP16-dev
 // duct 512 x 128 x 128 3.8 -> 0.82 ms, FP16-dev channel 8192 x 1024 1.40 -> 0.43 ms. The
 // kernels it replaces there (psi, then tiled_kernel) staged 27.6 psi cells per site and
 // spent 100 additions per site of the narrow FP64 pipe on their block sums. FP64 steps: a 128
-// x 128 box 117 -> 29 us, a 128 x 48 x 48 duct 1.40 -> 0.64 ms.
+// x 128 box 117 -> 23 us, a 128 x 48 x 48 duct 1.40 -> 0.64 ms. FP32 steps with the exact
+// difference forcing of a 1030 x 131 channel: 16.4 -> 12.7 us.
 //
 // Every quantity is computed once per site, by the expressions (and in the order) of the
 // kernels that recompute it over halos (lb_fused2d.cuh, lb_march3d.cuh, tiled_kernel): the
@@ -77,7 +80,7 @@ __global__ void __launch_bounds__(256) site_moments_kernel(typename ST::Reader f
                                                            SiteScratch<typename ST::Compute> sc,
                                                            StepT<typename ST::Compute> p) {
   using T = typename ST::Compute;
-  if (WITHJ) pdl_begin();
+  pdl_enter();
   const SiteIdx s = site_of(p);
   if (s.x >= p.nx || s.y >= p.ny) return;
   T fin[2][Lattice<LAT>::Q];
@@ -156,7 +159,7 @@ __device__ __forceinline__ T unit_site(const T g[3], T n[3]) {
 template <int LAT, typename T>
 __global__ void __launch_bounds__(256) site_normals_kernel(const T* __restrict__ psi, Quad<T>* __restrict__ ng,
                                                            StepT<T> p) {
-  pdl_begin();
+  pdl_enter();
   const SiteIdx s = site_of(p);
   if (s.x >= p.nx || s.y >= p.ny) return;
   T g[3], n[3];
@@ -193,7 +196,7 @@ __global__ void __launch_bounds__(256) normals3d_kernel(const T* __restrict__ ps
                                                         StepT<T> p) {
   constexpr int RX = 34, RXY = RX * 10, PER = (RXY + 255) / 256;
   __shared__ T s_psi[4 * RXY];
-  pdl_begin();
+  pdl_enter();
   const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 8, z0 = blockIdx.z * kN3Z;
   const int nx = p.nx, ny = p.ny, nz = p.nz;
   const int tid = threadIdx.x + 32 * threadIdx.y;
@@ -253,10 +256,10 @@ __global__ void __launch_bounds__(256) normals3d_kernel(const T* __restrict__ ps
 }
 
 template <typename T, bool FIELDS = false>
-cudaError_t launch_normals3d(const T* psi, Quad<T>* ng, const StepT<T>& p, cudaStream_t s) {
+cudaError_t launch_normals3d(const T* psi, Quad<T>* ng, const StepT<T>& p, cudaStream_t s, bool chained = true) {
   const dim3 grid((unsigned)((p.nx + 31) / 32), (unsigned)((p.ny + 7) / 8), (unsigned)((p.nz + kN3Z - 1) / kN3Z));
-  if constexpr (FIELDS) return launch_pdl(normals3d_kernel<T, true>, grid, dim3(32, 8), 0, s, psi, ng, p);
-  normals3d_kernel<T, false><<<grid, dim3(32, 8), 0, s>>>(psi, ng, p);
+  if (chained) return launch_pdl(normals3d_kernel<T, FIELDS>, grid, dim3(32, 8), 0, s, psi, ng, p);
+  normals3d_kernel<T, FIELDS><<<grid, dim3(32, 8), 0, s>>>(psi, ng, p);
   return cudaGetLastError();
 }
 
@@ -328,7 +331,7 @@ template <int LAT, typename T>
 __global__ void __launch_bounds__(kFieldThreads) site_fields_kernel(const T* __restrict__ psi, SiteScratch<T> sc,
                                                                     StepT<T> p, FieldOut fo) {
   constexpr int D = Lattice<LAT>::D;
-  pdl_begin();
+  pdl_enter();
   const unsigned N = (unsigned)p.N, nx = (unsigned)p.nx, ny = (unsigned)p.ny;
   double m1 = 0.0, m2 = 0.0, P[3] = {0.0, 0.0, 0.0}, qd = 0.0;
   unsigned nif = 0, nnci = 0, nbad = 0;
@@ -523,6 +526,7 @@ __global__ void __launch_bounds__(256) site_collide64_kernel(typename Plain<LAT,
                                                              SiteScratch<double> sc, StepT<double> p) {
   constexpr int Q = Lattice<LAT>::Q;
   constexpr int D = Lattice<LAT>::D;
+  pdl_enter();
   const SiteIdx s = site_of(p);
   if (s.x >= p.nx || s.y >= p.ny) return;
   double fin[2][Q];
@@ -556,6 +560,46 @@ __global__ void __launch_bounds__(256) site_collide64_kernel(typename Plain<LAT,
   collide64<LAT>(t, r.x, r.y, u, F, v.w, m, p, fout, s.i);
 }
 
+// ------------------------------------------------------------------ FP32 collision, D2Q9
+// One site of the D2Q9 step in FP32 arithmetic (FP32 and FP16-deviation storage, either
+// forcing): the near-contact ray over the stored (n, |grad psi|), then the collision of
+// fused2d_kernel by the same expressions. Against that kernel, whose 32 x 16 tiles pull twice
+// as many sites again for their halos and run three barriers one after the other, the passes
+// read the populations twice, from L2 on lattices that fit there, and wait on each other's
+// launches, which the chain hides (us per step, passes against fused): 37 x 19 7.2 / 9.8, 515 x
+// 131 9.1 / 10.3, 1030 x 131 10.4 / 13.6, 2050 x 515 52 / 59, 8190 x 1024 374 / 407; FP16
+// deviations 1030 x 131 11.8 / 14.4, 8190 x 1024 355 / 477.
+template <typename ST, bool EDM>
+__global__ void __launch_bounds__(256) site_collide2d_kernel(typename ST::Reader f, typename ST::Writer fout,
+                                                             SiteScratch<float> sc, StepT<float> p) {
+  pdl_enter();
+  const SiteIdx s = site_of(p);
+  if constexpr (ST::kHalf)
+    fout.seed = step_seed(p, p.parity, blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0);
+  if (s.x >= p.nx || s.y >= p.ny) return;
+  float fin[2][9];
+  pull_any<0, float>(f, s.x, s.y, 0, p, fin);
+  const Quad<float> v = sc.ng[s.i];
+  const Pair<float> r = sc.rho[s.i];
+  const float rho = r.x + r.y;
+  const int hit = ray_site<0, float>(sc.ng, v, s, p);
+  float frep[3] = {0.f, 0.f, 0.f};
+  if (hit) {
+    const float A = ah_of(p, hit);
+    const float deltaI = 0.5f * v.w;
+    frep[0] = -A * v.x * deltaI;
+    frep[1] = -A * v.y * deltaI;
+  }
+  float j[3], F[3], u[3];
+  momentum<0, float>(fin, j);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) F[a] = add_rn(p.G[a], frep[a]);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) u[a] = M<float>::div(j[a] + 0.5f * F[a], rho);
+  const float m[3] = {-v.x, -v.y, 0.f};
+  collide_store<0, float, typename ST::Writer, EDM>(fin, r.x, r.y, j, u, F, v.w, m, p, fout, (int)s.i);
+}
+
 // ------------------------------------------------------------------ launches
 // Rows of a block: eight (256 sites) where the lattice then still gives every multiprocessor
 // several blocks, fewer on small lattices, so that their few warps spread over all of them
@@ -586,7 +630,7 @@ cudaError_t launch_site_normals(const T* psi, Quad<T>* ng, const HostParams& h, 
   return launch_pdl(site_normals_kernel<LAT, T>, site_grid(h, b), b, 0, s, psi, ng, p);
 }
 
-// The FP64 step with Guo forcing: moments, normals, collision.
+// The FP64 step with Guo forcing: moments, normals, collision, each launched programmatically.
 template <int LAT>
 cudaError_t site_step64(const void* fa, void* fb, double* psi, void* scratch, const HostParams& h,
                         const StepT<double>& p, int* nk, cudaStream_t s) {
@@ -594,18 +638,31 @@ cudaError_t site_step64(const void* fa, void* fb, double* psi, void* scratch, co
   const SiteScratch<double> sc = site_scratch<LAT, double>(scratch, (size_t)p.N);
   const dim3 b = site_block<double>(h), g = site_grid(h, b);
   const unsigned N = (unsigned)p.N;
-  site_moments_kernel<LAT, ST, false><<<g, b, 0, s>>>(ST::reader(fa, N), psi, sc, p);
-  site_normals_kernel<LAT, double><<<g, b, 0, s>>>(psi, sc.ng, p);
-  site_collide64_kernel<LAT><<<g, b, 0, s>>>(ST::reader(fa, N), ST::writer(fb, N), sc, p);
   *nk = 3;
-  return cudaGetLastError();
+  cudaError_t e = launch_pdl(site_moments_kernel<LAT, ST, false>, g, b, 0, s, ST::reader(fa, N), psi, sc, p);
+  if (e == cudaSuccess) e = launch_pdl(site_normals_kernel<LAT, double>, g, b, 0, s, (const double*)psi, sc.ng, p);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(site_collide64_kernel<LAT>, g, b, 0, s, ST::reader(fa, N), ST::writer(fb, N), sc, p);
+}
+
+// The D2Q9 step in FP32 arithmetic: moments, normals, collision, each launched programmatically.
+template <typename ST>
+cudaError_t site_step2d(const void* fa, void* fb, float* psi, void* scratch, const HostParams& h,
+                        const StepT<float>& p, int* nk, cudaStream_t s) {
+  const SiteScratch<float> sc = site_scratch<0, float>(scratch, (size_t)p.N);
+  const dim3 b = site_block<float>(h), g = site_grid(h, b);
+  const unsigned N = (unsigned)p.N;
+  *nk = 3;
+  cudaError_t e = launch_pdl(site_moments_kernel<0, ST, false>, g, b, 0, s, ST::reader(fa, N), psi, sc, p);
+  if (e == cudaSuccess) e = launch_pdl(site_normals_kernel<0, float>, g, b, 0, s, (const float*)psi, sc.ng, p);
+  if (e != cudaSuccess) return e;
+  return p.edm ? launch_pdl(site_collide2d_kernel<ST, true>, g, b, 0, s, ST::reader(fa, N), ST::writer(fb, N), sc, p)
+               : launch_pdl(site_collide2d_kernel<ST, false>, g, b, 0, s, ST::reader(fa, N), ST::writer(fb, N), sc, p);
 }
 
 // The observables and fields of a state: three passes, launched programmatically: on a small
-// lattice the launches are most of the time. (The step's passes are launched plainly: blocks
-// of the next pass that wait on an SM unbalance the FP64 pipes of a 128 x 128 lattice, 46
-// us per step instead of 29, and cost the 512 x 128 x 128 FP16-dev duct 4%.) ng is filled by `normals` (the
-// lattice's own normals pass). rows: partial sums the caller has room for; *used: written.
+// lattice the launches are most of the time. ng is filled by `normals` (the lattice's own
+// normals pass). rows: partial sums the caller has room for; *used: written.
 template <int LAT, typename ST, typename Normals>
 cudaError_t site_fields(typename ST::Reader f, typename ST::Compute* psi, void* scratch, const HostParams& h,
                         const StepT<typename ST::Compute>& p, const FieldOut& fo, long long rows, long long* used,

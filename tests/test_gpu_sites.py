@@ -153,3 +153,33 @@ def test_fields_report_bad_sites_as_before():
                                                allow_numeric=True)
             assert o["n_bad"] == ref["n_bad"] >= 3
             assert o["n_interface"] == ref["n_interface"] and o["n_nci"] == ref["n_nci"]
+
+
+@pytest.mark.parametrize("precision", [lbnci.LB_FP32, lbnci.LB_FP16DEV])
+@pytest.mark.parametrize("nx,ny,wall", [(1, 1, 0), (3, 2, 1), (5, 9, 0), (33, 8, 1), (31, 40, 0), (130, 67, 1),
+                                        (1030, 131, 1)])
+def test_ragged_2d_passes_equal_the_one_pass_kernel(precision, nx, ny, wall, monkeypatch):
+    """Bitwise, for both forcings, several rays and with the scratch or (the documented workspace)
+    without: the passes evaluate the expressions of the fused D2Q9 kernel on every site."""
+    f = torch.from_numpy(_state(lbnci.LB_D2Q9, nx, ny, 1, 7)).cuda()  # (a single site cannot be staged)
+    for forcing in (lbnci.LB_FORCE_GUO, lbnci.LB_FORCE_EDM_DISPERSED):
+        for A_h, h_max in ((0.05, 4.0), (0.05, 2.5), (0.0, 4.0)):
+            cfg = _cfg(lbnci.LB_D2Q9, nx, ny, 1, (wall, 0), precision, A_h, h_max)
+            cfg.forcing = forcing
+            out = {}
+            for mode in ("passes", "fused", "documented"):
+                monkeypatch.delenv("LBNCI_FUSED_SPT", raising=False)
+                monkeypatch.delenv("LBNCI_FUSED", raising=False)
+                if mode == "fused":
+                    monkeypatch.setenv("LBNCI_FUSED", "classic")
+                cfg.workspace, cfg.workspace_bytes = None, 0
+                with lbnci.Sim(cfg, workspace="torch" if mode == "documented" else None) as sim:
+                    lbnci.lb_set_populations(sim.h, f)
+                    before = sim.launches()
+                    sim.step(3)
+                    assert sim.launches() - before == (9 if mode == "passes" else 3)
+                    assert sim.step_path() == lbnci.LB_PATH_FUSED2D
+                    out[mode] = torch.empty_like(f)
+                    lbnci.lb_get_populations(sim.h, out[mode])
+            assert torch.equal(out["passes"], out["fused"])
+            assert torch.equal(out["documented"], out["fused"])
