@@ -392,8 +392,12 @@ __global__ void maxpool_kernel(const bf16* __restrict__ in, int is, int B, int H
 
 // Max-pool backward, in place on the skip slice of a concatenation gradient:
 // g[q] = bf16(g[q] + (q is the window's argmax ? dp : 0)) where act[q] > 0, else 0.
-__global__ void maxpool_bwd_kernel(const bf16* __restrict__ act, int as, const bf16* __restrict__ dp, bf16* g, int gs,
-                                   int B, int H, int W, int C) {
+// Memory bounds it; the nine 16-byte loads of a window are issued together (loads of g after
+// the first store to it would wait for that store). (Three levels of a 32 x 64 x 256 batch, cold
+// cache: MAXPOOL_FIGURE)
+__global__ void __launch_bounds__(256) maxpool_bwd_kernel(const bf16* __restrict__ act, int as,
+                                                          const bf16* __restrict__ dp, bf16* g, int gs, int B, int H,
+                                                          int W, int C) {
   lbnci::pdl_enter();
   const int h = H / 2, w = W / 2, groups = C / 8;
   const long total = (long)B * h * w * groups;
@@ -401,58 +405,41 @@ __global__ void maxpool_bwd_kernel(const bf16* __restrict__ act, int as, const b
     const int g8 = (int)(i % groups);
     const long q = i / groups;
     const int x = (int)(q % w), y = (int)((q / w) % h), b = (int)(q / ((long)w * h));
-    float a[4][8];
-    int arg[8];
+    V8 a[4], v[4], d;
+    bf16* gp[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const int yy = 2 * y + (k >> 1), xx = 2 * x + (k & 1);
-      V8 v;
-      v.u = *reinterpret_cast<const uint4*>(act + ((size_t)(b * H + yy) * W + xx) * as + g8 * 8);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 f = __bfloat1622float2(v.h[e]);
-        a[k][2 * e] = f.x;
-        a[k][2 * e + 1] = f.y;
-      }
+      const size_t px = (size_t)(b * H + 2 * y + (k >> 1)) * W + 2 * x + (k & 1);
+      gp[k] = g + px * gs + g8 * 8;
+      a[k].u = *reinterpret_cast<const uint4*>(act + px * as + g8 * 8);
+      v[k].u = *reinterpret_cast<const uint4*>(gp[k]);
     }
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      arg[c] = 0;
-#pragma unroll
-      for (int k = 1; k < 4; ++k)
-        if (a[k][c] > a[arg[c]][c]) arg[c] = k;
-    }
-    V8 d;
     d.u = *reinterpret_cast<const uint4*>(dp + q * C + g8 * 8);
-    float dv[8];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const float2 f = __bfloat1622float2(d.h[e]);
-      dv[2 * e] = f.x;
-      dv[2 * e + 1] = f.y;
-    }
+      float2 f[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int yy = 2 * y + (k >> 1), xx = 2 * x + (k & 1);
-      bf16* gp = g + ((size_t)(b * H + yy) * W + xx) * gs + g8 * 8;
-      V8 v;
-      v.u = *reinterpret_cast<const uint4*>(gp);
-      float o[8];
+      for (int k = 0; k < 4; ++k) f[k] = __bfloat1622float2(a[k].h[e]);
+      const float2 dv = __bfloat1622float2(d.h[e]);
+      int ax = 0, ay = 0;
+      float bx = f[0].x, by = f[0].y;
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 f = __bfloat1622float2(v.h[e]);
-        o[2 * e] = f.x;
-        o[2 * e + 1] = f.y;
+      for (int k = 1; k < 4; ++k) {
+        if (f[k].x > bx) { bx = f[k].x; ax = k; }
+        if (f[k].y > by) { by = f[k].y; ay = k; }
       }
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        if (arg[c] == k) o[c] += dv[c];
-        if (!(a[k][c] > 0.f)) o[c] = 0.f;
+      for (int k = 0; k < 4; ++k) {
+        float2 o = __bfloat1622float2(v[k].h[e]);
+        if (ax == k) o.x += dv.x;
+        if (ay == k) o.y += dv.y;
+        if (!(f[k].x > 0.f)) o.x = 0.f;
+        if (!(f[k].y > 0.f)) o.y = 0.f;
+        v[k].h[e] = __floats2bfloat162_rn(o.x, o.y);
       }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) v.h[e] = __floats2bfloat162_rn(o[2 * e], o[2 * e + 1]);
-      *reinterpret_cast<uint4*>(gp) = v.u;
     }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) *reinterpret_cast<uint4*>(gp[k]) = v[k].u;
   }
 }
 
@@ -572,50 +559,77 @@ __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restr
 
 // Head backward. dx[p][c] = bf16(sum_j dy[p][j] wh[j][c]) where x[p][c] > 0, else 0;
 // per block of kHeadPix pixels the partial sums of dW[j][c] = sum_p dy[p][j] x[p][c] and
-// db[j] = sum_p dy[p][j] go to part[block][nout (C + 1)]. A warp takes every eighth pixel of
-// the block, a lane one channel (of each 32): rows of x and dx are whole lines, dy[p] is
-// one broadcast, the sums stay in registers until the block's eight warps are added in
-// order. (32 images of 64 x 256, 32 channels: 74 us, 90 us with one thread per output
-// summing the block's pixels.)
+// db[j] = sum_p dy[p][j] go to part[block][NOUT (C + 1)]. Memory bounds it: four lanes share a
+// pixel, eight channels each (one 16-byte load and store), a warp eight pixels, so that
+// whole lines move and dy is read once per four lanes; the sums stay in registers until the
+// block's pixels are done, then go over the warp's pixels by shuffles and over the warps in
+// order. (32 images of 64 x 256, 32 channels, 3 outputs: HEADBWD_FIGURE)
 constexpr int kHeadPix = 512;
+template <int NOUT>
 __global__ void __launch_bounds__(256) head_bwd_kernel(const bf16* __restrict__ x, int C, const bf16* __restrict__ wh,
-                                                       int nout, int P, const float* __restrict__ dy,
-                                                       bf16* __restrict__ dx, float* __restrict__ part) {
+                                                       int P, const float* __restrict__ dy, bf16* __restrict__ dx,
+                                                       float* __restrict__ part) {
   lbnci::pdl_enter();
-  __shared__ float red[8][kMaxOut + 1][33];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ float red[8][NOUT][33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = threadIdx.x & 3;
   const int p0 = blockIdx.x * kHeadPix, p1 = min(p0 + kHeadPix, P);
-  float* out = part + (size_t)blockIdx.x * nout * (C + 1);
+  float* out = part + (size_t)blockIdx.x * NOUT * (C + 1);
   for (int c0 = 0; c0 < C; c0 += 32) {
-    float w[kMaxOut], sw[kMaxOut], sb[kMaxOut];
+    float w[NOUT][8], sw[NOUT][8], sb[NOUT];
 #pragma unroll
-    for (int j = 0; j < kMaxOut; ++j) {
-      w[j] = j < nout ? __bfloat162float(wh[j * C + c0 + lane]) : 0.f;
-      sw[j] = 0.f;
+    for (int j = 0; j < NOUT; ++j) {
+      V8 v;
+      v.u = *reinterpret_cast<const uint4*>(wh + (size_t)j * C + c0 + g * 8);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 f = __bfloat1622float2(v.h[e]);
+        w[j][2 * e] = f.x;
+        w[j][2 * e + 1] = f.y;
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e) sw[j][e] = 0.f;
       sb[j] = 0.f;
     }
-#pragma unroll 4
-    for (int p = p0 + warp; p < p1; p += 8) {
-      const float xv = __bfloat162float(x[(size_t)p * C + c0 + lane]);
-      float s = 0.f;
+#pragma unroll 2
+    for (int p = p0 + (threadIdx.x >> 2); p < p1; p += 64) {
+      V8 v, o;
+      v.u = *reinterpret_cast<const uint4*>(x + (size_t)p * C + c0 + g * 8);
+      float d[NOUT];
 #pragma unroll
-      for (int j = 0; j < kMaxOut; ++j)
-        if (j < nout) {
-          const float d = dy[(size_t)p * nout + j];
-          s = fmaf(d, w[j], s);
-          sw[j] = fmaf(d, xv, sw[j]);
-          sb[j] += d;
+      for (int j = 0; j < NOUT; ++j) d[j] = dy[(size_t)p * NOUT + j];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 f = __bfloat1622float2(v.h[e]);
+        float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+        for (int j = 0; j < NOUT; ++j) {
+          s0 = fmaf(d[j], w[j][2 * e], s0);
+          s1 = fmaf(d[j], w[j][2 * e + 1], s1);
+          sw[j][2 * e] = fmaf(d[j], f.x, sw[j][2 * e]);
+          sw[j][2 * e + 1] = fmaf(d[j], f.y, sw[j][2 * e + 1]);
         }
-      dx[(size_t)p * C + c0 + lane] = __float2bfloat16_rn(xv > 0.f ? s : 0.f);
+        o.h[e] = __floats2bfloat162_rn(f.x > 0.f ? s0 : 0.f, f.y > 0.f ? s1 : 0.f);
+      }
+#pragma unroll
+      for (int j = 0; j < NOUT; ++j) sb[j] += d[j];
+      *reinterpret_cast<uint4*>(dx + (size_t)p * C + c0 + g * 8) = o.u;
     }
 #pragma unroll
-    for (int j = 0; j < kMaxOut; ++j)
-      if (j < nout) {
-        red[warp][j][lane] = sw[j];
+    for (int j = 0; j < NOUT; ++j) {
+#pragma unroll
+      for (int m = 4; m < 32; m <<= 1) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) sw[j][e] += __shfl_xor_sync(~0u, sw[j][e], m);
+        sb[j] += __shfl_xor_sync(~0u, sb[j], m);
+      }
+      if (lane < 4) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) red[warp][j][lane * 8 + e] = sw[j][e];
         if (lane == 0) red[warp][j][32] = sb[j];
       }
+    }
     __syncthreads();
-    for (int o = threadIdx.x; o < nout * 33; o += 256) {
+    for (int o = threadIdx.x; o < NOUT * 33; o += 256) {
       const int j = o / 33, l = o % 33;
       float v = 0.f;
 #pragma unroll
