@@ -696,7 +696,21 @@ lb_status backward_impl(lbu_net* n, int B) {
   {
     const int hi = head_i(n), C0 = n->cfg.base;
     const int nblk = (P + lbu::kHeadPix - 1) / lbu::kHeadPix;
-    lbnci::launch_pdl(lbu::head_bwd_kernel, dim3(nblk), dim3(256), 0, s, n->db[0], C0, WB(n, hi), n->cfg.out_ch, P, n->dy, n->gB[0], n->work);
+    auto head_bwd = [&](auto NOUT) {
+      lbnci::launch_pdl(lbu::head_bwd_kernel<decltype(NOUT)::value>, dim3(nblk), dim3(256), 0, s, n->db[0], C0,
+                        WB(n, hi), P, n->dy, n->gB[0], n->work);
+    };
+    static_assert(lbu::kMaxOut == 8, "one build per number of outputs");
+    switch (n->cfg.out_ch) {
+      case 1: head_bwd(std::integral_constant<int, 1>{}); break;
+      case 2: head_bwd(std::integral_constant<int, 2>{}); break;
+      case 3: head_bwd(std::integral_constant<int, 3>{}); break;
+      case 4: head_bwd(std::integral_constant<int, 4>{}); break;
+      case 5: head_bwd(std::integral_constant<int, 5>{}); break;
+      case 6: head_bwd(std::integral_constant<int, 6>{}); break;
+      case 7: head_bwd(std::integral_constant<int, 7>{}); break;
+      default: head_bwd(std::integral_constant<int, 8>{}); break;
+    }
     lbnci::launch_pdl(lbu::head_reduce_kernel, dim3(n->cfg.out_ch * (C0 + 1)), dim3(128), 0, s, n->work, nblk, n->cfg.out_ch, C0, GW(hi), GB(hi));
     n->launches += 2;
   }

@@ -393,8 +393,8 @@ __global__ void maxpool_kernel(const bf16* __restrict__ in, int is, int B, int H
 // Max-pool backward, in place on the skip slice of a concatenation gradient:
 // g[q] = bf16(g[q] + (q is the window's argmax ? dp : 0)) where act[q] > 0, else 0.
 // Memory bounds it; the nine 16-byte loads of a window are issued together (loads of g after
-// the first store to it would wait for that store). (Three levels of a 32 x 64 x 256 batch, cold
-// cache: MAXPOOL_FIGURE)
+// the first store to it would wait for that store). (Three levels of 32 images of 64 x 256, cold
+// cache: 50 us, 73 us with the loads of g in the loop of its stores.)
 __global__ void __launch_bounds__(256) maxpool_bwd_kernel(const bf16* __restrict__ act, int as,
                                                           const bf16* __restrict__ dp, bf16* g, int gs, int B, int H,
                                                           int W, int C) {
@@ -563,7 +563,8 @@ __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restr
 // pixel, eight channels each (one 16-byte load and store), a warp eight pixels, so that
 // whole lines move and dy is read once per four lanes; the sums stay in registers until the
 // block's pixels are done, then go over the warp's pixels by shuffles and over the warps in
-// order. (32 images of 64 x 256, 32 channels, 3 outputs: HEADBWD_FIGURE)
+// order. (32 images of 64 x 256, 32 channels, 3 outputs: 23 us cold, 73 us with one channel per
+// lane, whose loads of dy and x a warp had few of in flight.)
 constexpr int kHeadPix = 512;
 template <int NOUT>
 __global__ void __launch_bounds__(256) head_bwd_kernel(const bf16* __restrict__ x, int C, const bf16* __restrict__ wh,

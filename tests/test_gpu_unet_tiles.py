@@ -92,3 +92,34 @@ def test_network_outputs_equal_and_gradients_agree(H, W, B, levels, monkeypatch)
     assert torch.equal(got[0][0], got[1][0]) and got[0][1] == got[1][1]
     a, b = got[0][2].double(), got[1][2].double()
     assert float((a - b).norm() / b.norm()) <= 100 * 2.0 ** -23
+
+
+@pytest.mark.parametrize("out_ch", [1, 2, 5, 8])
+def test_head_gradient_for_other_output_counts(out_ch):
+    """The 1x1 head's weight and bias gradients (the last layer's) from the activations' own
+    gradient identity: dL/db = sum dy and, with the head's weights scaled, dL/dy . y = sum over the
+    head's weights and biases of theta dL/dtheta (y is linear in them); FP32 sums of P = 1152
+    terms, 2^-23 each relative to sum|terms|, which random data exceeds the sum of by about 100."""
+    H, W, B = 16, 24, 3
+    cfg = unet.make_config(levels=2, base=32, out_ch=out_ch, H=H, W=W, max_batch=B)
+    shapes = U.layer_shapes(2, 32, 5, out_ch)
+    params = unet.flatten(inputs.unet_params(shapes, 4, bias_scale=0.05))
+    g = torch.Generator(device="cuda").manual_seed(9)
+    X = torch.randn((B, H, W, 5), device="cuda", generator=g)
+    T = torch.randn((B, H, W, out_ch), device="cuda", generator=g)
+    with unet.Net(cfg) as net:
+        net.set_params(params)
+        y = torch.empty((B, H, W, out_ch), device="cuda")
+        net.forward(X, y)
+        G = torch.zeros(net.nparams, device="cuda")
+        net.loss_grad(X, T, grads=G)
+        torch.cuda.synchronize()
+    gw, gb = unet.unflatten(G.cpu().numpy().astype(np.float64), unet.layer_shapes(cfg))[-1]
+    w, b = unet.unflatten(np.asarray(params, dtype=np.float32).astype(np.float64), unet.layer_shapes(cfg))[-1]
+    w = torch.from_numpy(np.ascontiguousarray(w)).float().bfloat16().double().numpy()  # the head multiplies BF16 weights
+    dy = (2.0 / (B * H * W) * (y.double() - T.double())).reshape(-1, out_ch).cpu().numpy()
+    tol = 100 * 2.0 ** -23
+    assert np.all(np.abs(gb - dy.sum(0)) <= tol * np.abs(dy).sum(0))
+    terms = dy * (y.double().reshape(-1, out_ch).cpu().numpy() - np.asarray(b))
+    assert np.all(np.abs((gw * w).reshape(out_ch, -1).sum(1) - terms.sum(0)) <= tol * (np.abs(terms).sum(0) +
+                                                                                     np.abs(gw * w).reshape(out_ch, -1).sum(1)))
