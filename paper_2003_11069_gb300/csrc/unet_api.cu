@@ -362,11 +362,12 @@ bool plan_rows(int B, int H, int W, int cin, int cout, int up, bool mask, ConvPl
     for (int occ = 2; occ >= 1; --occ) {
       const int cols = 512 / occ;
       const int R = std::min(lbu::kRowsMaxSlot, cols / (npx * BN)) & ~1;
-      if (R < 4) continue;
+      if (R < 6) continue;  // three pairs: one drained, one completed, one begun
       const int weights = 9 * nchunk * BN * rowb, staging = 2 * 128 * BN * 2;
       const int room = kSmemSm / occ - 1024 - (int)sizeof(lbu::RowsTail) - 16 - weights - staging;
-      const int nrow = std::min(lbu::kRowsMaxStage, room / (nchunk * cstride));
-      if (nrow < 3) continue;
+      int nrow = std::min(lbu::kRowsMaxStage, room / (nchunk * cstride));
+      if (!up) nrow &= ~1;  // stages of two rows
+      if (nrow < (up ? 3 : 4)) continue;
       const double n3 = 3 * BN, mma = 3.0 * nchunk * (rowb / 32) * npx * (n3 <= 128 ? 32 + n3 / 4 : n3 / 2);
       for (int TH = 2; TH <= Ho; TH += 2) {
         if (TH > 2 && TH - 2 >= Ho) break;

@@ -494,6 +494,15 @@ conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
 // An accumulator starts from zeros that the draining warps store (a row's first MMA shares
 // its instruction with two rows that accumulate); 0 + a is a.
 //
+// The issuing warp bounds the kernel: a row is 6 to 24 MMAs of 56 cycles, and each barrier it
+// waits on or commits to costs it 100 to 300 cycles. So everything goes by units of two virtual
+// rows (up: one input row): a stage of the ring is a unit's input rows, and output rows come
+// in pairs q (rows 2q, 2q + 1; up: 2q - 1, 2q), of which unit u begins pair u and completes
+// pair u - 1: three waits and two commits per unit instead of per row. Slots are handed out
+// by pairs; three pairs at least, so that one drains while the next completes. (One row per
+// barrier -> two, 32 images: 64 x 256, 32 -> 32 channels 26.7 -> 22.8 us, 64 -> 32 41.0 -> 28.7,
+// 32 -> 64 45.1 -> 37.3; 32 x 128, 64 -> 64 24.6 -> 18.4, 128 -> 64 30.8 -> 24.7.)
+//
 // Warps: 0 copies, 1 issues MMAs, 2..9 drain (two groups of four, alternate rows), 10 patches
 // the periodic columns.
 constexpr int kRowsThreads = 352, kRowsMaxStage = 8, kRowsMaxSlot = 16;
@@ -502,7 +511,7 @@ struct ConvRows {
   int xs, H, W, up;        // input image
   int tiles_x, tiles_h, TH;  // strips of 128 columns, groups of TH output rows
   int nchunk, cstride;     // chunks of ROWB/2 channels; bytes of a row's chunk in shared memory
-  int nrow, R;             // ring stages (input rows), accumulator slots (output rows, even)
+  int nrow, R;             // input rows in the ring (even unless up), accumulator slots (output rows, even)
   int w_off, stg_off, tail;
   int cols;
   const float* bias;
@@ -514,7 +523,7 @@ struct ConvRows {
 };
 struct RowsTail {
   unsigned long long bar_w, bar_full[kRowsMaxStage], bar_patched[kRowsMaxStage], bar_empty[kRowsMaxStage];
-  unsigned long long bar_row[kRowsMaxSlot], bar_free[kRowsMaxSlot];
+  unsigned long long bar_row[kRowsMaxSlot / 2], bar_free[kRowsMaxSlot / 2];
   unsigned tmem;
   int fail;
   alignas(16) float bias[64];
@@ -536,17 +545,20 @@ conv3x3_rows_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
   const int nh = min(a.TH, Ho - h0);
   const int first = a.up ? (h0 >> 1) - 1 : h0 - 1, nin = a.up ? (nh >> 1) + 2 : nh + 2;
   const int row_bytes = a.nchunk * a.cstride;
+  // units: input rows of a stage, stages, units; output pairs (rows 2q - a.up, + 1) and their slots
+  const int rpu = 2 - a.up, ns = a.nrow / rpu, nu = (nin + rpu - 1) / rpu;
+  const int nq = a.up ? (nh >> 1) + 1 : (nh + 1) >> 1, RP = a.R >> 1;
 
   if (tid == 0) {
     lbnci::mbar_init(&t.bar_w, 1);
-    for (int s = 0; s < a.nrow; ++s) {
+    for (int s = 0; s < ns; ++s) {
       lbnci::mbar_init(&t.bar_full[s], 1);
       lbnci::mbar_init(&t.bar_patched[s], 1);
       lbnci::mbar_init(&t.bar_empty[s], 1);
     }
-    for (int s = 0; s < a.R; ++s) {
+    for (int s = 0; s < RP; ++s) {
       lbnci::mbar_init(&t.bar_row[s], 1);
-      lbnci::mbar_init(&t.bar_free[s], 4);
+      lbnci::mbar_init(&t.bar_free[s], 8);
     }
     t.fail = (smem_u32(sm) & 1023u) ? 2 : 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -574,97 +586,104 @@ conv3x3_rows_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
   } else if (warp == 0) {
     if (lane == 0) {  // copies of the rows
       int issued = 0;
-      for (int i = 0; i < nin; ++i) {
-        const int s = i % a.nrow, u = i / a.nrow;
-        if (u > 0 && !lbnci::mbar_wait(&t.bar_empty[s], (unsigned)((u - 1) & 1))) {
+      for (int u = 0; u < nu; ++u) {
+        const int s = u % ns, w = u / ns, rows = min(rpu, nin - u * rpu);
+        if (w > 0 && !lbnci::mbar_wait(&t.bar_empty[s], (unsigned)((w - 1) & 1))) {
           atomicOr(&t.fail, 1);
           break;
         }
-        lbnci::mbar_expect_tx(&t.bar_full[s], (unsigned)(a.nchunk * XW * ROWB));
-        for (int k = 0; k < a.nchunk; ++k)
-          lbnci::tma_load_4d(sm + s * row_bytes + k * a.cstride, &map_x, k * CH, x0 - 1, first + i, b, &t.bar_full[s]);
-        issued = i + 1;
+        lbnci::mbar_expect_tx(&t.bar_full[s], (unsigned)(rows * a.nchunk * XW * ROWB));
+        for (int r = 0; r < rows; ++r)
+          for (int k = 0; k < a.nchunk; ++k)
+            lbnci::tma_load_4d(sm + (s * rpu + r) * row_bytes + k * a.cstride, &map_x, k * CH, x0 - 1,
+                               first + u * rpu + r, b, &t.bar_full[s]);
+        issued = u + 1;
       }
       lbnci::mbar_wait(&t.bar_w, 0u);  // every copy has landed before the CTA may end (bounded)
-      for (int i = issued > a.nrow ? issued - a.nrow : 0; i < issued; ++i)
-        lbnci::mbar_wait(&t.bar_full[i % a.nrow], (unsigned)((i / a.nrow) & 1));
+      for (int u = issued > ns ? issued - ns : 0; u < issued; ++u)
+        lbnci::mbar_wait(&t.bar_full[u % ns], (unsigned)((u / ns) & 1));
     }
   } else if (warp == 1) {  // MMAs: the whole warp runs the loop
     const unsigned long long d0 = tc::desc_base(ROWB, 16u, 8u * ROWB);
     const unsigned hi = (unsigned)(d0 >> 32);
     const unsigned loA = (unsigned)d0 + (smem_u32(sm) >> 4), loW = (unsigned)d0 + (smem_u32(sW) >> 4);
     bool bad = __any_sync(~0u, !lbnci::mbar_wait(&t.bar_w, 0u));
-    int s = 0;
-    unsigned ph = 0u;
-    for (int i = 0; i < nin && !bad; ++i) {
-      bad = __any_sync(~0u, !lbnci::mbar_wait(&t.bar_full[s], ph) || !lbnci::mbar_wait(&t.bar_patched[s], ph));
+    int s = 0, q = 0, last = RP - 1, base = a.R - 2;  // stage, slots of pairs u and u - 1, slot of row v - 1
+    unsigned ph = 0u, qph = 0u;
+    for (int u = 0; u < nu; ++u) {
+      bad = bad || !lbnci::mbar_wait(&t.bar_full[s], ph) || !lbnci::mbar_wait(&t.bar_patched[s], ph) ||
+            (u < nq && !lbnci::mbar_wait(&t.bar_free[q], qph));  // the pair's slots are drained and zeroed
+      bad = __any_sync(~0u, bad);
       if (bad) break;
       tc::fence_after_sync();
-      const unsigned la = loA + (unsigned)((s * row_bytes) >> 4);
-      for (int pass = 0; pass < npx; ++pass) {
-        const int v = a.up ? 2 * (i - 1) + pass : i - 1;  // virtual input row, relative to h0
-        if (v < -1 || v > nh) continue;
-        const int lo = max(0, v - 1), hi_row = min(nh - 1, v + 1), n = hi_row - lo + 1;
-        if (hi_row == v + 1) {  // a new output row: its slot is drained and zeroed
-          bad = __any_sync(~0u, !lbnci::mbar_wait(&t.bar_free[hi_row % a.R], (unsigned)((hi_row / a.R) & 1)));
-          if (bad) break;
-          tc::fence_after_sync();
-        }
-        // rows lo .. hi_row in slots; beyond the last slot they continue at slot 0
-        const int slot = lo % a.R, n1 = min(n, a.R - slot), n2 = n - n1, j0 = lo - (v - 1);
-        auto rows = [&](int sl, int j, int nn) {
-          const unsigned id = tc::idesc_bf16(128, 0) | ((unsigned)(nn * BN / 8) << 17);
-          // dx outermost, then channels: the order of the taps
 #pragma unroll
-          for (int dxi = 0; dxi < 3; ++dxi)
-            for (int k = 0; k < a.nchunk; ++k) {
-              const unsigned lw = loW + (unsigned)((((dxi * a.nchunk + k) * 3 + j) * WB) >> 4);
-              const unsigned lk = la + (unsigned)((k * a.cstride) >> 4);
-              for (int px = 0; px < npx; ++px) {
-                const int ox = a.up ? (px + dxi - 1) >> 1 : dxi - 1;
-                const unsigned lr = lk + (unsigned)(((ox + 1) * ROWB) >> 4);
-                const unsigned d = tmem + (unsigned)((px * a.R + sl) * BN);
+      for (int pass = 0; pass < 2; ++pass) {
+        const int v = 2 * u - 1 - a.up + pass;  // virtual input row, relative to h0
+        if (v >= -1 && v <= nh) {
+          const unsigned la = loA + (unsigned)(((s * rpu + (a.up ? 0 : pass)) * row_bytes) >> 4);
+          const int lo = max(0, v - 1), n = min(nh - 1, v + 1) - lo + 1, j0 = lo - (v - 1);
+          // rows lo .. lo + n - 1 in slots; beyond the last slot they continue at slot 0
+          const int at = base + j0, slot = at >= a.R ? at - a.R : at, n1 = min(n, a.R - slot);
+          auto rows = [&](int sl, int j, int nn) {
+            const unsigned id = tc::idesc_bf16(128, 0) | ((unsigned)(nn * BN / 8) << 17);
+            // dx outermost, then channels: the order of the taps
 #pragma unroll
-                for (int kk = 0; kk < KK; ++kk)
-                  tc::mma_bf16<true>(d, tc::desc64(hi, lr + 2 * kk), tc::desc64(hi, lw + 2 * kk), id);
+            for (int dxi = 0; dxi < 3; ++dxi)
+              for (int k = 0; k < a.nchunk; ++k) {
+                const unsigned lw = loW + (unsigned)((((dxi * a.nchunk + k) * 3 + j) * WB) >> 4);
+                const unsigned lk = la + (unsigned)((k * a.cstride) >> 4);
+                for (int px = 0; px < npx; ++px) {
+                  const int ox = a.up ? (px + dxi - 1) >> 1 : dxi - 1;
+                  const unsigned lr = lk + (unsigned)(((ox + 1) * ROWB) >> 4);
+                  const unsigned d = tmem + (unsigned)((px * a.R + sl) * BN);
+#pragma unroll
+                  for (int kk = 0; kk < KK; ++kk)
+                    tc::mma_bf16<true>(d, tc::desc64(hi, lr + 2 * kk), tc::desc64(hi, lw + 2 * kk), id);
+                }
               }
-            }
-        };
-        rows(slot, j0, n1);
-        if (n2 > 0) rows(0, j0 + n1, n2);
-        if (v >= 1) tc::mma_commit(&t.bar_row[(v - 1) % a.R]);  // output row v - 1 is complete
+          };
+          rows(slot, j0, n1);
+          if (n1 < n) rows(0, j0 + n1, n - n1);
+        }
+        if (++base == a.R) base = 0;
       }
       tc::mma_commit(&t.bar_empty[s]);
-      if (++s == a.nrow) {
+      if (u > 0) tc::mma_commit(&t.bar_row[last]);  // output pair u - 1 is complete
+      last = q;
+      if (++q == RP) {
+        q = 0;
+        qph ^= 1u;
+      }
+      if (++s == ns) {
         s = 0;
         ph ^= 1u;
       }
     }
     if (lane == 0 && bad) atomicOr(&t.fail, 1);
-    // the MMAs issued are done before tensor memory is released: the last row's barrier below
+    // the MMAs issued are done before tensor memory is released: the last pair's barrier below
   } else if (warp == 10) {  // the periodic images of the columns beyond the image
     const int left = x0 == 0 ? 1 : 0, right = x0 + 128 >= a.W ? 1 : 0, ncol = left + right;
     const int vpp = a.nchunk * (ROWB / 16), count = ncol * vpp;
     bool ok = true;
-    for (int i = 0; i < nin && ok; ++i) {
-      const int s = i % a.nrow, yy = first + i;
-      const bool in = yy >= 0 && yy < a.H;
-      for (int e0 = 0; e0 < count || e0 == 0; e0 += 64) {
+    for (int u = 0; u < nu && ok; ++u) {
+      const int s = u % ns;
+      for (int e0 = 0; e0 < rpu * count || e0 == 0; e0 += 64) {
         uint4 v[2];
         int dst[2];
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           const int e = e0 + 32 * j + lane;
           dst[j] = -1;
-          if (in && e < count) {
-            const int col = e / vpp, p = e - col * vpp, k = p / (ROWB / 16);
+          const int r = e >= count ? 1 : 0, f = e - r * count, i = u * rpu + r, yy = first + i;
+          if (e < rpu * count && i < nin && yy >= 0 && yy < a.H) {
+            const int col = f / vpp, p = f - col * vpp, k = p / (ROWB / 16);
             const bool lft = left && col == 0;
             v[j] = *reinterpret_cast<const uint4*>(a.x + ((size_t)(b * a.H + yy) * a.W + (lft ? a.W - 1 : 0)) * a.xs + p * 8);
-            dst[j] = s * row_bytes + k * a.cstride +
+            dst[j] = (s * rpu + r) * row_bytes + k * a.cstride +
                      (int)tc::swizzled<ROWB>(lft ? 0 : a.W - x0 + 1, p - k * (ROWB / 16));
           }
         }
-        if (e0 == 0) ok = __all_sync(~0u, lbnci::mbar_wait(&t.bar_full[s], (unsigned)((i / a.nrow) & 1)));
+        if (e0 == 0) ok = __all_sync(~0u, lbnci::mbar_wait(&t.bar_full[s], (unsigned)((u / ns) & 1)));
         if (!ok) break;
 #pragma unroll
         for (int j = 0; j < 2; ++j)
@@ -687,15 +706,29 @@ conv3x3_rows_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
       tc::tmem_wait_st();
       tc::fence_before_sync();
       __syncwarp();
-      if (lane == 0) lbnci::mbar_arrive(&t.bar_free[slot]);
+      if (lane == 0) lbnci::mbar_arrive(&t.bar_free[slot >> 1]);
     };
     for (int s = g; s < a.R; s += 2) zero(s);
     unsigned char* const stg = sm + a.stg_off + g * (128 * BN * 2);
     constexpr int NV = BN / 8;
     auto piece = [](int r, int v) { return r * (BN * 2) + ((v ^ ((BN == 32 ? r >> 1 : r) & (NV - 1))) << 4); };
     bool ok = true;
-    for (int h = g; h < nh && ok; h += 2) {
-      const int slot = h % a.R;
+    int qs = 0;
+    unsigned qph = 0u;
+    for (int q = 0; q < nq && ok; ++q) {
+      const int h = 2 * q - a.up + g, slot = 2 * qs + g;
+      unsigned long long* const done = &t.bar_row[qs];
+      const unsigned dph = qph;
+      if (++qs == RP) {
+        qs = 0;
+        qph ^= 1u;
+      }
+      if (h < 0 || h >= nh) {  // the pair's other row is the image's first or last
+        ok = lbnci::mbar_wait(done, dph);
+        if (!ok) atomicOr(&t.fail, 1);
+        if (q + RP < nq) zero(slot);
+        continue;
+      }
       for (int px = 0; px < npx; ++px) {
         // this thread's pieces: row (128 k + gt) / NV, piece gt % NV; the masks are in flight
         // while the row is awaited
@@ -709,7 +742,7 @@ conv3x3_rows_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             mk[k] = *reinterpret_cast<const uint4*>(a.mask + (size_t)orow[k] * a.ms + n0 + (gt % NV) * 8);
         }
         if (px == 0) {
-          ok = lbnci::mbar_wait(&t.bar_row[slot], (unsigned)((h / a.R) & 1));
+          ok = lbnci::mbar_wait(done, dph);
           if (!ok) atomicOr(&t.fail, 1);
           tc::fence_after_sync();
         }
@@ -733,7 +766,7 @@ conv3x3_rows_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             *reinterpret_cast<uint4*>(stg + piece(l, c0 / 8 + v)) = o.u;
           }
         }
-        if (px == npx - 1 && h + a.R < nh) zero(slot);  // for row h + R
+        if (px == npx - 1 && q + RP < nq) zero(slot);  // for row h + R
         ok = bar_all(1 + g, 128, ok);
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
