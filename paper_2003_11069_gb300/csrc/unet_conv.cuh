@@ -99,6 +99,15 @@ __device__ __forceinline__ void mma_bf16(unsigned tmem_d, unsigned long long a, 
       "l"(a), "l"(b), "r"(idesc), "n"(ACC ? 1 : 0)
       : "memory");
 }
+// The same with the choice at run time, where a second copy of a loop would cost more.
+__device__ __forceinline__ void mma_bf16_if(unsigned tmem_d, unsigned long long a, unsigned long long b, unsigned idesc,
+                                            int acc) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t.reg .b32 x;\n\tsetp.ne.b32 p, %4, 0;\n\telect.sync x|q, 0xffffffff;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      : "memory");
+}
 // The mbarrier receives one arrival when every MMA issued before has completed (whole warp).
 __device__ __forceinline__ void mma_commit(unsigned long long* bar) {
   asm volatile(
@@ -113,15 +122,15 @@ __device__ __forceinline__ unsigned long long desc64(unsigned hi, unsigned lo) {
 // The K = 16 MMAs kk = 0 .. KK - 1 of one stage for G accumulators (d + g dstep), whose A
 // operands start at the descriptors lo[g]: unrolled, accumulators innermost, so that an MMA
 // costs a few instructions of the issuing warp and seldom follows one into its accumulator.
-template <int G, int KK, bool ACC>
+template <int G, int KK>
 __device__ __forceinline__ void mma_group(unsigned d, unsigned dstep, const unsigned lo[G], unsigned hiA, unsigned loB,
-                                          unsigned hiB, unsigned idesc) {
+                                          unsigned hiB, unsigned idesc, int acc) {
 #pragma unroll
   for (int kk = 0; kk < KK; ++kk)
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      if (ACC || kk > 0) mma_bf16<true>(d + g * dstep, desc64(hiA, lo[g] + 2 * kk), desc64(hiB, loB + 2 * kk), idesc);
-      else mma_bf16<false>(d + g * dstep, desc64(hiA, lo[g]), desc64(hiB, loB), idesc);
+      if (kk > 0) mma_bf16<true>(d + g * dstep, desc64(hiA, lo[g] + 2 * kk), desc64(hiB, loB + 2 * kk), idesc);
+      else mma_bf16_if(d + g * dstep, desc64(hiA, lo[g]), desc64(hiB, loB), idesc, acc);
     }
 }
 // 16 or 32 consecutive 32-bit columns of this thread's lane (shape 32x32b: lane = warp's base
@@ -279,53 +288,62 @@ conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     // lower halves in 16-byte units: addresses below 256 KB never carry out of their field
     const unsigned loA0 = (unsigned)dA + (smem_u32(sA) >> 4), loB0 = (unsigned)dB + (smem_u32(sB) >> 4);
     const unsigned mstep = (unsigned)(a.mstart * ROWB) >> 4;
-    unsigned ph = 0u;
+    // A stage's addresses advance by additions and stand before its wait: what the issuing warp
+    // does between two stages is time the tensor cores wait for (16 x 64, 256 -> 128 channels,
+    // 32 images: 28.6 -> 26.7 us; 8 x 32, 256 -> 256: 26.4 -> 24.6). The loops stay rolled and the
+    // first MMAs' "do not accumulate" is a value: in a network each kernel runs once between
+    // others, its instructions not cached (batch-8 forward 219 -> 210 us, with the taps of a row
+    // unrolled 230).
+    const unsigned step = (unsigned)(a.a_stride >> 4), row = (unsigned)(a.pitch * ROWB) >> 4;
+    unsigned ph = 0u, lb = loB0;
     int s = 0;
-    auto stage = [&](int tap, int k, auto ACC) {  // (a converged warp: __any_sync before it)
-      constexpr bool acc = decltype(ACC)::value;
-      const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-      const unsigned lb = loB0 + (unsigned)(s * (BBYTES >> 4)), la = loA0 + (unsigned)((k * a.a_stride) >> 4);
-      auto at = [&](int oy, int ox) { return la + (unsigned)((((oy + 1) * a.pitch + ox + 1) * ROWB) >> 4); };
+    auto issue = [&](const unsigned at[4], int acc) {  // (a converged warp: __any_sync before it)
+      unsigned lo[4];
       if (a.up) {
-        // the four parities of an upsampled input: low-resolution row and column
-        // floor((parity + tap)/2)
-        unsigned lo[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) lo[q] = at(((q >> 1) + dy) >> 1, ((q & 1) + dx) >> 1);
         for (int m = 0; m < a.nm; ++m) {
-          tc::mma_group<4, KK, acc>(tmem + m * BN, (unsigned)(a.nm * BN), lo, hiA, lb, hiB, IDESC);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) lo[q] += mstep;
+          for (int q = 0; q < 4; ++q) lo[q] = at[q] + m * mstep;
+          tc::mma_group<4, KK>(tmem + m * BN, (unsigned)(a.nm * BN), lo, hiA, lb, hiB, IDESC, acc);
         }
       } else {
-        unsigned lo[4];
-        lo[0] = at(dy, dx);
-        lo[1] = lo[0] + mstep;
-        lo[2] = lo[1] + mstep;
-        lo[3] = lo[2] + mstep;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) lo[g] = at[0] + g * mstep;
         int m = 0;
         for (; m + 4 <= a.nm; m += 4) {
-          tc::mma_group<4, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC);
+          tc::mma_group<4, KK>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC, acc);
 #pragma unroll
           for (int g = 0; g < 4; ++g) lo[g] += 4 * mstep;
         }
-        if (a.nm - m == 3) tc::mma_group<3, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC);
-        else if (a.nm - m == 2) tc::mma_group<2, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC);
-        else if (a.nm - m == 1) tc::mma_group<1, KK, acc>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC);
-      }
-      tc::mma_commit(&t.bar_empty[s]);
-      if (++s == ST) {
-        s = 0;
-        ph ^= 1u;
+        if (a.nm - m == 3) tc::mma_group<3, KK>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC, acc);
+        else if (a.nm - m == 2) tc::mma_group<2, KK>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC, acc);
+        else if (a.nm - m == 1) tc::mma_group<1, KK>(tmem + m * BN, BN, lo, hiA, lb, hiB, IDESC, acc);
       }
     };
-    for (int tap = 0; tap < 9 && !bad; ++tap)
-      for (int k = 0; k < a.nchunk; ++k) {
-        bad = __any_sync(~0u, !lbnci::mbar_wait(&t.bar_full[s], ph));
-        if (bad) break;
-        tc::fence_after_sync();
-        if (tap == 0 && k == 0) stage(tap, k, std::false_type{});
-        else stage(tap, k, std::true_type{});
+#pragma unroll 1
+    for (int dy = 0; dy < 3 && !bad; ++dy)
+#pragma unroll 1
+      for (int dx = 0; dx < 3; ++dx) {
+        unsigned at[4];  // up: the parities, at low-resolution row and column floor((parity + tap)/2)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          at[q] = loA0 + (a.up ? (unsigned)((((q >> 1) + dy - 1) >> 1) + 1) * row +
+                                     (unsigned)((((((q & 1) + dx - 1) >> 1) + 1) * ROWB) >> 4)
+                               : (unsigned)dy * row + (unsigned)((dx * ROWB) >> 4));
+        for (int k = 0; k < a.nchunk; ++k) {
+          if (!bad) bad = __any_sync(~0u, !lbnci::mbar_wait(&t.bar_full[s], ph));
+          if (bad) break;
+          tc::fence_after_sync();
+          issue(at, dx + dy + k);
+          tc::mma_commit(&t.bar_empty[s]);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) at[q] += step;
+          lb += BBYTES >> 4;
+          if (++s == ST) {
+            s = 0;
+            lb = loB0;
+            ph ^= 1u;
+          }
+        }
       }
     if (lane == 0) {
       if (bad) atomicOr(&t.fail, 1);
@@ -616,7 +634,7 @@ conv3x3_rows_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
       bad = __any_sync(~0u, bad);
       if (bad) break;
       tc::fence_after_sync();
-#pragma unroll
+#pragma unroll 1
       for (int pass = 0; pass < 2; ++pass) {
         const int v = 2 * u - 1 - a.up + pass;  // virtual input row, relative to h0
         if (v >= -1 && v <= nh) {
@@ -923,17 +941,16 @@ conv3x3_wgrad_tma_kernel(const __grid_constant__ WgradMaps maps, WgradTma a, int
     const unsigned dpar = (unsigned)(a.d_bytes >> 4);
     unsigned ph = 0u;
     int s = 0;
-    auto block = [&](unsigned ua, unsigned ub, auto ACC) {  // the MMAs of K = 16 pixels of a row
-      constexpr bool acc = decltype(ACC)::value;
+    auto block = [&](unsigned ua, unsigned ub, int acc) {  // the MMAs of K = 16 pixels of a row
       if (ROWB == 128 && a.up) {
 #pragma unroll
         for (int j = 0; j < NA; ++j)
-          tc::mma_bf16<acc>(tmem + j * BN, tc::desc64(hiA, ua + rel[j]), tc::desc64(hiB, ub + (unsigned)(j >> 1) * dpar),
-                            IDESC);
+          tc::mma_bf16_if(tmem + j * BN, tc::desc64(hiA, ua + rel[j]), tc::desc64(hiB, ub + (unsigned)(j >> 1) * dpar),
+                          IDESC, acc);
       } else {
 #pragma unroll
         for (int j = 0; j < (ROWB == 64 ? 3 : 5); ++j)
-          tc::mma_bf16<acc>(tmem + j * BN, tc::desc64(hiA, ua + rel[j]), tc::desc64(hiB, ub), IDESC);
+          tc::mma_bf16_if(tmem + j * BN, tc::desc64(hiA, ua + rel[j]), tc::desc64(hiB, ub), IDESC, acc);
       }
     };
     for (int i = 0; i < nt; ++i) {
@@ -945,8 +962,7 @@ conv3x3_wgrad_tma_kernel(const __grid_constant__ WgradMaps maps, WgradTma a, int
       for (int r = 0; r < a.TH; ++r) {
         unsigned ua = ux + (unsigned)((r * a.pitch * ROWB) >> 4), ub = ud + (unsigned)((r * a.TW * DROW) >> 4);
         for (int c = 0; c < kx; ++c) {
-          if (i == 0 && r == 0 && c == 0) block(ua, ub, std::false_type{});
-          else block(ua, ub, std::true_type{});
+          block(ua, ub, i | r | c);
           ua += ROWB;  // 16 pixels of ROWB bytes, in 16-byte units
           ub += DROW;
         }
