@@ -95,9 +95,11 @@ WORKLOADS = {
 }
 
 # The kernels lb_step launches, by lb_step_path().
-STEP_KERNELS = {0: "fused2d_kernel (one-pass D2Q9 step)",
+STEP_KERNELS = {0: "site_moments_kernel + site_normals_kernel + site_collide*_kernel (D2Q9 step as passes over the "
+                   "sites: FP64 with Guo forcing, nx % 4 != 0; three launches) or fused2d_kernel (one-pass step)",
                 1: "tma2d_kernel (persistent TMA-fed D2Q9 step, one launch per step)",
-                2: "moments_kernel + march3d_kernel (D3Q27 two-pass step, two launches)",
+                2: "moments, normals and collision passes (D3Q27 FP64 with Guo forcing and lattices of no whole "
+                   "columns, three launches) or moments_kernel + march3d_kernel (two launches)",
                 3: "interface3d_kernel + nci3d_kernel + carry3d_kernel (D3Q27 single-read step: densities "
                    "carried by the previous collision, interface pass, NCI ray pass, TMA-fed collision; three "
                    "launches)",
