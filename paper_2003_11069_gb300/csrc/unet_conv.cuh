@@ -84,22 +84,21 @@ __device__ __forceinline__ void tmem_dealloc(unsigned taddr, unsigned ncols) {  
 __device__ __forceinline__ void fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// D (tensor memory) = A B^T (+ D when ACC), run by a whole warp and issued by the lane that
+// D (tensor memory) += A B^T, run by a whole warp and issued by the lane that
 // elect.sync picks (always the same one). With the whole warp in the issue loop its
 // addresses are warp-uniform values, and the elected predicate needs no per-lane branch.
 // Cycles per MMA of M = 128, K = 16, measured: 40, 48, 56, 64, 96 and 127 for N = 32, 64, 96,
 // 128, 192 and 256, that is the operands' bytes at 128 a cycle up to N = 128, then the tensor
 // cores' rate; a predicate from the lane number gave 50 to 72 up to N = 128, and a branch that
 // one lane takes around descriptors built with run-time multiplications 80 to 250.
-template <bool ACC>
 __device__ __forceinline__ void mma_bf16(unsigned tmem_d, unsigned long long a, unsigned long long b, unsigned idesc) {
   asm volatile(
-      "{\n\t.reg .pred p, q;\n\t.reg .b32 x;\n\tsetp.ne.b32 p, %4, 0;\n\telect.sync x|q, 0xffffffff;\n\t"
+      "{\n\t.reg .pred p, q;\n\t.reg .b32 x;\n\tsetp.ne.b32 p, 1, 0;\n\telect.sync x|q, 0xffffffff;\n\t"
       "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(a), "l"(b), "r"(idesc), "n"(ACC ? 1 : 0)
+      "l"(a), "l"(b), "r"(idesc)
       : "memory");
 }
-// The same with the choice at run time, where a second copy of a loop would cost more.
+// The same, D = A B^T where acc is 0: a value, as a second copy of a loop costs more than it.
 __device__ __forceinline__ void mma_bf16_if(unsigned tmem_d, unsigned long long a, unsigned long long b, unsigned idesc,
                                             int acc) {
   asm volatile(
@@ -129,7 +128,7 @@ __device__ __forceinline__ void mma_group(unsigned d, unsigned dstep, const unsi
   for (int kk = 0; kk < KK; ++kk)
 #pragma unroll
     for (int g = 0; g < G; ++g) {
-      if (kk > 0) mma_bf16<true>(d + g * dstep, desc64(hiA, lo[g] + 2 * kk), desc64(hiB, loB + 2 * kk), idesc);
+      if (kk > 0) mma_bf16(d + g * dstep, desc64(hiA, lo[g] + 2 * kk), desc64(hiB, loB + 2 * kk), idesc);
       else mma_bf16_if(d + g * dstep, desc64(hiA, lo[g]), desc64(hiB, loB), idesc, acc);
     }
 }
@@ -656,7 +655,7 @@ conv3x3_rows_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                   const unsigned d = tmem + (unsigned)((px * a.R + sl) * BN);
 #pragma unroll
                   for (int kk = 0; kk < KK; ++kk)
-                    tc::mma_bf16<true>(d, tc::desc64(hi, lr + 2 * kk), tc::desc64(hi, lw + 2 * kk), id);
+                    tc::mma_bf16(d, tc::desc64(hi, lr + 2 * kk), tc::desc64(hi, lw + 2 * kk), id);
                 }
               }
           };
@@ -1088,7 +1087,9 @@ conv3x3_wgrad_tma_kernel(const __grid_constant__ WgradMaps maps, WgradTma a, int
 // threads to each (thread k the splits k, k + S, ...; their sums added in thread order), S
 // so large that the grid fills the multiprocessors: whole lines are read, every load of a
 // thread is independent. up: a tap's sum also runs over the four parities, each at the
-// shift floor((parity + tap)/2) the tap has there.
+// shift floor((parity + tap)/2) the tap has there, the four loads of a split issued together (32
+// images, cold: 12.4, 20.3 and 17.7 us for the three such layers with a parity at a time, all 17
+// reductions 174 us, now 158).
 __global__ void __launch_bounds__(256) wgrad_reduce_tma_kernel(const float* __restrict__ part,
                                                                const float* __restrict__ bpart, int nsplit, int Cout,
                                                                int Cin, int cin_true, int up, int S, int wblocks,
@@ -1125,19 +1126,28 @@ __global__ void __launch_bounds__(256) wgrad_reduce_tma_kernel(const float* __re
     o = r / 9;
     const size_t stride = (size_t)Cout * nk * Cin;
     const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-    for (int q = 0; q < (up ? 4 : 1); ++q) {
+    const float* p[4];  // the parities' parts: shift row py - 1 + sy, column px - 1 + sx
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
       const int py = q >> 1, px = q & 1;
-      // shift row py - 1 + sy, column px - 1 + sx
       const int k = up ? 4 * q + 2 * (((py + dy) >> 1) - py + 1) + (((px + dx) >> 1) - px + 1) : tap;
-      const float* p = part + ((size_t)o * nk + k) * Cin + c;
+      p[q] = part + ((size_t)o * nk + k) * Cin + c;
+    }
+    auto add = [&](const float* at) {
+      const float4 w = *reinterpret_cast<const float4*>(at);
+      v.x += w.x;
+      v.y += w.y;
+      v.z += w.z;
+      v.w += w.w;
+    };
+    if (up) {
+#pragma unroll 2
+      for (int z = share; z < nsplit; z += S)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) add(p[q] + (size_t)z * stride);
+    } else {
 #pragma unroll 4
-      for (int z = share; z < nsplit; z += S) {
-        const float4 w = *reinterpret_cast<const float4*>(p + (size_t)z * stride);
-        v.x += w.x;
-        v.y += w.y;
-        v.z += w.z;
-        v.w += w.w;
-      }
+      for (int z = share; z < nsplit; z += S) add(p[0] + (size_t)z * stride);
     }
   }
   s[threadIdx.x] = v;
