@@ -524,7 +524,7 @@ cudaError_t launch_wgrad_tma(const WgradTmaPlan& p, const lbu::WgradMaps& maps, 
   e = lbnci::allow_smem(lbu::conv3x3_wgrad_tma_kernel<BN, ROWB>, (size_t)p.smem, configured);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)p.a.nsplit, (unsigned)(p.a.Cin / (ROWB / 2)), (unsigned)(p.a.Cout / BN));
-  lbnci::launch_pdl(lbu::conv3x3_wgrad_tma_kernel<BN, ROWB>, dim3(grid), dim3(lbu::kConvThreads), p.smem, s, maps, p.a, err);
+  lbnci::launch_pdl(lbu::conv3x3_wgrad_tma_kernel<BN, ROWB>, grid, dim3(lbu::kConvThreads), p.smem, s, maps, p.a, err);
   return cudaGetLastError();
 }
 
@@ -602,8 +602,8 @@ lb_status wgrad(lbu_net* n, int site, const bf16* x, int xs, int up, const bf16*
       int S = 1;  // threads to each group of four values: about four blocks per multiprocessor
       while (S < 32 && 2 * S <= p.a.nsplit && (long long)n4 * S < 152LL * 4 * 256) S *= 2;
       const int wblocks = (n4 + 256 / S - 1) / (256 / S), bblocks = db_master ? (cout + 31) / 32 : 0;
-      lbnci::launch_pdl(lbu::wgrad_reduce_tma_kernel, dim3(wblocks + bblocks), dim3(256), 0, s, work, bp, p.a.nsplit, cout, cin, cin_true, up, S,
-                                                                     wblocks, dw_master, db_master);
+      lbnci::launch_pdl(lbu::wgrad_reduce_tma_kernel, dim3(wblocks + bblocks), dim3(256), 0, s, work, bp, p.a.nsplit,
+                        cout, cin, cin_true, up, S, wblocks, dw_master, db_master);
       if (n) n->launches += 2;
       e = cudaGetLastError();
       return e == cudaSuccess ? LB_OK : cuda_fail(n, e, "wgrad reduction launch");
@@ -643,6 +643,22 @@ int enc_b(int l) { return 2 * l + 1; }
 int up_i(const lbu_net* n, int l) { return 2 * n->cfg.levels + 3 * (n->cfg.levels - 2 - l); }
 int head_i(const lbu_net* n) { return (int)n->L.size() - 1; }
 
+// The head's kernels are built for each number of outputs.
+template <typename F>
+void for_outputs(int nout, F&& f) {
+  static_assert(lbu::kMaxOut == 8, "one build per number of outputs");
+  switch (nout) {
+    case 1: return f(std::integral_constant<int, 1>{});
+    case 2: return f(std::integral_constant<int, 2>{});
+    case 3: return f(std::integral_constant<int, 3>{});
+    case 4: return f(std::integral_constant<int, 4>{});
+    case 5: return f(std::integral_constant<int, 5>{});
+    case 6: return f(std::integral_constant<int, 6>{});
+    case 7: return f(std::integral_constant<int, 7>{});
+    default: return f(std::integral_constant<int, 8>{});
+  }
+}
+
 lb_status forward_impl(lbu_net* n, int B) {
   const int Lv = n->cfg.levels;
   cudaStream_t s = n->stream;
@@ -656,7 +672,8 @@ lb_status forward_impl(lbu_net* n, int B) {
       LBU_TRY(conv(n, enc_b(l), n->ea[l], C, B, H, W, C, 0, WB(n, enc_b(l)), BIAS(n, enc_b(l)), 1, n->cat[l] + C, 2 * C, C,
                    nullptr, 0, s));
       const long long work = (long long)B * (H / 2) * (W / 2) * (C / 8);
-      lbnci::launch_pdl(lbu::maxpool_kernel, dim3(grid_for(work, 256)), dim3(256), 0, s, n->cat[l] + C, 2 * C, B, H, W, C, n->pool[l]);
+      lbnci::launch_pdl(lbu::maxpool_kernel, dim3(grid_for(work, 256)), dim3(256), 0, s,
+                        n->cat[l] + C, 2 * C, B, H, W, C, n->pool[l]);
       ++n->launches;
       h = n->pool[l];
       hs = C;
@@ -678,8 +695,10 @@ lb_status forward_impl(lbu_net* n, int B) {
   }
   const int hi = head_i(n);
   const int P = B * n->cfg.H * n->cfg.W;
-  lbnci::launch_pdl(lbu::head_fwd_kernel, dim3(grid_for(P, 256)), dim3(256), 0, s, n->db[0], n->cfg.base, WB(n, hi), BIAS(n, hi),
-                                                        n->cfg.out_ch, P, n->y);
+  for_outputs(n->cfg.out_ch, [&](auto NOUT) {
+    lbnci::launch_pdl(lbu::head_fwd_kernel<decltype(NOUT)::value>, dim3(grid_for(P, 256)), dim3(256), 0, s, n->db[0],
+                      n->cfg.base, WB(n, hi), BIAS(n, hi), P, n->y);
+  });
   ++n->launches;
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? LB_OK : cuda_fail(n, e, "forward launch");
@@ -697,22 +716,12 @@ lb_status backward_impl(lbu_net* n, int B) {
   {
     const int hi = head_i(n), C0 = n->cfg.base;
     const int nblk = (P + lbu::kHeadPix - 1) / lbu::kHeadPix;
-    auto head_bwd = [&](auto NOUT) {
+    for_outputs(n->cfg.out_ch, [&](auto NOUT) {
       lbnci::launch_pdl(lbu::head_bwd_kernel<decltype(NOUT)::value>, dim3(nblk), dim3(256), 0, s, n->db[0], C0,
                         WB(n, hi), P, n->dy, n->gB[0], n->work);
-    };
-    static_assert(lbu::kMaxOut == 8, "one build per number of outputs");
-    switch (n->cfg.out_ch) {
-      case 1: head_bwd(std::integral_constant<int, 1>{}); break;
-      case 2: head_bwd(std::integral_constant<int, 2>{}); break;
-      case 3: head_bwd(std::integral_constant<int, 3>{}); break;
-      case 4: head_bwd(std::integral_constant<int, 4>{}); break;
-      case 5: head_bwd(std::integral_constant<int, 5>{}); break;
-      case 6: head_bwd(std::integral_constant<int, 6>{}); break;
-      case 7: head_bwd(std::integral_constant<int, 7>{}); break;
-      default: head_bwd(std::integral_constant<int, 8>{}); break;
-    }
-    lbnci::launch_pdl(lbu::head_reduce_kernel, dim3(n->cfg.out_ch * (C0 + 1)), dim3(128), 0, s, n->work, nblk, n->cfg.out_ch, C0, GW(hi), GB(hi));
+    });
+    lbnci::launch_pdl(lbu::head_reduce_kernel,
+                      dim3(n->cfg.out_ch * (C0 + 1)), dim3(128), 0, s, n->work, nblk, n->cfg.out_ch, C0, GW(hi), GB(hi));
     n->launches += 2;
   }
   // decoder, finest level first
@@ -732,8 +741,8 @@ lb_status backward_impl(lbu_net* n, int B) {
     LBU_TRY(wgrad(n, k, hin, C1, 1, n->gCat[l], 2 * C, B, H, W, C1, C, n->work, n->work_bytes, s, GW(k), GB(k), C1));
     LBU_TRY(conv(n, nl + k, n->gCat[l], 2 * C, B, H, W, C, 0, WT(n, k), nullptr, 0, n->gU[l], C1, C1, nullptr, 0, s));
     const long long work = (long long)B * Hl(n, l + 1) * Wl(n, l + 1) * (C1 / 8);
-    lbnci::launch_pdl(lbu::upsample_bwd_kernel, dim3(grid_for(work, 256)), dim3(256), 0, s, n->gU[l], hin, n->gB[l + 1], B, Hl(n, l + 1),
-                                                                 Wl(n, l + 1), C1);
+    lbnci::launch_pdl(lbu::upsample_bwd_kernel, dim3(grid_for(work, 256)), dim3(256), 0, s,
+                      n->gU[l], hin, n->gB[l + 1], B, Hl(n, l + 1), Wl(n, l + 1), C1);
     ++n->launches;
   }
   // encoder, coarsest level first; gB[Lv-1] holds the bottom output's gradient
@@ -746,8 +755,8 @@ lb_status backward_impl(lbu_net* n, int B) {
       gs = C;
     } else {
       const long long work = (long long)B * (H / 2) * (W / 2) * (C / 8);
-      lbnci::launch_pdl(lbu::maxpool_bwd_kernel, dim3(grid_for(work, 256)), dim3(256), 0, s, n->cat[l] + C, 2 * C, n->gPool[l],
-                                                                  n->gCat[l] + C, 2 * C, B, H, W, C);
+      lbnci::launch_pdl(lbu::maxpool_bwd_kernel, dim3(grid_for(work, 256)), dim3(256), 0, s,
+                        n->cat[l] + C, 2 * C, n->gPool[l], n->gCat[l] + C, 2 * C, B, H, W, C);
       ++n->launches;
       g = n->gCat[l] + C;
       gs = 2 * C;
@@ -770,7 +779,7 @@ lb_status refresh(lbu_net* n) {
   size_t maxn = 0;
   for (auto& l : n->L) maxn = std::max(maxn, (size_t)l.cout * l.taps * l.cin_pad);
   dim3 grid((unsigned)std::min<size_t>((maxn + 255) / 256, 1024), (unsigned)n->L.size());
-  lbnci::launch_pdl(lbu::refresh_weights_kernel, dim3(grid), dim3(256), 0, n->stream, n->Ldev, n->params, n->wb, n->wt);
+  lbnci::launch_pdl(lbu::refresh_weights_kernel, grid, dim3(256), 0, n->stream, n->Ldev, n->params, n->wb, n->wt);
   ++n->launches;
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? LB_OK : cuda_fail(n, e, "refresh launch");
@@ -781,8 +790,8 @@ lb_status loss_impl(lbu_net* n, const float* T, const int* idx, int B, const flo
   float lm[8];
   for (int j = 0; j < 8; ++j) lm[j] = (lam && j < n->cfg.out_ch) ? lam[j] : 1.f;
   const int blocks = std::min(n->npartial, grid_for(P, 256));
-  lbnci::launch_pdl(lbu::mse_kernel, dim3(blocks), dim3(256), 0, n->stream, n->y, T, idx, HW, n->cfg.out_ch, P, lm[0], lm[1], lm[2], lm[3],
-                                                 lm[4], lm[5], lm[6], lm[7], n->dy, n->partial);
+  lbnci::launch_pdl(lbu::mse_kernel, dim3(blocks), dim3(256), 0, n->stream, n->y, T, idx, HW, n->cfg.out_ch, P, lm[0],
+                    lm[1], lm[2], lm[3], lm[4], lm[5], lm[6], lm[7], n->dy, n->partial);
   lbnci::launch_pdl(lbu::sum_partials_kernel, dim3(1), dim3(256), 0, n->stream, n->partial, blocks, 1.0 / P, n->loss);
   n->launches += 2;
   cudaError_t e = cudaGetLastError();
@@ -791,8 +800,8 @@ lb_status loss_impl(lbu_net* n, const float* T, const int* idx, int B, const flo
 
 lb_status pack(lbu_net* n, const float* X, const int* idx, int B) {
   const long long work = (long long)B * n->cfg.H * n->cfg.W * (kInPad / 8);
-  lbnci::launch_pdl(lbu::pack_input_kernel, dim3(grid_for(work, 256)), dim3(256), 0, n->stream, X, idx, B, n->cfg.H * n->cfg.W, n->cfg.in_ch,
-                                                                     kInPad, n->x0);
+  lbnci::launch_pdl(lbu::pack_input_kernel, dim3(grid_for(work, 256)), dim3(256), 0,
+                    n->stream, X, idx, B, n->cfg.H * n->cfg.W, n->cfg.in_ch, kInPad, n->x0);
   ++n->launches;
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? LB_OK : cuda_fail(n, e, "pack launch");
@@ -1034,8 +1043,8 @@ lb_status lbu_train_step(lbu_net* n, const float* X, const float* T, const int* 
   ++n->t;
   const float c1 = (float)(1.0 / (1.0 - std::pow((double)n->b1, (double)n->t)));
   const float c2 = (float)(1.0 / (1.0 - std::pow((double)n->b2, (double)n->t)));
-  lbnci::launch_pdl(lbu::adam_kernel, dim3(grid_for(n->nparams, 256)), dim3(256), 0, n->stream, n->params, n->grads, n->m, n->v, n->nparams,
-                                                                    lr, n->b1, n->b2, n->eps, c1, c2);
+  lbnci::launch_pdl(lbu::adam_kernel, dim3(grid_for(n->nparams, 256)), dim3(256), 0, n->stream, n->params, n->grads,
+                    n->m, n->v, n->nparams, lr, n->b1, n->b2, n->eps, c1, c2);
   ++n->launches;
   LBU_CUDA(n, cudaGetLastError());
   LBU_TRY(refresh(n));

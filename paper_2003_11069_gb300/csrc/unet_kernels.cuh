@@ -482,32 +482,38 @@ __global__ void upsample_bwd_kernel(const bf16* __restrict__ du, const bf16* __r
 // ------------------------------------------------------------------ head, loss
 constexpr int kMaxOut = 8, kMaxHeadIn = 256;
 
-// y[p][j] = b[j] + sum_c wh[j][c] x[p][c]; x BF16 [P][C], wh BF16 [nout][C], y FP32
-__global__ void head_fwd_kernel(const bf16* __restrict__ x, int C, const bf16* __restrict__ wh,
-                                const float* __restrict__ bh, int nout, int P, float* __restrict__ y) {
+// y[p][j] = b[j] + sum_c wh[j][c] x[p][c]; x BF16 [P][C], wh BF16 [NOUT][C], y FP32. One pixel a
+// thread, the loads of 32 channels issued together (32 images of 64 x 256, cold: 12 us, 20 us with
+// eight channels at a time and the number of outputs a run-time bound).
+template <int NOUT>
+__global__ void __launch_bounds__(256) head_fwd_kernel(const bf16* __restrict__ x, int C, const bf16* __restrict__ wh,
+                                                       const float* __restrict__ bh, int P, float* __restrict__ y) {
   lbnci::pdl_enter();
-  __shared__ float sw[kMaxOut * kMaxHeadIn];
-  for (int i = threadIdx.x; i < nout * C; i += blockDim.x) sw[i] = __bfloat162float(wh[i]);
+  __shared__ float sw[NOUT * kMaxHeadIn];
+  for (int i = threadIdx.x; i < NOUT * C; i += blockDim.x) sw[i] = __bfloat162float(wh[i]);
   __syncthreads();
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
-    float acc[kMaxOut];
+    float acc[NOUT];
 #pragma unroll
-    for (int j = 0; j < kMaxOut; ++j) acc[j] = j < nout ? bh[j] : 0.f;
-    for (int c0 = 0; c0 < C; c0 += 8) {
-      V8 v;
-      v.u = *reinterpret_cast<const uint4*>(x + (size_t)p * C + c0);
+    for (int j = 0; j < NOUT; ++j) acc[j] = bh[j];
+    for (int c0 = 0; c0 < C; c0 += 32) {
+      V8 v[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 f = __bfloat1622float2(v.h[e]);
+      for (int k = 0; k < 4; ++k) v[k].u = *reinterpret_cast<const uint4*>(x + (size_t)p * C + c0 + 8 * k);
 #pragma unroll
-        for (int j = 0; j < kMaxOut; ++j)
-          if (j < nout) {
-            acc[j] = fmaf(sw[j * C + c0 + 2 * e], f.x, acc[j]);
-            acc[j] = fmaf(sw[j * C + c0 + 2 * e + 1], f.y, acc[j]);
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float2 f = __bfloat1622float2(v[k].h[e]);
+#pragma unroll
+          for (int j = 0; j < NOUT; ++j) {
+            acc[j] = fmaf(sw[j * C + c0 + 8 * k + 2 * e], f.x, acc[j]);
+            acc[j] = fmaf(sw[j * C + c0 + 8 * k + 2 * e + 1], f.y, acc[j]);
           }
-      }
+        }
     }
-    for (int j = 0; j < nout; ++j) y[(size_t)p * nout + j] = acc[j];
+#pragma unroll
+    for (int j = 0; j < NOUT; ++j) y[(size_t)p * NOUT + j] = acc[j];
   }
 }
 
