@@ -127,6 +127,11 @@ lb_status cuda_fail(lb_sim* s, cudaError_t e, const char* what) {
   return fail(s, LB_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+// The per-site passes launch blocks of at least 32 x 8 sites of one plane (fewer rows only on
+// lattices of few): a grid has at most 65535 blocks along y and z. Longer lattices keep the
+// kernels that count blocks or sites along x.
+bool site_grid_fits(int ny, int nz) { return ny <= 8 * 65535 && nz <= 65535; }
+
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 // The result area holds 16 doubles: the kRedSlots reductions, then, in slot
@@ -212,7 +217,9 @@ lb_status validate(const lb_config* c, HostParams* p, Layout* lay, long long* nb
   const bool col_ok = c->lattice == LB_D3Q27 && (c->precision == LB_FP32 || c->precision == LB_FP16DEV) &&
                       c->nx % 32 == 0 && c->ny % 8 == 0 && (c->wall_z || c->nz >= 2);
   p->carry3d = 0;
-  p->stream3d = c->lattice == LB_D3Q27 && c->precision != LB_FP64 && (c->wall_z || c->nz >= 2) ? 1 : 0;
+  const bool grid_ok = site_grid_fits(c->ny, c->nz);
+  p->stream3d =
+      c->lattice == LB_D3Q27 && c->precision != LB_FP64 && (c->wall_z || c->nz >= 2) && (col_ok || grid_ok) ? 1 : 0;
   // FP64 steps with Guo forcing run the per-site passes of lb_sites.cuh at every size: the
   // FP64 pipe bounds both ways, and the passes recompute nothing over halos (128 x 128: 23 us
   // per step against 117 us with the fused kernel, whose 32 tiles also leave most
@@ -225,6 +232,7 @@ lb_status validate(const lb_config* c, HostParams* p, Layout* lay, long long* nb
   if (c->lattice == LB_D3Q27) sites = sites && !std::getenv("LBNCI_D3_KERNEL");
   else sites = (sites || (c->precision != LB_FP64 && c->nx % 4 != 0)) && !std::getenv("LBNCI_FUSED_SPT") &&
                !std::getenv("LBNCI_FUSED");
+  sites = sites && grid_ok;
   if (const char* e = std::getenv("LBNCI_D3_KERNEL")) {
     if (std::strcmp(e, "march") == 0 || std::strcmp(e, "tiled") == 0) p->stream3d = 0;
     if (std::strcmp(e, "carry") == 0 && col_ok) { p->carry3d = 1; p->stream3d = 0; }
@@ -295,7 +303,8 @@ lb_status run_fields(lb_sim* s, const FieldOut& outs, size_t staged = 0) {
   int nk = 0;
   const size_t state = s->L->state_bytes((size_t)s->p.N) & ~(size_t)255;
   const size_t need = s->L->fields_scratch((size_t)s->p.N);
-  void* scratch = need + staged <= state ? (void*)((unsigned char*)s->fb + (state - need)) : nullptr;
+  const bool room = need + staged <= state && site_grid_fits(s->p.ny, s->p.nz);
+  void* scratch = room ? (void*)((unsigned char*)s->fb + (state - need)) : nullptr;
   long long rows = s->nblocks;
   if (scratch) {  // the fields pass adds its own sums and writes them to the pinned result
     fo.out = s->host_result;

@@ -183,3 +183,24 @@ def test_ragged_2d_passes_equal_the_one_pass_kernel(precision, nx, ny, wall, mon
                     lbnci.lb_get_populations(sim.h, out[mode])
             assert torch.equal(out["passes"], out["fused"])
             assert torch.equal(out["documented"], out["fused"])
+
+
+@pytest.mark.parametrize("precision", [lbnci.LB_FP64, lbnci.LB_FP32, lbnci.LB_FP16DEV])
+@pytest.mark.parametrize("lat,nx,ny,nz", [(lbnci.LB_D2Q9, 1, 8 * 65535 + 3, 1), (lbnci.LB_D3Q27, 3, 2, 65537)])
+def test_lattices_longer_than_a_grid_axis(lat, nx, ny, nz, precision, monkeypatch):
+    """Lattices that the passes' grids cannot hold step on the kernels that count blocks along x, as
+    the environment variables select them: the same bits."""
+    f = torch.from_numpy(_state(lat, nx, ny, nz, 5)).cuda()
+    got = []
+    for old in (False, True):
+        for k, v in (("LBNCI_D3_KERNEL", "march"), ("LBNCI_FUSED", "classic")):
+            monkeypatch.setenv(k, v) if old else monkeypatch.delenv(k, raising=False)
+        with lbnci.Sim(_cfg(lat, nx, ny, nz, (1, int(nz > 1)), precision)) as sim:
+            lbnci.lb_set_populations(sim.h, f)
+            sim.step(2)
+            got.append(torch.empty_like(f))
+            lbnci.lb_get_populations(sim.h, got[-1])
+            if nz > 1:
+                o = sim.observables(allow_numeric=True)
+                assert np.isfinite(o["mass"][0])
+    assert torch.equal(got[0], got[1])
