@@ -34,11 +34,12 @@
 // columns, then drain the accumulators: bias, ReLU, BF16, through shared memory so that
 // the mask's loads and the output's stores are whole lines.
 //
-// What bounds it: an MMA of M = 128, K = 16 takes about 60 cycles up to N = 128 (the fetch of
-// A), and the copy before and the drain after a tile's MMAs are hidden only by the other
-// CTA of the multiprocessor, where two fit. Measured on GB300 against the mma.sync kernel
-// (conv3x3_kernel), 32 images: 32 -> 32 channels at 64 x 256, 37 us (72 us); 256 -> 256 at
-// 8 x 32, 25 us (75 us).
+// What bounds it: the warp that issues the MMAs, whose waits, commits and addresses between two
+// stages are not hidden behind the stage's MMAs (40 to 64 cycles each up to N = 128), then the
+// copy before and the drain after a tile's MMAs, which only the other CTA of the
+// multiprocessor hides, where two fit. Measured on GB300 against the mma.sync kernel
+// (conv3x3_kernel), 32 images: 128 -> 128 channels at 16 x 64, 18.4 us (55 us); 256 -> 256 at
+// 8 x 32, 24.6 us (75 us). Wide images take conv3x3_rows_kernel below.
 //
 // Every mbarrier wait is bounded (about a second of %globaltimer); on expiry the kernel
 // sets its error word, waits (bounded) for the copies and MMAs in flight, releases its
