@@ -115,7 +115,8 @@ lb_status lbu_conv3x3(const unsigned short* x, int x_stride, int batch, int h, i
 
 /* Weight gradient of that convolution: dw[o][t][c] (FP32, [C_out][9][C_in]) =
  * sum_p dy[p][o] xpad[p + tap t][c] and db[o] = sum_p dy[p][o] (db may be NULL).
- * work: device scratch of at least lbu_conv3x3_wgrad_work(...) bytes. */
+ * work: device scratch of at least lbu_conv3x3_wgrad_work(...) bytes, 8-byte aligned (with
+ * less than 16-byte alignment the mma.sync kernel runs). */
 size_t lbu_conv3x3_wgrad_work(int batch, int h, int w, int c_in, int c_out);
 lb_status lbu_conv3x3_wgrad(const unsigned short* x, int x_stride, int batch, int h, int w, int c_in,
                             int upsample, const unsigned short* dy, int dy_stride, int c_out,

@@ -577,7 +577,9 @@ lb_status conv(lbu_net* n, int site, const bf16* x, int xs, int B, int H, int W,
 lb_status wgrad(lbu_net* n, int site, const bf16* x, int xs, int up, const bf16* dy, int dys, int B, int H, int W, int cin,
                 int cout, float* work, size_t work_bytes, cudaStream_t s, float* dw_master, float* db_master,
                 int cin_true) {
-  if (!conv_on_mma_sync() && xs % 8 == 0 && dys % 8 == 0 && (((uintptr_t)x | (uintptr_t)dy) & 15u) == 0) {
+  // 16-byte pieces of x and dy are copied, and the reduction loads the partial sums in work as such
+  if (!conv_on_mma_sync() && xs % 8 == 0 && dys % 8 == 0 &&
+      (((uintptr_t)x | (uintptr_t)dy | (uintptr_t)work) & 15u) == 0) {
     WgradCache once;
     WgradCache& c = n ? n->wgrad_cache[site] : once;
     if (c.B != B) {
