@@ -100,10 +100,11 @@ lb_status lbu_train_step(lbu_net* net, const float* X, const float* T, const int
  * y[p][o] (BF16 bits, pixel stride y_stride elements) = act(b[o] + sum w[o][t][c] x[...])
  * with x BF16 [batch][h][w][c] (pixel stride x_stride, image h x w, or h/2 x w/2 when
  * upsample = 1: nearest 2x upsampling on the fly), w BF16 [C_out][9][C_in], b FP32 or
- * NULL, act = ReLU when relu = 1. C_in and C_out multiples of 32; strides multiples of 8.
+ * NULL, act = ReLU when relu = 1. C_in and C_out multiples of 32; strides multiples of 8;
+ * x and w 16-byte aligned, y 4-byte (else LB_EINVAL: no kernel could load or store them).
  * The convolutions and weight gradients run on tcgen05.mma with the accumulators in tensor
  * memory, or, where a layer's operands do not fit that kernel (input tiles larger than
- * shared memory, operands not 16-byte aligned) or with the environment variable
+ * shared memory, y not 16-byte aligned) or with the environment variable
  * LBNCI_UNET_MMA=sync (read at every launch), on mma.sync: the convolution's outputs are
  * the same bits. The tcgen05 kernels' waits are bounded: an expired wait leaves output
  * unwritten and sets a device error word, which the next lbu_forward (host output),
@@ -115,8 +116,9 @@ lb_status lbu_conv3x3(const unsigned short* x, int x_stride, int batch, int h, i
 
 /* Weight gradient of that convolution: dw[o][t][c] (FP32, [C_out][9][C_in]) =
  * sum_p dy[p][o] xpad[p + tap t][c] and db[o] = sum_p dy[p][o] (db may be NULL).
- * work: device scratch of at least lbu_conv3x3_wgrad_work(...) bytes, 8-byte aligned (with
- * less than 16-byte alignment the mma.sync kernel runs). */
+ * x and dy are 16-byte aligned; work: device scratch of at least lbu_conv3x3_wgrad_work(...)
+ * bytes, 8-byte aligned (with less than 16-byte alignment the mma.sync kernel runs); else
+ * LB_EINVAL. */
 size_t lbu_conv3x3_wgrad_work(int batch, int h, int w, int c_in, int c_out);
 lb_status lbu_conv3x3_wgrad(const unsigned short* x, int x_stride, int batch, int h, int w, int c_in,
                             int upsample, const unsigned short* dy, int dy_stride, int c_out,

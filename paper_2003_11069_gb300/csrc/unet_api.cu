@@ -809,6 +809,11 @@ lb_status pack(lbu_net* n, const float* X, const int* idx, int B) {
   return e == cudaSuccess ? LB_OK : cuda_fail(n, e, "pack launch");
 }
 
+// Whether p is a multiple of n bytes. Both convolution kernels copy x, the weights and dy in
+// 16-byte pieces (mma.sync by cp.async), mma.sync stores pairs of channels and pairs of partial
+// sums: a pointer below that alignment is refused, no kernel could take it.
+bool aligned(const void* p, unsigned n) { return ((uintptr_t)p & (n - 1u)) == 0; }
+
 lb_status check_batch(lbu_net* n, int B) {
   if (B <= 0 || B > n->cfg.max_batch) return fail(n, LB_EINVAL, "batch must be 1..max_batch");
   return LB_OK;
@@ -1068,6 +1073,8 @@ lb_status lbu_conv3x3(const unsigned short* x, int x_stride, int batch, int h, i
     return fail(nullptr, LB_EINVAL, "sizes: positive, channels multiples of 32");
   if (x_stride < c_in || y_stride < c_out || x_stride % 8 || y_stride % 8)
     return fail(nullptr, LB_EINVAL, "strides: at least the channel count, multiples of 8");
+  if (!aligned(x, 16) || !aligned(wgt, 16) || !aligned(y, 4))
+    return fail(nullptr, LB_EINVAL, "alignment: x and weights 16 bytes, y 4 bytes");
   if (upsample && (h % 2 || w % 2)) return fail(nullptr, LB_EINVAL, "upsampled output must have even size");
   return conv(nullptr, 0, (const bf16*)x, x_stride, batch, h, w, c_in, upsample ? 1 : 0, (const bf16*)wgt, bias, relu,
               (bf16*)y, y_stride, c_out, nullptr, 0, (cudaStream_t)stream);
@@ -1086,6 +1093,8 @@ lb_status lbu_conv3x3_wgrad(const unsigned short* x, int x_stride, int batch, in
     return fail(nullptr, LB_EINVAL, "sizes: positive, channels multiples of 32");
   if (x_stride < c_in || dy_stride < c_out || x_stride % 8 || dy_stride % 8)
     return fail(nullptr, LB_EINVAL, "strides: at least the channel count, multiples of 8");
+  if (!aligned(x, 16) || !aligned(dy, 16) || !aligned(work, 8))
+    return fail(nullptr, LB_EINVAL, "alignment: x and dy 16 bytes, work 8 bytes");
   if (upsample && (h % 2 || w % 2)) return fail(nullptr, LB_EINVAL, "upsampled output must have even size");
   return wgrad(nullptr, 0, (const bf16*)x, x_stride, upsample ? 1 : 0, (const bf16*)dy, dy_stride, batch, h, w, c_in,
                c_out, (float*)work, work_bytes, (cudaStream_t)stream, dw, db, c_in);
