@@ -127,9 +127,9 @@ lb_status cuda_fail(lb_sim* s, cudaError_t e, const char* what) {
   return fail(s, LB_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
-// The per-site passes launch blocks of at least 32 x 8 sites of one plane (fewer rows only on
-// lattices of few): a grid has at most 65535 blocks along y and z. Longer lattices keep the
-// kernels that count blocks or sites along x.
+// The per-site passes and the streaming D3Q27 kernels launch blocks of at least 32 x 8 sites of
+// one plane (fewer rows only on lattices of few): a grid has at most 65535 blocks along y and z.
+// The steps of longer lattices keep the kernels that count blocks or sites along x.
 bool site_grid_fits(int ny, int nz) { return ny <= 8 * 65535 && nz <= 65535; }
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -214,12 +214,10 @@ lb_status validate(const lb_config* c, HostParams* p, Layout* lay, long long* nb
   // no whole columns keep the two-population state (a 150 x 66 x 66 FP32 duct: 0.106 ms per
   // step against 0.175 ms with the marching collision, whose few columns leave CTAs short of
   // planes and whose barriers expose every pull's latency; the states are the same bits)
-  const bool col_ok = c->lattice == LB_D3Q27 && (c->precision == LB_FP32 || c->precision == LB_FP16DEV) &&
-                      c->nx % 32 == 0 && c->ny % 8 == 0 && (c->wall_z || c->nz >= 2);
-  p->carry3d = 0;
   const bool grid_ok = site_grid_fits(c->ny, c->nz);
-  p->stream3d =
-      c->lattice == LB_D3Q27 && c->precision != LB_FP64 && (c->wall_z || c->nz >= 2) && (col_ok || grid_ok) ? 1 : 0;
+  p->carry3d = 0;
+  p->stream3d = c->lattice == LB_D3Q27 && c->precision != LB_FP64 && (c->wall_z || c->nz >= 2) && grid_ok ? 1 : 0;
+  const bool col_ok = p->stream3d && c->nx % 32 == 0 && c->ny % 8 == 0;
   // FP64 steps with Guo forcing run the per-site passes of lb_sites.cuh at every size: the
   // FP64 pipe bounds both ways, and the passes recompute nothing over halos (128 x 128: 23 us
   // per step against 117 us with the fused kernel, whose 32 tiles also leave most

@@ -320,6 +320,7 @@ cudaError_t stream3d_step(const void* fa, void* fb, void* psi, void* ng, void* r
 // two-population reader.
 cudaError_t stream3d_form_fields(const void* f, void* psi, const HostParams& h, const FieldOut& fo, cudaStream_t s,
                                  int* nk, void* scratch, long long rows, long long* used) {
+  if (!scratch) return cudaErrorInvalidValue;  // no kernel without scratch reads these forms
   const StepT<float> p = to_step3(h);
   auto normals = [&](const float* q, Quad<float>* ng) { return launch_normals3d<float, true>(q, ng, p, s); };
   const unsigned N = (unsigned)h.N;

@@ -179,7 +179,7 @@ bool stream3d_stores_totals(const HostParams& h);
 cudaError_t stream3d_step(const void* fa, void* fb, void* psi, void* ng, void* rho12, int totals_in,
                           const HostParams& h, cudaStream_t s, int* nk);
 // fields and population copies of a state in the total + recolouring form (the
-// Launchers::fields / decode of the other states)
+// Launchers::fields / decode of the other states; the fields need the scratch)
 cudaError_t stream3d_form_fields(const void* f, void* psi, const HostParams& h, const FieldOut& fo, cudaStream_t s,
                                  int* nk, void* scratch, long long rows, long long* used);
 cudaError_t stream3d_form_decode(const void* f, double* out, int s0, int count, long long pitch, const HostParams& h,
