@@ -182,6 +182,13 @@ __device__ __forceinline__ bool bar_all(int id, int n, bool ok) {
   return r != 0;
 }
 
+// A bounded wait of a whole warp: the phase's end, or for every lane the limit. Each lane decides for
+// itself whether its wait ran out, so near the limit lanes may differ; what the warp does next (leave
+// a loop, tensor-memory loads, __syncwarp) has to be the same for all of them.
+__device__ __forceinline__ bool warp_wait(unsigned long long* bar, unsigned parity) {
+  return __all_sync(~0u, lbnci::mbar_wait(bar, parity));
+}
+
 constexpr int kConvThreads = 320;  // copy warp, MMA warp, eight epilogue warps
 constexpr int kConvEpiThreads = 256;
 
@@ -379,7 +386,7 @@ conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             }
           }
         }
-        if (e0 == 0) ok = lbnci::mbar_wait(&t.bar_a, 0u);  // the copy's zeros have landed
+        if (e0 == 0) ok = warp_wait(&t.bar_a, 0u);  // the copy's zeros have landed
         if (ok) {
 #pragma unroll
           for (int j = 0; j < U; ++j)
@@ -414,7 +421,7 @@ conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             asm volatile("prefetch.global.L2 [%0];" ::"l"(a.mask + (size_t)row * a.ms + n0 + j));
       }
     // drain: group g of four warps takes accumulators g, g + 2, ...
-    const bool done = lbnci::mbar_wait(&t.bar_d, 0u);
+    const bool done = warp_wait(&t.bar_d, 0u);
     if (!done) atomicOr(&t.fail, 1);
     tc::fence_after_sync();
     if (bar_all(1, kConvEpiThreads, done && *(volatile int*)&t.fail == 0)) {
@@ -701,7 +708,7 @@ conv3x3_rows_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
                      (int)tc::swizzled<ROWB>(lft ? 0 : a.W - x0 + 1, p - k * (ROWB / 16));
           }
         }
-        if (e0 == 0) ok = __all_sync(~0u, lbnci::mbar_wait(&t.bar_full[s], (unsigned)((u / ns) & 1)));
+        if (e0 == 0) ok = warp_wait(&t.bar_full[s], (unsigned)((u / ns) & 1));
         if (!ok) break;
 #pragma unroll
         for (int j = 0; j < 2; ++j)
@@ -742,8 +749,9 @@ conv3x3_rows_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
         qph ^= 1u;
       }
       if (h < 0 || h >= nh) {  // the pair's other row is the image's first or last
-        ok = lbnci::mbar_wait(done, dph);
+        ok = warp_wait(done, dph);
         if (!ok) atomicOr(&t.fail, 1);
+        ok = bar_all(1 + g, 128, ok);  // the group leaves the loop together: its barriers count all of it
         if (q + RP < nq) zero(slot);
         continue;
       }
@@ -760,7 +768,7 @@ conv3x3_rows_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_cons
             mk[k] = *reinterpret_cast<const uint4*>(a.mask + (size_t)orow[k] * a.ms + n0 + (gt % NV) * 8);
         }
         if (px == 0) {
-          ok = lbnci::mbar_wait(done, dph);
+          ok = warp_wait(done, dph);
           if (!ok) atomicOr(&t.fail, 1);
           tc::fence_after_sync();
         }
@@ -1010,7 +1018,7 @@ conv3x3_wgrad_tma_kernel(const __grid_constant__ WgradMaps maps, WgradTma a, int
             }
           }
         }
-        if (e0 == 0) ok = lbnci::mbar_wait(&t.bar_full[s], ph);
+        if (e0 == 0) ok = warp_wait(&t.bar_full[s], ph);
         if (!ok) break;
 #pragma unroll
         for (int j = 0; j < U; ++j)
@@ -1035,7 +1043,7 @@ conv3x3_wgrad_tma_kernel(const __grid_constant__ WgradMaps maps, WgradTma a, int
       if (lane == 0) lbnci::mbar_arrive(&t.bar_empty[s]);
     }
     if (!ok) atomicOr(&t.fail, 1);
-    if (!lbnci::mbar_wait(&t.bar_d, 0u)) {
+    if (!warp_wait(&t.bar_d, 0u)) {
       ok = false;
       atomicOr(&t.fail, 1);
     }
