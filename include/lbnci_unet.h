@@ -107,9 +107,12 @@ lb_status lbu_train_step(lbu_net* net, const float* X, const float* T, const int
  * shared memory, y not 16-byte aligned) or with the environment variable
  * LBNCI_UNET_MMA=sync (read at every launch), on mma.sync: the convolution's outputs are
  * the same bits. The tcgen05 kernels' waits are bounded: an expired wait leaves output
- * unwritten and sets a device error word, which the next lbu_forward (host output),
- * lbu_loss_grad or lbu_train_step (with a loss pointer) reports as LB_ECUDA after it
- * synchronises. */
+ * unwritten and sets an error word. Every network has its own: its next lbu_forward (host
+ * output), lbu_loss_grad or lbu_train_step (with a loss pointer) returns LB_ECUDA after it
+ * synchronises and clears the word; until then the calls that do not synchronise return LB_OK
+ * over incomplete results, and lbu_train_step leaves the parameters as they are. The word of
+ * the single calls is reported in the same way by the next such call of any network on the
+ * device, whose own results are complete then (lbu_last_error says which of the two it was). */
 lb_status lbu_conv3x3(const unsigned short* x, int x_stride, int batch, int h, int w, int c_in,
                       int upsample, const unsigned short* wgt, const float* bias, int relu,
                       unsigned short* y, int y_stride, int c_out, void* stream);

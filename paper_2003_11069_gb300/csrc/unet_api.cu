@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -16,10 +17,11 @@
 #include "unet_conv.cuh"
 #include "lb_launch.h"
 
-// Error word of the tensor-core convolutions: bit 0 set when a bounded mbarrier wait
-// expired (the launch then wrote no output). Read and cleared by the calls that
-// synchronise their stream.
+// Error word of the single tensor-core convolutions (lbu_conv3x3, lbu_conv3x3_wgrad): bit 0 set
+// when a bounded mbarrier wait expired (the launch then wrote no output). A network's kernels
+// set a word of its own (lbu_net::tc_err).
 __device__ int g_tc_err;
+static std::atomic<bool> g_single_used{false};  // some single call has run such a kernel
 
 using lbu::bf16;
 
@@ -203,6 +205,13 @@ struct WgradCache {
 
 }  // namespace
 
+// What the calls that synchronise read back: the loss, the network's error word and the number
+// of parameter updates left out since it was set.
+struct Report {
+  double loss;
+  int err, skipped;
+};
+
 struct lbu_net {
   lbu_config cfg;
   std::vector<LayerHost> L;
@@ -218,7 +227,8 @@ struct lbu_net {
   float *y = nullptr, *dy = nullptr, *xstage = nullptr, *ystage = nullptr;
   float* work = nullptr;
   size_t work_bytes = 0;
-  double *partial = nullptr, *loss = nullptr;
+  double *partial = nullptr, *loss = nullptr;  // loss: a Report
+  int* tc_err = nullptr;  // in that Report
   int npartial = 0;
   float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   long long t = 0;
@@ -474,10 +484,7 @@ cudaError_t launch_conv_rows(const ConvPlan& p, int* err, cudaStream_t s, bool c
 }
 // chained: the launch follows a kernel of the network on its stream (whose wait the weights
 // precede), so it may start while that one drains; a single convolution takes no part in it.
-cudaError_t launch_conv_plan(const ConvPlan& p, cudaStream_t s, bool chained) {
-  int* err = nullptr;
-  cudaError_t e = cudaGetSymbolAddress((void**)&err, g_tc_err);
-  if (e != cudaSuccess) return e;
+cudaError_t launch_conv_plan(const ConvPlan& p, int* err, cudaStream_t s, bool chained) {
   if (p.rows)
     return p.rowb == 128 ? (p.BN == 64 ? launch_conv_rows<64, 128>(p, err, s, chained) : launch_conv_rows<32, 128>(p, err, s, chained))
                          : (p.BN == 64 ? launch_conv_rows<64, 64>(p, err, s, chained) : launch_conv_rows<32, 64>(p, err, s, chained));
@@ -516,28 +523,56 @@ bool wgrad_maps(lbu::WgradMaps* m, const WgradTmaPlan& p, const bf16* x, int xs,
 }
 
 template <int BN, int ROWB>
-cudaError_t launch_wgrad_tma(const WgradTmaPlan& p, const lbu::WgradMaps& maps, cudaStream_t s) {
+cudaError_t launch_wgrad_tma(const WgradTmaPlan& p, const lbu::WgradMaps& maps, int* err, cudaStream_t s) {
   static lbnci::SmemAllowance configured;
-  int* err = nullptr;
-  cudaError_t e = cudaGetSymbolAddress((void**)&err, g_tc_err);
-  if (e != cudaSuccess) return e;
-  e = lbnci::allow_smem(lbu::conv3x3_wgrad_tma_kernel<BN, ROWB>, (size_t)p.smem, configured);
+  cudaError_t e = lbnci::allow_smem(lbu::conv3x3_wgrad_tma_kernel<BN, ROWB>, (size_t)p.smem, configured);
   if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)p.a.nsplit, (unsigned)(p.a.Cin / (ROWB / 2)), (unsigned)(p.a.Cout / BN));
   lbnci::launch_pdl(lbu::conv3x3_wgrad_tma_kernel<BN, ROWB>, grid, dim3(lbu::kConvThreads), p.smem, s, maps, p.a, err);
   return cudaGetLastError();
 }
 
-// Reports (and clears) an expired wait of a tensor-core convolution; call after a
-// synchronisation of the stream.
-lb_status check_tc(lbu_net* n) {
+// The error word of a launch: the network's, or that of the single calls.
+cudaError_t error_word(lbu_net* n, int** err) {
+  if (n) {
+    *err = n->tc_err;
+    return cudaSuccess;
+  }
+  g_single_used = true;
+  return cudaGetSymbolAddress((void**)err, g_tc_err);
+}
+
+// Test of the reporting (never set in use): LBNCI_UNET_FAIL_TEST=1 sets the error word behind
+// every tensor-core launch, as a kernel whose wait ran out would.
+cudaError_t fail_test(int* err, cudaStream_t s) {
+  const char* e = std::getenv("LBNCI_UNET_FAIL_TEST");
+  return e && std::atoi(e) == 1 ? cudaMemsetAsync(err, 1, sizeof(int), s) : cudaSuccess;
+}
+
+// Synchronises the network's stream, reports and clears an expired wait of its kernels, and
+// returns the loss. An expired wait of a single call is reported too, after the results.
+lb_status finish(lbu_net* n, float* loss) {
+  Report r;
+  cudaError_t e = cudaMemcpyAsync(&r, n->loss, sizeof(r), cudaMemcpyDeviceToHost, n->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(n->stream);
+  if (e != cudaSuccess) return cuda_fail(n, e, "result read");
+  if (r.err) {
+    e = cudaMemsetAsync(n->tc_err, 0, 2 * sizeof(int), n->stream);
+    if (e != cudaSuccess) return cuda_fail(n, e, "error word reset");
+    n->t -= r.skipped;
+    return fail(n, LB_ECUDA, "a tensor-core convolution's mbarrier wait expired (no output written; " +
+                                 std::to_string(r.skipped) + " parameter updates left out since)");
+  }
+  if (loss) *loss = (float)r.loss;
+  if (!g_single_used) return LB_OK;
   int v = 0;
-  cudaError_t e = cudaMemcpyFromSymbol(&v, g_tc_err, sizeof(int));
+  e = cudaMemcpyFromSymbol(&v, g_tc_err, sizeof(int));
   if (e != cudaSuccess) return cuda_fail(n, e, "error word read");
   if (v) {
     const int zero = 0;
     cudaMemcpyToSymbol(g_tc_err, &zero, sizeof(int));
-    return fail(n, LB_ECUDA, "a tensor-core convolution's mbarrier wait expired (no output written)");
+    return fail(n, LB_ECUDA, "an earlier single convolution's (lbu_conv3x3, lbu_conv3x3_wgrad) mbarrier wait expired, "
+                             "it wrote no output; this call's results are complete");
   }
   return LB_OK;
 }
@@ -554,7 +589,10 @@ lb_status conv(lbu_net* n, int site, const bf16* x, int xs, int B, int H, int W,
       c.B = B;
     }
     if (c.p.ok) {
-      cudaError_t e = launch_conv_plan(c.p, s, n != nullptr);
+      int* err = nullptr;
+      cudaError_t e = error_word(n, &err);
+      if (e == cudaSuccess) e = launch_conv_plan(c.p, err, s, n != nullptr);
+      if (e == cudaSuccess) e = fail_test(err, s);
       if (n) ++n->launches;
       return e == cudaSuccess ? LB_OK : cuda_fail(n, e, "conv3x3 (tensor memory) launch");
     }
@@ -595,10 +633,14 @@ lb_status wgrad(lbu_net* n, int site, const bf16* x, int xs, int up, const bf16*
       p.a.part = work;
       float* bp = work + (size_t)p.a.nsplit * cout * (up ? 16 : 9) * cin;
       p.a.bpart = db_master ? bp : nullptr;
-      cudaError_t e = p.rowb == 128 ? (p.BN == 64 ? launch_wgrad_tma<64, 128>(p, maps, s)
-                                                  : launch_wgrad_tma<32, 128>(p, maps, s))
-                                    : (p.BN == 64 ? launch_wgrad_tma<64, 64>(p, maps, s)
-                                                  : launch_wgrad_tma<32, 64>(p, maps, s));
+      int* err = nullptr;
+      cudaError_t e = error_word(n, &err);
+      if (e == cudaSuccess)
+        e = p.rowb == 128 ? (p.BN == 64 ? launch_wgrad_tma<64, 128>(p, maps, err, s)
+                                        : launch_wgrad_tma<32, 128>(p, maps, err, s))
+                          : (p.BN == 64 ? launch_wgrad_tma<64, 64>(p, maps, err, s)
+                                        : launch_wgrad_tma<32, 64>(p, maps, err, s));
+      if (e == cudaSuccess) e = fail_test(err, s);
       if (e != cudaSuccess) return cuda_fail(n, e, "wgrad (tensor memory) launch");
       const int n4 = cout * 9 * cin / 4;
       int S = 1;  // threads to each group of four values: about four blocks per multiprocessor
@@ -946,12 +988,14 @@ lb_status lbu_create(const lbu_config* cfg, lbu_net** out) {
   LBU_ALLOC(n->work, wb / sizeof(float) + 1);
   n->npartial = 152 * 16;
   LBU_ALLOC(n->partial, n->npartial);
-  LBU_ALLOC(n->loss, 1);
+  LBU_ALLOC(n->loss, sizeof(Report) / sizeof(double));
+  n->tc_err = &reinterpret_cast<Report*>(n->loss)->err;
 #undef LBU_ALLOC
   if (cudaMemset(n->params, 0, n->nparams * sizeof(float)) != cudaSuccess ||
       cudaMemset(n->m, 0, n->nparams * sizeof(float)) != cudaSuccess ||
       cudaMemset(n->v, 0, n->nparams * sizeof(float)) != cudaSuccess ||
-      cudaMemset(n->grads, 0, n->nparams * sizeof(float)) != cudaSuccess)
+      cudaMemset(n->grads, 0, n->nparams * sizeof(float)) != cudaSuccess ||
+      cudaMemset(n->loss, 0, sizeof(Report)) != cudaSuccess)
     return bail(cuda_fail(n, cudaGetLastError(), "cudaMemset"));
   if (refresh(n) != LB_OK || cudaStreamSynchronize(n->stream) != cudaSuccess)
     return bail(cuda_fail(n, cudaGetLastError(), "initial weight refresh"));
@@ -978,6 +1022,7 @@ lb_status lbu_set_params(lbu_net* n, const float* p, int on_device) {
                               on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, n->stream));
   LBU_CUDA(n, cudaMemsetAsync(n->m, 0, n->nparams * sizeof(float), n->stream));
   LBU_CUDA(n, cudaMemsetAsync(n->v, 0, n->nparams * sizeof(float), n->stream));
+  LBU_CUDA(n, cudaMemsetAsync(n->tc_err + 1, 0, sizeof(int), n->stream));  // Report::skipped
   n->t = 0;
   LBU_TRY(refresh(n));
   LBU_CUDA(n, cudaStreamSynchronize(n->stream));
@@ -1015,11 +1060,7 @@ lb_status lbu_forward(lbu_net* n, const float* x, int batch, float* y, int on_de
   LBU_TRY(forward_impl(n, batch));
   LBU_CUDA(n, cudaMemcpyAsync(y, n->y, batch * HW * n->cfg.out_ch * sizeof(float),
                               on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, n->stream));
-  if (!on_device) {
-    LBU_CUDA(n, cudaStreamSynchronize(n->stream));
-    LBU_TRY(check_tc(n));
-  }
-  return LB_OK;
+  return on_device ? LB_OK : finish(n, nullptr);
 }
 
 lb_status lbu_loss_grad(lbu_net* n, const float* X, const float* T, const int* idx, int batch, const float* lam,
@@ -1032,14 +1073,7 @@ lb_status lbu_loss_grad(lbu_net* n, const float* X, const float* T, const int* i
   LBU_TRY(backward_impl(n, batch));
   if (grads)
     LBU_CUDA(n, cudaMemcpyAsync(grads, n->grads, n->nparams * sizeof(float), cudaMemcpyDeviceToDevice, n->stream));
-  if (loss) {
-    double h = 0.0;
-    LBU_CUDA(n, cudaMemcpyAsync(&h, n->loss, sizeof(double), cudaMemcpyDeviceToHost, n->stream));
-    LBU_CUDA(n, cudaStreamSynchronize(n->stream));
-    LBU_TRY(check_tc(n));
-    *loss = (float)h;
-  }
-  return LB_OK;
+  return loss ? finish(n, loss) : LB_OK;
 }
 
 lb_status lbu_train_step(lbu_net* n, const float* X, const float* T, const int* idx, int batch, const float* lam,
@@ -1051,18 +1085,11 @@ lb_status lbu_train_step(lbu_net* n, const float* X, const float* T, const int* 
   const float c1 = (float)(1.0 / (1.0 - std::pow((double)n->b1, (double)n->t)));
   const float c2 = (float)(1.0 / (1.0 - std::pow((double)n->b2, (double)n->t)));
   lbnci::launch_pdl(lbu::adam_kernel, dim3(grid_for(n->nparams, 256)), dim3(256), 0, n->stream, n->params, n->grads,
-                    n->m, n->v, n->nparams, lr, n->b1, n->b2, n->eps, c1, c2);
+                    n->m, n->v, n->nparams, lr, n->b1, n->b2, n->eps, c1, c2, n->tc_err);
   ++n->launches;
   LBU_CUDA(n, cudaGetLastError());
   LBU_TRY(refresh(n));
-  if (loss) {
-    double h = 0.0;
-    LBU_CUDA(n, cudaMemcpyAsync(&h, n->loss, sizeof(double), cudaMemcpyDeviceToHost, n->stream));
-    LBU_CUDA(n, cudaStreamSynchronize(n->stream));
-    LBU_TRY(check_tc(n));
-    *loss = (float)h;
-  }
-  return LB_OK;
+  return loss ? finish(n, loss) : LB_OK;
 }
 
 lb_status lbu_conv3x3(const unsigned short* x, int x_stride, int batch, int h, int w, int c_in, int upsample,

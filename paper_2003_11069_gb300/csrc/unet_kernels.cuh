@@ -694,11 +694,17 @@ __global__ void refresh_weights_kernel(const LayerDev* __restrict__ L, const flo
   }
 }
 
-// Adam (bias-corrected): c1 = 1/(1 - b1^t), c2 = 1/(1 - b2^t)
+// Adam (bias-corrected): c1 = 1/(1 - b1^t), c2 = 1/(1 - b2^t). Nothing is updated, and the left-out
+// update counted in err[1], while the error word err[0] is set: the gradients came from a pass in
+// which some layer wrote no output.
 __global__ void adam_kernel(float* __restrict__ theta, const float* __restrict__ g, float* __restrict__ m,
                             float* __restrict__ v, long long n, float lr, float b1, float b2, float eps, float c1,
-                            float c2) {
+                            float c2, int* err) {
   lbnci::pdl_enter();
+  if (err[0] != 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) ++err[1];
+    return;
+  }
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const float gi = g[i];
     const float mi = b1 * m[i] + (1.f - b1) * gi;

@@ -3,7 +3,8 @@ tcgen05.mma with operands copied by TMA is the default, mma.sync (csrc/unet_kern
 of operands that it cannot take and of LBNCI_UNET_MMA=sync."""
 import pytest
 
-from paper_2003_11069_gb300 import unet
+from oracle import unet_oracle as U
+from paper_2003_11069_gb300 import inputs, lbnci, unet
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -40,3 +41,54 @@ def test_weight_gradient_scratch_of_eight_byte_alignment(B, H, W, Ci, Co, up, mo
     assert torch.equal(at8[0], sync[0]) and torch.equal(at8[1], sync[1])
     assert torch.equal(at16[0], tc[0]) and torch.equal(at16[1], tc[1])
     assert not torch.equal(tc[0], sync[0])  # the two kernels add in different orders
+
+
+def _net(B=2, seed=3):
+    cfg = unet.make_config(levels=2, base=32, H=16, W=32, max_batch=B)
+    net = unet.Net(cfg)
+    net.set_params(unet.flatten(inputs.unet_params(U.layer_shapes(2, 32, 5, 3), seed, bias_scale=0.05)))
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return net, torch.randn((B, 16, 32, 5), device="cuda", generator=g), torch.randn((B, 16, 32, 3), device="cuda", generator=g)
+
+
+def test_an_expired_wait_is_reported_to_its_own_network(monkeypatch):
+    """LBNCI_UNET_FAIL_TEST=1 sets the error word from the host as a kernel whose wait ran out would
+    (no wait is made to run out). The network whose launch it was reports it once, at its next call
+    that synchronises; another network, called before, does not; no update is applied meanwhile, and
+    the updates that follow are those of a network that never failed."""
+    monkeypatch.delenv("LBNCI_UNET_MMA", raising=False)
+    (a, X, T), (b, _, _), (c, _, _) = _net(), _net(), _net()
+    Y = torch.empty((2, 16, 32, 3), device="cuda")
+    with a, b, c:
+        start = a.get_params()
+        monkeypatch.setenv("LBNCI_UNET_FAIL_TEST", "1")
+        a.forward(X, Y)                      # device output: not synchronised, not checked
+        monkeypatch.delenv("LBNCI_UNET_FAIL_TEST")
+        b.forward(X.cpu().numpy())           # checked: not b's
+        assert b.loss_grad(X, T) > 0
+        for _ in range(2):
+            a.train_step(X, T)               # the word is set: left out
+        assert (a.get_params() == start).all()
+        with pytest.raises(lbnci.LBError, match="2 parameter updates left out"):
+            a.loss_grad(X, T)
+        for _ in range(3):                   # cleared; Adam goes on at its first step
+            assert a.train_step(X, T, want_loss=True) == c.train_step(X, T, want_loss=True)
+        assert (a.get_params() == c.get_params()).all()
+        assert not (a.get_params() == start).all()
+
+
+def test_an_expired_wait_of_a_single_call_is_told_apart(monkeypatch):
+    """The next synchronising network call reports it with its own results complete."""
+    monkeypatch.delenv("LBNCI_UNET_MMA", raising=False)
+    x = torch.zeros((1, 8, 16, 32), device="cuda", dtype=torch.bfloat16)
+    w, y = torch.zeros((32, 9, 32), device="cuda", dtype=torch.bfloat16), torch.empty_like(x)
+    net, X, T = _net()
+    with net:
+        loss = net.loss_grad(X, T)
+        monkeypatch.setenv("LBNCI_UNET_FAIL_TEST", "1")
+        unet.conv3x3(x, 32, 1, 8, 16, 32, 0, w, None, 0, y, 32, 32)
+        monkeypatch.delenv("LBNCI_UNET_FAIL_TEST")
+        torch.cuda.synchronize()
+        with pytest.raises(lbnci.LBError, match="single convolution"):
+            net.loss_grad(X, T)
+        assert net.loss_grad(X, T) == loss
