@@ -961,13 +961,21 @@ conv3x3_wgrad_tma_kernel(const __grid_constant__ WgradMaps maps, WgradTma a, int
           tc::mma_bf16_if(tmem + j * BN, tc::desc64(hiA, ua + rel[j]), tc::desc64(hiB, ub), IDESC, acc);
       }
     };
+    // Only the image's rows of a tile are multiplied: below the last one dy arrives as zeros, which
+    // times an infinite x of the row above would be NaN in taps that this x has no part in.
+    int tx = t0 % a.tiles_x, ty = (t0 / a.tiles_x) % a.tiles_y;
     for (int i = 0; i < nt; ++i) {
+      const int rows = min(a.TH, a.H - ty * a.TH);
+      if (++tx == a.tiles_x) {
+        tx = 0;
+        if (++ty == a.tiles_y) ty = 0;
+      }
       bad = __any_sync(~0u, !lbnci::mbar_wait(&t.bar_full[s], ph) || !lbnci::mbar_wait(&t.bar_patched[s], ph));
       if (bad) break;
       tc::fence_after_sync();
       const unsigned ux = base + (unsigned)((s * stage_bytes) >> 4);
       const unsigned ud = ux + (unsigned)(a.x_bytes >> 4) + (unsigned)dB;
-      for (int r = 0; r < a.TH; ++r) {
+      for (int r = 0; r < rows; ++r) {
         unsigned ua = ux + (unsigned)((r * a.pitch * ROWB) >> 4), ub = ud + (unsigned)((r * a.TW * DROW) >> 4);
         for (int c = 0; c < kx; ++c) {
           block(ua, ub, i | r | c);

@@ -92,3 +92,32 @@ def test_an_expired_wait_of_a_single_call_is_told_apart(monkeypatch):
         with pytest.raises(lbnci.LBError, match="single convolution"):
             net.loss_grad(X, T)
         assert net.loss_grad(X, T) == loss
+
+
+@pytest.mark.parametrize("B,H,W,Ci,Co,up", [(2, 17, 32, 32, 32, 0), (1, 10, 40, 64, 64, 0), (2, 18, 36, 64, 32, 1),
+                                            (1, 3, 16, 32, 64, 0)])
+@pytest.mark.parametrize("row", [0, -1])
+def test_weight_gradient_of_an_infinite_input(row, B, H, W, Ci, Co, up, monkeypatch):
+    """An infinite x reaches the sums that it is a term of and no other: the entries of dw that are
+    finite are those of the mma.sync kernel, and agree (P products exact in FP32, each sum within
+    P 2^-23 sum|terms| of the exact one), in tiles that are cut off by the image's last row too."""
+    g = torch.Generator(device="cuda").manual_seed(H + Ci)
+    hi, wi = (H // 2, W // 2) if up else (H, W)
+    x = torch.randn((B, hi, wi, Ci), device="cuda", generator=g).to(torch.bfloat16)
+    dy = torch.randn((B, H, W, Co), device="cuda", generator=g).to(torch.bfloat16)
+    finite = x.clone()
+    finite[0, row, 1, 2] = 0
+    x[0, row, 1, 2] = float("inf")
+    out = {}
+    for mma in ("tcgen05", "sync"):
+        monkeypatch.setenv("LBNCI_UNET_MMA", mma)
+        out[mma] = _wgrad(x, dy, up)[0].view(Co, 9, Ci).double()
+    monkeypatch.setenv("LBNCI_UNET_MMA", "sync")
+    scale = _wgrad(finite.abs(), dy.abs(), up)[0].view(Co, 9, Ci).double()
+    ok = torch.ones((Co, 9, Ci), dtype=torch.bool, device="cuda")
+    ok[:, :, 2] = False
+    if not up:  # no pixel lies beyond the image: one row of taps never meets its first or last row
+        ok[:, slice(0, 3) if row else slice(6, 9), 2] = True
+    assert torch.equal(torch.isfinite(out["sync"]), ok)
+    assert torch.equal(torch.isfinite(out["tcgen05"]), ok)
+    assert bool(((out["tcgen05"] - out["sync"])[ok].abs() <= 2.1 * B * H * W * 2.0 ** -23 * scale[ok]).all())
