@@ -136,14 +136,16 @@ size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 // The result area holds 16 doubles: the kRedSlots reductions, then, in slot
 // kErrSlot, the kernels' error word (an int), in slot kErrSlot + 1 the two tile
-// counters of the TMA step kernel (ints), and in slot kErrSlot + 2 the two dither-seed
-// words of the FP16-deviation stores (StepT::seedw).
+// counters of the TMA step kernel (ints), in slot kErrSlot + 2 the two dither-seed
+// words of the FP16-deviation stores (StepT::seedw), and in slot kErrSlot + 3 the ticket
+// counter of the fields pass (FieldOut::ticket).
 static_assert(lbnci::kErrSlot == 12, "result area");
 
 struct Layout {
   size_t fa, fb, psi, partials, result, carry, ring, ghost, ng, hit, rho1, sites;
   size_t total;  // with the scratch of the step's per-site passes
   size_t least;  // without it, where the step has kernels that need none
+  bool has_sites;  // sites is the scratch of the D2Q9 or FP64 passes (HostParams::sites)
 };
 
 const Launchers* launchers_for(const lb_config* c) {
@@ -192,7 +194,8 @@ lb_status validate(const lb_config* c, HostParams* p, Layout* lay, long long* nb
   p->smax = smax;
   p->forcing = c->forcing;
   p->num_sms = 1;
-  // D3Q27 collision kernel: LBNCI_D3_KERNEL=march (z-marching, default) or tiled.
+  // Collision kernel of the two-pass D3Q27 step (lattices and workspaces that no other step
+  // takes, or LBNCI_D3_KERNEL=march or tiled): marching along z, or tiled.
   p->d3_kernel = 0;
   if (const char* e = std::getenv("LBNCI_D3_KERNEL")) p->d3_kernel = std::strcmp(e, "tiled") == 0 ? 1 : 0;
   // Tile of the fused D2Q9 kernel: LBNCI_FUSED_SPT=2 (32x16, the default) or 4 (32x32).
@@ -274,6 +277,7 @@ lb_status validate(const lb_config* c, HostParams* p, Layout* lay, long long* nb
     lay->ng = off; off = align256(off + (size_t)N * 16);
   }
   p->sites = nullptr;
+  lay->has_sites = sites;
   if (sites) {
     lay->sites = off; off = align256(off + L->step_scratch((size_t)N));
   }
@@ -465,7 +469,7 @@ lb_status lb_create(const lb_config* cfg, lb_sim** out) {
     s->rho1 = base + lay.rho1;
   }
   if (!s->p.stream3d) s->p.totals = 0;
-  if (passes && lay.total > lay.sites && lay.sites >= lay.least) s->p.sites = base + lay.sites;
+  if (passes && lay.has_sites) s->p.sites = base + lay.sites;
   s->totals_state = false;
   s->carry_ok = false;
   e = cudaMallocHost((void**)&s->host_result, 16 * sizeof(double));
