@@ -115,11 +115,13 @@ typedef struct {
 } lb_obs;
 
 /* Device bytes lb_create needs when it is given a workspace (cfg->workspace): two
- * population states of the two sets f^k_i of Eq. (CGLBE) plus scratch. A workspace larger
- * by 48 N + 1024 bytes (FP64 with Guo forcing) or 16 N + 1024 bytes (FP32 and FP16-dev D3Q27
- * lattices with nx % 32 != 0 or ny % 8 != 0) also holds the per-site arrays of those steps'
- * faster kernels, which a sim that allocates its own memory takes when it can; without
- * them the step runs kernels that recompute over halos, to the same bits. */
+ * population states of the two sets f^k_i of Eq. (CGLBE) plus scratch. A larger workspace
+ * also holds the per-site arrays (N sites) of the faster kernels that some steps have:
+ *   FP64 with Guo forcing, D2Q9 and D3Q27                          48 N + 1024 bytes more
+ *   FP32 and FP16-dev D2Q9 with nx % 4 != 0                        24 N + 1024
+ *   FP32 and FP16-dev D3Q27 with nx % 32 != 0 or ny % 8 != 0       16 N + 1024
+ * A sim that allocates its own memory takes them when it can; without them the step runs
+ * kernels that recompute over halos, to the same bits. */
 lb_status lb_workspace_size(const lb_config* cfg, size_t* bytes);
 
 /* Validate cfg, take the current CUDA device, allocate (or carve from the
