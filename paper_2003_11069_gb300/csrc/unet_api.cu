@@ -356,15 +356,22 @@ bool plan_tile(int B, int H, int W, int cin, int cout, int up, bool mask, ConvPl
   return best < 1e30;
 }
 
-// Strips of conv3x3_rows_kernel over B images of H x W positions: wide images (at most a third
-// of the 128-column strips beyond the image) whose weights for BN output channels and three
-// input rows fit in shared memory. Two CTAs per multiprocessor where they fit, and the number
+// Strips of conv3x3_rows_kernel over B images of H x W positions: wide images (at most a quarter
+// of the 128-column strips' columns beyond the image, so W >= 96) whose weights for BN = 32 or 64
+// output channels, with three input rows, fit in shared memory. More output channels are blocks of
+// BN that each copy the input again. Every such layer takes the strips: this estimate and
+// plan_tile's carry overheads fitted to their own kernel and are not comparable. Strips against
+// tiles, us alone on the GPU, 32 images: 64 x 256, 32 -> 32 channels 20.9 / 29.3, 64 -> 32 29.2 /
+// 60.6, 32 -> 64 37.2 / 59.2; 32 x 128, 128 -> 64 24.9 / 37.2; 32 x 96, 32 -> 32 10.9 / 16.7;
+// 64 x 256 upsampled, 64 -> 32 28.4 / 41.5. One image: 64 x 256, 64 -> 32 8.7 / 10.5. Equal in
+// several deep layers; slower where two blocks of 64 channels fill the chip: 32 x 128, 64 -> 128,
+// 32 images 39.1 / 27.0 (8 images 12.8 / 13.0, one image 8.7 / 10.6). Two CTAs per multiprocessor where they fit, and the number
 // of output rows per CTA with the smallest estimated time: waves of CTAs, each the longer of
 // its MMAs (32 + N/4 cycles, N/2 above N = 128), its copies and its drain, and about 4,000
 // cycles to start and end.
 bool plan_rows(int B, int H, int W, int cin, int cout, int up, bool mask, ConvPlan* p) {
   const int tiles_x = (W + 127) / 128;
-  if (W < 64 || 4 * W < 3 * tiles_x * 128) return false;
+  if (4 * W < 3 * tiles_x * 128) return false;
   const int rowb = cin % 64 == 0 ? 128 : 64, nchunk = cin / (rowb / 2), npx = up ? 2 : 1, Ho = H << up;
   const int cstride = (130 * rowb + 1023) / 1024 * 1024;
   double best = 1e30;
@@ -380,7 +387,6 @@ bool plan_rows(int B, int H, int W, int cin, int cout, int up, bool mask, ConvPl
       if (nrow < (up ? 3 : 4)) continue;
       const double n3 = 3 * BN, mma = 3.0 * nchunk * (rowb / 32) * npx * (n3 <= 128 ? 32 + n3 / 4 : n3 / 2);
       for (int TH = 2; TH <= Ho; TH += 2) {
-        if (TH > 2 && TH - 2 >= Ho) break;
         const int th = std::min(TH, Ho), tiles_h = (Ho + th - 1) / th;
         const double ctas = (double)B * tiles_x * tiles_h * (cout / BN);
         const double waves = std::ceil(ctas / (152.0 * occ));
@@ -495,8 +501,9 @@ cudaError_t launch_conv_plan(const ConvPlan& p, int* err, cudaStream_t s, bool c
                      : (p.BN == 64 ? launch_conv_tma<64, 64>(p, err, s, chained) : launch_conv_tma<32, 64>(p, err, s, chained));
 }
 
-// LBNCI_UNET_MMA=sync selects the mma.sync convolution for every layer. It stays for the
-// layers whose input tile does not fit in shared memory (more than about 512 channels).
+// LBNCI_UNET_MMA=sync selects the mma.sync convolution and weight gradient for every layer. They
+// stay for the layers whose input tile does not fit in shared memory (more than about 512
+// channels) and for operands of single calls that are aligned to less than 16 bytes.
 bool conv_on_mma_sync() {
   const char* e = std::getenv("LBNCI_UNET_MMA");
   return e && std::strcmp(e, "sync") == 0;

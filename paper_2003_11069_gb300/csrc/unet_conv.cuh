@@ -502,7 +502,7 @@ conv3x3_tma_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
 }
 
 // ------------------------------------------------------------------ wide images, few channels
-// The same convolution for 32 or 64 output channels on wide images, row by row. An MMA's
+// The same convolution for blocks of 32 or 64 output channels on wide images, row by row. An MMA's
 // operand fetch (128 rows of A) costs as much for N = 32 as the products of N = 96, so here
 // one MMA multiplies an input row, shifted by dx, with the weights of the three dy at once
 // (N = 3 BN, the weights stacked dy = +1, 0, -1) into the accumulators of the three output
