@@ -33,10 +33,14 @@ def test_waits_of_whole_warps_are_votes():
         count += 1
         if any(a < m.start() < b for a, b in single):
             continue
-        # the statement that holds the wait, and the one after it
+        # the statement that holds the wait, and the one after it: a vote of the warp
         start = max(code.rfind(c, 0, m.start()) for c in ";{}")
         end = code.index(";", code.index(";", m.start()) + 1)
-        assert re.search(r"__(any|all)_sync\(~0u", code[start:end]), code[start:end]
+        if re.search(r"__(any|all)_sync\(~0u", code[start:end]):
+            continue
+        # or the group's reduction, with nothing on the way that lanes could leave by or meet at
+        until = code[m.start():code.index("bar_all(", m.start())]
+        assert not re.search(r"\b(break|continue|return|while)\b|__syncwarp|bar\.sync|&& ok", until), until
     assert count >= 10
 
 
@@ -47,7 +51,7 @@ def test_drain_groups_leave_their_loop_together():
     at = code.index("for (int q = 0; q < nq && ok; ++q) {")
     a, b = _block(code, at)
     body = code[a:b]
-    waits = [m.start() for m in re.finditer(r"ok = warp_wait\(done", body)]
+    waits = [m.start() for m in re.finditer(r"ok = (?:warp|lbnci::mbar)_wait\(done", body)]
     assert len(waits) == 2
     for w in waits:
         vote = body.index("ok = bar_all(1 + g, 128, ok)", w)
