@@ -66,8 +66,8 @@ cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cuda
 // read what the predecessor does not write (a network's weights), and blocks that hold
 // tensor memory at the wait never keep it from a block that has yet to start. Measured on
 // the U-Net's chains of 5 to 60 us kernels (setup, barrier initialisation, tensor-memory
-// allocation and the first weights overlap the kernel before): batch-8 forward of 23 launches
-// 289 -> 239 us, batch-32 training step of 86 launches 1771 -> 1587 us.
+// allocation and the first weights overlap the kernel before): batch-8 forward of 22 launches
+// 289 -> 239 us, batch-32 loss and gradients of 82 launches 1771 -> 1587 us.
 __device__ __forceinline__ void pdl_enter() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
